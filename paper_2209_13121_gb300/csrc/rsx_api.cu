@@ -129,6 +129,7 @@ struct rsx_context {
   void* dir = nullptr;      // FP64 Algorithm 1: the morphology's director, [c][3][N] double
   std::vector<double> energies, constants;
   void* p = nullptr;    // kx x 3 N complex workspace (one p per angle of a batch)
+  long long p_cap = 0;  // its size in complex elements (at least kx x 3 N; see p_elems)
   int kx = 1;           // angle batch of the Algorithm 1 x pass
   void* img = nullptr;  // one detector image
   void* acc = nullptr;  // running sum of rotated images
@@ -165,8 +166,11 @@ struct rsx_context {
   // bins of the fused y-FFT + pruned z pass (FP32, Algorithms 1 and 2):
   // [kYzSlots][nf][ny][nx] float4
   void* part = nullptr;
-  // linearity path: the images of a batch of angles ([kMaxAngleBatch][ny][nx])
+  // the images of a batch of n_img angles ([n_img][ny][nx]): the linearity
+  // path's, or the planes path's (there in the memory of part where it exists)
   void* imgs = nullptr;
+  int n_img = 0;
+  bool imgs_owned = false;
   // page-locked staging of host output (grown on demand)
   void* host_stage = nullptr;
   size_t host_stage_bytes = 0;
@@ -188,8 +192,7 @@ namespace {
 
 void free_all(rsx_context* c) {
   void* ptrs[] = {c->M_owned, c->p,    c->img, c->acc,  c->geo,  c->twx, c->twy,
-                  c->twz,     c->tw4,  c->flag, c->err, c->part, c->imgs, c->dir, c->tw2k,
-                  c->b0idx};
+                  c->twz,     c->tw4,  c->flag, c->err, c->part, c->dir, c->tw2k, c->b0idx};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   for (auto& r : c->recs) {
@@ -204,6 +207,7 @@ void free_all(rsx_context* c) {
     if (c->ev_copied[b]) cudaEventDestroy(c->ev_copied[b]);
     if (c->ev_used[b]) cudaEventDestroy(c->ev_used[b]);
   }
+  if (c->imgs_owned) cudaFree(c->imgs);
   if (c->nt) cudaFree(c->nt);
   if (c->ft) cudaFree(c->ft);
   if (c->bins5) cudaFree(c->bins5);
@@ -745,6 +749,56 @@ static bool zfirst_plan_of(const rsx_config& g, int kx, double k, ZPlan* zp) {
   return zp->kz >= 1;
 }
 
+// The general planes path serves Algorithms 1 and 2 with nz <= kMaxPlanesNz.
+static bool planes_cfg(const rsx_config* cfg) {
+  return cfg->algorithm != 3 && cfg->nz <= rsx::kMaxPlanesNz;
+}
+
+// Complex elements of the p workspace: one p (3 N) per angle of the batch; on
+// the planes path at least 32 angles' p or 96 MB (within the 126 MB L2, so
+// that the planes of a batch of a small grid pass from kernel to kernel
+// there), whichever is less.
+static long long p_elems(const rsx_config* cfg) {
+  const long long one = 3LL * cfg->nx * cfg->ny * cfg->nz, base = one * angle_batch_of(cfg);
+  if (!planes_cfg(cfg)) return base;
+  const long long pool = (96LL << 20) / (long long)complex_size(cfg->precision);
+  const long long want = 32 * one < pool ? 32 * one : pool;
+  return want > base ? want : base;
+}
+
+// Images held at once: a launch's worth for the linearity path; on the
+// planes path as many as the fused y+z pass's bins have room for, or 64 MB.
+static int image_batch(const rsx_config* cfg) {
+  if (cfg->algorithm == 3) return rsx::kMaxAngleBatch;
+  if (!planes_cfg(cfg)) return 0;
+  const long long img = (long long)cfg->nx * cfg->ny * (long long)real_size(cfg->precision);
+  const long long n = uses_yz(cfg) ? (long long)part_bytes(cfg) / img : (64LL << 20) / img;
+  return n < 1 ? 1 : n > rsx::kMaxAngleBatch ? rsx::kMaxAngleBatch : (int)n;
+}
+
+// The planes path's plan: the run of bins the pixels read (all of them where
+// the run would wrap onto itself) and the angles whose planes fit in p.
+// FP64: the pass evaluates the kept bins one by one, 6 ns fused multiply-adds
+// per voxel and angle, and the lateral transforms of the kept planes take
+// ~230 ns / nz; it pays while that is below what transforming every slice and
+// evaluating the morphology per angle takes (~330; FP64 arithmetic is the
+// bound).  FP32 with rows of 512, 1024 or 2048 points keeps the x-first
+// passes (~4x the general lateral transforms' rate).
+static bool planes_plan(const rsx_context* c, int ie, ZPlan* zp) {
+  const rsx_config& g = c->cfg;
+  if (!planes_cfg(&g) || !c->imgs || ie < 0 || ie >= (int)c->energies.size()) return false;
+  if (x_multi_cap(&g) || (g.precision == 32 && g.algorithm == 2 && (g.nx == 512 || g.nx == 1024)))
+    return false;
+  const int blo = lowest_bin(g, wavenumber(c->energies[ie]));
+  zp->ns = 2 - blo < g.nz ? 2 - blo : g.nz;
+  zp->kb = zp->ns == g.nz ? 0 : ((blo % g.nz) + g.nz) % g.nz;
+  if (!rsx::pol_planes_fits(g.precision, g.nz, zp->ns)) return false;
+  if (g.precision == 64 && 6.0 * zp->ns + 230.0 * zp->ns / g.nz > 330.0) return false;
+  const long long kz = c->p_cap / (3LL * zp->ns * c->npix);
+  zp->kz = kz < rsx::kMaxAngleBatch ? (int)kz : rsx::kMaxAngleBatch;
+  return zp->kz >= 1;
+}
+
 static bool zfirst_plan(const rsx_context* c, int ie, ZPlan* zp) {
   const rsx_config& g = c->cfg;
   if (!zfirst_ok(&g) || c->n_sm <= 0 || !c->part || !c->b0idx || ie < 0 ||
@@ -765,14 +819,15 @@ size_t rsx_workspace_bytes(const rsx_config* cfg) {
                  ? (size_t)cfg->n_components * N * 4 * R  // morphology copy (Table 1: 4c N)
                  : 5 * (size_t)N * Cs + 2 * (size_t)stage_vox * 4 * R;  // N_t + staging (Table 2)
   if (cfg->algorithm == 3) b += 5 * (size_t)N * Cs + 10 * (size_t)npix * Cs;  // FFT'd N_t, bins
-  b += 3 * (size_t)N * Cs * angle_batch_of(cfg);     // p_x, p_y, p_z (Table 1: 6 N) per angle
+  b += (size_t)p_elems(cfg) * Cs;                    // p_x, p_y, p_z (Table 1: 6 N) per angle
   if (cfg->precision == 64 && cfg->algorithm == 1)
     b += 3 * (size_t)cfg->n_components * N * R;      // the cached director
   b += 2 * (size_t)npix * R;                         // Ewald, Ewald_Avg (Table 1: 2 nx ny)
   b += (size_t)npix * geo_size(cfg->precision);
   b += (size_t)(cfg->nx + cfg->ny + cfg->nz) * Cs + sizeof(int);
   if (uses_yz(cfg)) b += part_bytes(cfg) + 2 * (size_t)npix;  // fused y + z pass: bins, bin indices
-  if (cfg->algorithm == 3) b += (size_t)rsx::kMaxAngleBatch * npix * R;  // a batch of images
+  if (!uses_yz(cfg) || cfg->algorithm == 3)
+    b += (size_t)image_batch(cfg) * npix * R;        // a batch of images
   return b;
 }
 
@@ -832,12 +887,13 @@ int rsx_create(const rsx_config* cfg, rsx_context** out) {
     return cuda_fail(e, "cudaGetDevice");
   }
   const size_t R = real_size(cfg->precision), Cs = complex_size(cfg->precision);
+  c->p_cap = p_elems(cfg);
   struct {
     void** dst;
     size_t bytes;
     const char* what;
   } allocs[] = {
-      {&c->p, 3 * (size_t)c->N * Cs * c->kx, "p workspace"},
+      {&c->p, (size_t)p_elems(cfg) * Cs, "p workspace"},
       {&c->img, (size_t)c->npix * R, "Ewald image"},
       {&c->acc, (size_t)c->npix * R, "Ewald average"},
       {&c->geo, (size_t)c->npix * geo_size(cfg->precision), "Ewald geometry"},
@@ -920,19 +976,25 @@ int rsx_create(const rsx_config* cfg, rsx_context** out) {
       c->has_tmap_ftz = make_tmap(c, c->ft, 5LL * cfg->nz, &c->tmap_ftz, box,
                                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
   }
-  if (cfg->algorithm == 3 &&
-      (e = cudaMalloc(&c->imgs, (size_t)rsx::kMaxAngleBatch * c->npix * R)) != cudaSuccess) {
-    rc = cuda_fail(e, "linearity path images");
-    free_all(c);
-    delete c;
-    return rc;
-  }
   if (uses_yz(cfg) && ((e = cudaMalloc(&c->part, part_bytes(cfg))) != cudaSuccess ||
                        (e = cudaMalloc((void**)&c->b0idx, (size_t)c->npix * 2)) != cudaSuccess)) {
     rc = cuda_fail(e, "y + z pass bins");
     free_all(c);
     delete c;
     return rc;
+  }
+  c->n_img = image_batch(cfg);
+  if (c->n_img > 0 && cfg->algorithm != 3 && c->part) {
+    c->imgs = c->part;  // the planes path does not use the bins
+  } else if (c->n_img > 0) {
+    if ((e = cudaMalloc(&c->imgs, (size_t)c->n_img * c->npix * R)) != cudaSuccess) {
+      c->imgs = nullptr;
+      rc = cuda_fail(e, "images of a batch of angles");
+      free_all(c);
+      delete c;
+      return rc;
+    }
+    c->imgs_owned = true;
   }
   if ((rc = upload_twiddles(c, cfg->nx, &c->twx)) || (rc = upload_twiddles(c, cfg->ny, &c->twy)) ||
       (rc = upload_twiddles(c, cfg->nz, &c->twz))) {
@@ -1297,6 +1359,93 @@ int run_energy_zfirst(rsx_context* c, int ie, double start, double inc, int nang
   return RSX_OK;
 }
 
+// x-FFT of nrows contiguous rows of the planes in p, in place.
+template <typename R>
+cudaError_t planes_x_fft(rsx_context* c, long long nrows, cudaStream_t s) {
+  const rsx_config& g = c->cfg;
+  if (g.nx == 1) return cudaSuccess;
+  if (sizeof(R) == 4 && (g.nx == 512 || (g.nx == 1024 && c->tw4) || (g.nx == 2048 && c->tw2k)))
+    return rsx::launch_xfft_rows(c->p, g.nx, nrows,
+                                 g.nx == 1024 ? c->tw4 : g.nx == 2048 ? c->tw2k : c->twx, s);
+  if (g.nx == 1024 && c->tw4) return rsx::launch_row_fft4s<R>(c->p, nrows, c->tw4, s);
+  return rsx::launch_row_fft<R>(c->p, g.nx, nrows, c->twx, s);
+}
+
+// y-FFT of nplanes contiguous [ny][nx] planes in p, in place.
+template <typename R>
+cudaError_t planes_y_fft(rsx_context* c, long long nplanes, cudaStream_t s) {
+  const rsx_config& g = c->cfg;
+  const rsx::ColBatches bt = {nplanes, 1, c->npix, 0, 0};
+  if (g.ny == 1024 && g.nx % 8 == 0 && c->tw4)
+    return rsx::launch_col_fft4s<R>(c->p, g.nx, g.nx, bt, c->tw4, s);
+  return rsx::launch_col_fft<R>(c->p, g.ny, g.nx, g.nx, bt, c->twy, s);
+}
+
+// All angles of one energy on the general planes path (plan from
+// planes_plan): per batch of angles one launch each for p and its pruned z
+// transform, the x-FFT and the y-FFT of every kept plane, then the images
+// and the rotation into the average, n_img angles at a time.
+template <typename R>
+int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang, int rotation,
+                      const ZPlan& zp, cudaStream_t s) {
+  const rsx_config& g = c->cfg;
+  int rc = ensure_geo<R>(c, ie, s);
+  if (rc) return rc;
+  if (g.algorithm == 2 && (rc = ensure_nt<R>(c, ie, s))) return rc;
+  const PolParams<R> pp = make_params<R>(c, ie, 0.0, 0);
+  const double ref = -(double)(g.n_components - 1) / (4.0 * kPi) * (double)c->N;
+  const int npass = (nang + zp.kz - 1) / zp.kz, per = (nang + npass - 1) / npass;
+  for (int a0 = 0; a0 < nang; a0 += per) {
+    const int nk = nang - a0 < per ? nang - a0 : per;
+    double alpha[rsx::kMaxAngleBatch];
+    rsx::AngleBatch<R> ab;
+    memset(&ab, 0, sizeof(ab));
+    for (int k = 0; k < nk; ++k) {
+      alpha[k] = rotation ? (start + inc * (a0 + k)) * (kPi / 180.0) : 0.0;
+      rsx::add_angle(ab, alpha[k], g.nx, g.ny);
+    }
+    {
+      PhaseTimer pt(c, RSX_PHASE_POL_FFTX, s);
+      RSX_CK(rsx::launch_pol_planes<R>(c->M, g.algorithm == 2 ? c->nt : nullptr, c->dir, c->npix,
+                                       g.nz, pp, ab, c->p, zp.kb, zp.ns, c->twz, s),
+             "polarisation + z-transform kernel");
+    }
+    {
+      PhaseTimer pt(c, RSX_PHASE_FFTX, s);
+      RSX_CK(planes_x_fft<R>(c, (long long)nk * 3 * zp.ns * g.ny, s), "x-FFT kernel");
+    }
+    if (g.ny > 1) {
+      PhaseTimer pt(c, RSX_PHASE_FFTY, s);
+      RSX_CK(planes_y_fft<R>(c, (long long)nk * 3 * zp.ns, s), "y-FFT kernel");
+    }
+    for (int i0 = 0; i0 < nk; i0 += c->n_img) {
+      const int ni = nk - i0 < c->n_img ? nk - i0 : c->n_img;
+      rsx::ImageDc<R> dc;
+      memset(&dc, 0, sizeof(dc));
+      rsx::AngleBatch<R> rb;
+      memset(&rb, 0, sizeof(rb));
+      dc.n = ni;
+      for (int k = 0; k < ni; ++k) {
+        const bool lit = g.frame == RSX_FRAME_LITERAL;
+        dc.x[k] = (R)(lit ? ref : ref * cos(alpha[i0 + k]));
+        dc.y[k] = (R)(lit ? 0.0 : ref * sin(alpha[i0 + k]));
+        rsx::add_angle(rb, alpha[i0 + k], g.nx, g.ny);
+      }
+      {
+        PhaseTimer pt(c, RSX_PHASE_EWALD, s);
+        RSX_CK(rsx::launch_plane_images<R>((const char*)c->p + (size_t)i0 * 3 * zp.ns * c->npix * 2 * sizeof(R),
+                                           g.nx, g.ny, g.nz, zp.kb, zp.ns, (const Geo<R>*)c->geo,
+                                           dc, c->imgs, s),
+               "Ewald kernel");
+      }
+      PhaseTimer pt(c, RSX_PHASE_ROTATE, s);
+      RSX_CK(rsx::launch_rotate_acc_many<R>(c->imgs, c->acc, g.nx, g.ny, rb, rotation != 0, s),
+             "rotation kernel");
+    }
+  }
+  return RSX_OK;
+}
+
 template <typename R>
 int run_energy_angles(rsx_context* c, int ie, double start, double inc, int nang, int rotation,
                       cudaStream_t s) {
@@ -1307,6 +1456,9 @@ int run_energy_angles(rsx_context* c, int ie, double start, double inc, int nang
         ((uintptr_t)c->M & 15) == 0)
       return run_energy_angles_batched(c, ie, start, inc, nang, rotation, s);
   }
+  ZPlan pl;
+  if (planes_plan(c, ie, &pl))
+    return run_energy_planes<R>(c, ie, start, inc, nang, rotation, pl, s);
   for (int a = 0; a < nang; ++a) {
     const double alpha = rotation ? (start + inc * a) * (kPi / 180.0) : 0.0;
     int rc = scatter_angle<R>(c, ie, alpha, c->img, s);
@@ -1373,7 +1525,7 @@ int run_impl(rsx_context* c, double start, double inc, int nang, int rotation,
   for (size_t o = 0; o < sel.size(); ++o) {
     const int ie = sel[o];
     RSX_CK(cudaMemsetAsync(c->acc, 0, img_bytes, s), "clear average");
-    const int rc = c->cfg.algorithm == 3 && c->imgs
+    const int rc = c->cfg.algorithm == 3
                        ? run_energy_linear<R>(c, ie, start, inc, nang, rotation, s)
                        : run_energy_angles<R>(c, ie, start, inc, nang, rotation, s);
     if (rc) return rc;

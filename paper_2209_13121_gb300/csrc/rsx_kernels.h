@@ -306,6 +306,29 @@ cudaError_t launch_rotate_acc_many(const void* imgs, void* acc, int nx, int ny,
 template <typename R>
 cudaError_t launch_rotate_acc(const void* img, void* acc, int nx, int ny, double alpha,
                               bool rotate, cudaStream_t s);
+// The general planes path (rsx_planes.cu), any grid with nz <= kMaxPlanesNz.
+// launch_pol_planes: p of the ang.n angles (from the morphology M, with the
+// cached director dir if given, or from Algorithm 2's nt), z-transformed, only
+// the ns bins kb .. kb + ns - 1 (mod nz) kept: plane s of field f of angle k
+// goes to out + ((k * 3 + f) * ns + s) * npix.  pol_planes_fits: whether the
+// pass has a launch shape for this stack (its twiddles in shared memory).
+// launch_plane_images: the angles' images ([n][ny][nx], fftshift order) from
+// the x- and y-transformed planes; dc: the x and y parts, per angle, of the
+// constant left out of p (returned at q = 0).
+constexpr int kMaxPlanesNz = 255;
+template <typename R> struct ImageDc {
+  int n;
+  R x[kMaxAngleBatch], y[kMaxAngleBatch];
+};
+bool pol_planes_fits(int precision, int nz, int ns);
+template <typename R>
+cudaError_t launch_pol_planes(const void* M, const void* nt, const void* dir, long long npix,
+                              int nz, const PolParams<R>& pp, const AngleBatch<R>& ang, void* out,
+                              int kb, int ns, const void* twz, cudaStream_t s);
+template <typename R>
+cudaError_t launch_plane_images(const void* planes, int nx, int ny, int nz, int kb, int ns,
+                                const Geo<R>* geo, const ImageDc<R>& dc, void* imgs,
+                                cudaStream_t s);
 template <typename R>
 cudaError_t launch_scale(const void* acc, void* out, long long n, double scale, cudaStream_t s);
 template <typename R>

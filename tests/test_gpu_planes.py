@@ -1,0 +1,85 @@
+"""The general planes path of rsx_run (Algorithms 1 and 2, nz <= 255, both
+precisions): per pixel column p and its z transform at only the q_z bins the
+detector reads, the lateral transforms of those planes, images and rotation
+for a batch of angles at a time.  Checked at the edges of its rules: one
+slice, odd and even stacks, the tallest stack it takes and the first beyond
+it, pixel tiles with a remainder, runs of bins that wrap onto themselves,
+energies and voxels that read few or nearly all bins, more angles than a
+batch holds."""
+import numpy as np
+import pytest
+
+from oracle import cyrsoxs_oracle as O
+from paper_2209_13121_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+# the parity tests' tolerances: relative L2 away from q = 0, per pixel above a floor
+TOL = {64: dict(norm=1e-10, pix=1e-8, floor=1e-8), 32: dict(norm=1e-4, pix=2e-3, floor=1e-4)}
+
+
+@pytest.fixture(scope="module")
+def rsx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2209_13121_gb300 import rsx as R
+    return R
+
+
+def _close(got, ref, prec, r=2.5):
+    got, ref = np.asarray(got, np.float64), np.asarray(ref, np.float64)
+    ny, nx = ref.shape[-2:]
+    iy, ix = np.meshgrid(np.arange(ny) - ny // 2, np.arange(nx) - nx // 2, indexing="ij")
+    far = np.broadcast_to(np.hypot(ix, iy) > r, ref.shape)
+    t = TOL[prec]
+    assert np.all(np.isfinite(got))
+    if far.any() and np.abs(ref[far]).max() > 0:
+        assert np.linalg.norm((got - ref)[far]) <= t["norm"] * np.linalg.norm(ref[far])
+    big = np.abs(ref) > t["floor"] * np.abs(ref).max()
+    assert (np.abs(got - ref)[big] / np.abs(ref)[big]).max() <= t["pix"]
+
+
+# (nz, ny, nx), c, voxel nm, energy eV
+EDGES = [((1, 24, 40), 2, 5.0, 285.0), ((2, 9, 10), 3, 5.0, 285.0), ((3, 16, 64), 2, 5.0, 270.0),
+         ((16, 20, 52), 3, 5.0, 285.0), ((45, 12, 11), 2, 5.0, 285.0), ((64, 8, 24), 2, 2.0, 300.0),
+         ((127, 6, 10), 2, 5.0, 285.0), ((128, 8, 8), 2, 5.0, 285.0), ((254, 4, 6), 1, 5.0, 285.0),
+         ((255, 3, 7), 2, 5.0, 285.0), ((256, 4, 4), 1, 5.0, 285.0), ((16, 16, 16), 2, 5.0, 60.0),
+         ((32, 10, 12), 2, 1.0, 17000.0), ((30, 33, 17), 4, 10.0, 310.0)]
+
+
+@pytest.mark.parametrize("prec", [32, 64])
+@pytest.mark.parametrize("shape,c,voxel,E", EDGES,
+                         ids=["x".join(map(str, e[0])) + f"@{e[3]:g}" for e in EDGES])
+def test_edges_match_oracle_and_the_general_path(rsx, shape, c, voxel, E, prec):
+    nz, ny, nx = shape
+    M = synth.morphology_random(shape, c, seed=11, dtype=np.float32 if prec == 32 else np.float64)
+    K = synth.optical_constants([E], c, seed=12)
+    dev = torch.from_numpy(M).cuda()
+    for alg, frame in ((1, 0), (2, 1)):
+        ref = O.run_alg1(M, K, [E], voxel, angles_deg=(0.0, 40.0, 160.0),
+                         uT_mode="lab" if frame else "literal")
+        with rsx.Context(nx, ny, nz, c, voxel, precision=prec, algorithm=alg, frame=frame) as ctx:
+            ctx.set_morphology(dev)
+            ctx.set_optical_constants([E], K)
+            _close(ctx.run((0.0, 40.0, 160.0)), ref, prec)
+            # one angle without rotation is the single image, which takes the
+            # passes of the general path
+            img = torch.empty((ny, nx), device="cuda", dtype=dev.dtype)
+            ctx.scatter_angle(0, 0.0, img)
+            _close(ctx.run(rotation=False)[0], img.cpu().numpy(), prec, r=1.5)
+
+
+def test_more_angles_than_one_batch_holds(rsx):
+    """181 angles in three or more batches of at most 64; two energies."""
+    shape, c, E = (6, 12, 20), 2, [275.0, 300.0]
+    M = synth.morphology_random(shape, c, seed=13, dtype=np.float32)
+    K = synth.optical_constants(E, c, seed=14)
+    ref = O.run_alg1(M, K, E, 5.0, angles_deg=(0.0, 1.0, 180.0))
+    with rsx.Context(20, 12, 6, c, 5.0) as ctx:
+        ctx.set_morphology(M)
+        ctx.set_optical_constants(E, K)
+        _close(ctx.run((0.0, 1.0, 180.0)), ref, 32)
