@@ -455,18 +455,15 @@ int ensure_nt(rsx_context* c, int ie, cudaStream_t s) {
 // The fused y-FFT + q_z bins pass over nf fields (3: p; 5: the linearity
 // path's N_t entries) through the tensor map `map`: the 1024-row kernel or
 // the 512-row one.
-// sel: the z-first path's ns planes per field (sel.nzfull > 0) instead of
-// the nz slices.
-cudaError_t fused_yz(rsx_context* c, const CUtensorMap* map, int nf, long long* L, cudaStream_t s,
-                     rsx::YzSel sel = rsx::YzSel(), int ns = 0) {
+cudaError_t fused_yz(rsx_context* c, const CUtensorMap* map, int nf, long long* L,
+                     cudaStream_t s) {
   const rsx_config& g = c->cfg;
-  const int nzv = sel.nzfull > 0 ? ns : g.nz;
   if (g.ny == 512)
-    return rsx::launch_yz512_tma(map, g.nx, nzv, nf, (const Geo<float>*)c->geo, c->twz, c->twy,
-                                 c->b0idx, c->part, c->err, c->n_sm, c->wait_polls, L, s, sel);
-  return rsx::launch_yz_tma(map, g.nx, g.ny, nzv, nf, (const Geo<float>*)c->geo, c->twz, c->tw4,
+    return rsx::launch_yz512_tma(map, g.nx, g.nz, nf, (const Geo<float>*)c->geo, c->twz, c->twy,
+                                 c->b0idx, c->part, c->err, c->n_sm, c->wait_polls, L, s);
+  return rsx::launch_yz_tma(map, g.nx, g.ny, g.nz, nf, (const Geo<float>*)c->geo, c->twz, c->tw4,
                             g.ny == 2048 ? c->twy : nullptr, c->b0idx, c->part, c->err, c->n_sm,
-                            c->wait_polls, L, s, sel);
+                            c->wait_polls, L, s);
 }
 
 // Linearity fast path, once per energy: FFT (x and y) of N_t's five
@@ -657,6 +654,11 @@ static bool uses_yz(const rsx_config* cfg) {
   return cfg->precision == 32 && rsx::yz_fusable(cfg->nx, cfg->ny, cfg->nz);
 }
 // kYzSlots slots of (3 fields of p, or the linearity path's 5 N_t entries) x 2 bins
+// The planes path's tuned y pass (FP32).
+static bool y_tuned(const rsx_config* cfg) {
+  return cfg->precision == 32 && cfg->algorithm != 3 && cfg->nz <= rsx::kMaxPlanesNz &&
+         rsx::y_planes_ok(cfg->nx, cfg->ny);
+}
 static size_t part_bytes(const rsx_config* cfg) {
   return rsx::kYzSlots * (size_t)(cfg->algorithm == 3 ? 5 : 3) * cfg->nx * cfg->ny * 16;
 }
@@ -704,6 +706,7 @@ static int angle_batch_of(const rsx_config* cfg) {
 // and a t within 1e-9 above an integer also takes the bin below.
 struct ZPlan {
   int kb = 0, ns = 0, kz = 0;
+  bool zfft = false;  // p and its z transform by launch_pol_zfft_multi
 };
 
 static int lowest_bin(const rsx_config& g, double k) {
@@ -776,29 +779,6 @@ static int image_batch(const rsx_config* cfg) {
   return n < 1 ? 1 : n > rsx::kMaxAngleBatch ? rsx::kMaxAngleBatch : (int)n;
 }
 
-// The planes path's plan: the run of bins the pixels read (all of them where
-// the run would wrap onto itself) and the angles whose planes fit in p.
-// FP64: the pass evaluates the kept bins one by one, 6 ns fused multiply-adds
-// per voxel and angle, and the lateral transforms of the kept planes take
-// ~230 ns / nz; it pays while that is below what transforming every slice and
-// evaluating the morphology per angle takes (~330; FP64 arithmetic is the
-// bound).  FP32 with rows of 512, 1024 or 2048 points keeps the x-first
-// passes (~4x the general lateral transforms' rate).
-static bool planes_plan(const rsx_context* c, int ie, ZPlan* zp) {
-  const rsx_config& g = c->cfg;
-  if (!planes_cfg(&g) || !c->imgs || ie < 0 || ie >= (int)c->energies.size()) return false;
-  if (x_multi_cap(&g) || (g.precision == 32 && g.algorithm == 2 && (g.nx == 512 || g.nx == 1024)))
-    return false;
-  const int blo = lowest_bin(g, wavenumber(c->energies[ie]));
-  zp->ns = 2 - blo < g.nz ? 2 - blo : g.nz;
-  zp->kb = zp->ns == g.nz ? 0 : ((blo % g.nz) + g.nz) % g.nz;
-  if (!rsx::pol_planes_fits(g.precision, g.nz, zp->ns)) return false;
-  if (g.precision == 64 && 6.0 * zp->ns + 230.0 * zp->ns / g.nz > 330.0) return false;
-  const long long kz = c->p_cap / (3LL * zp->ns * c->npix);
-  zp->kz = kz < rsx::kMaxAngleBatch ? (int)kz : rsx::kMaxAngleBatch;
-  return zp->kz >= 1;
-}
-
 static bool zfirst_plan(const rsx_context* c, int ie, ZPlan* zp) {
   const rsx_config& g = c->cfg;
   if (!zfirst_ok(&g) || c->n_sm <= 0 || !c->part || !c->b0idx || ie < 0 ||
@@ -807,6 +787,42 @@ static bool zfirst_plan(const rsx_context* c, int ie, ZPlan* zp) {
   if ((g.nx == 1024 && !c->tw4) || (g.nx == 2048 && !c->tw2k) || (g.ny == 2048 && !c->twy))
     return false;
   return zfirst_plan_of(g, c->kx, wavenumber(c->energies[ie]), zp);
+}
+
+// The planes path's plan: the z-first path's where that serves the energy
+// (its p and z-FFT pass also takes other lateral sizes, FP32 Algorithm 1);
+// else the run of bins the pixels read (all of them where the run would wrap
+// onto itself) and the angles whose planes fit in p.
+// FP64: the general pass evaluates the kept bins one by one, 6 ns fused
+// multiply-adds per voxel and angle, and the lateral transforms of the kept
+// planes take ~230 ns / nz; it pays while that is below what transforming
+// every slice and evaluating the morphology per angle takes (~330; FP64
+// arithmetic is the bound).  FP32 with rows the x-first passes serve (x and
+// p fused, then y and the two bins fused: half the passes over p): while at
+// most 3/4 of the bins are kept.
+static bool planes_plan(const rsx_context* c, int ie, ZPlan* zp) {
+  const rsx_config& g = c->cfg;
+  if (!planes_cfg(&g) || !c->imgs || ie < 0 || ie >= (int)c->energies.size()) return false;
+  if (zfirst_plan(c, ie, zp)) {
+    zp->zfft = true;
+    return true;
+  }
+  const int blo = lowest_bin(g, wavenumber(c->energies[ie]));
+  zp->ns = 2 - blo < g.nz ? 2 - blo : g.nz;
+  zp->kb = zp->ns == g.nz ? 0 : ((blo % g.nz) + g.nz) % g.nz;
+  const bool x_first =
+      x_multi_cap(&g) || (g.precision == 32 && g.algorithm == 2 && (g.nx == 512 || g.nx == 1024));
+  if (x_first && 4 * zp->ns > 3 * g.nz) return false;
+  if (g.precision == 64 && 6.0 * zp->ns + 230.0 * zp->ns / g.nz > 330.0) return false;
+  // the z-first pass's tiles of 1024 / nz pixels of a row, at least two per SM
+  zp->zfft = g.precision == 32 && g.algorithm == 1 && (g.nz == 32 || g.nz == 64 || g.nz == 128) &&
+             g.nx % (1024 / g.nz) == 0 && c->n_sm > 0 && ((uintptr_t)c->M & 15) == 0 &&
+             c->npix * g.nz >= 2048LL * c->n_sm;
+  if (!zp->zfft && !rsx::pol_planes_fits(g.precision, g.nz, zp->ns)) return false;
+  const long long kz = c->p_cap / (3LL * zp->ns * c->npix);
+  const int cap = zp->zfft ? rsx::kMaxXAngles : rsx::kMaxAngleBatch;
+  zp->kz = kz < cap ? (int)kz : cap;
+  return zp->kz >= 1;
 }
 
 size_t rsx_workspace_bytes(const rsx_config* cfg) {
@@ -825,7 +841,8 @@ size_t rsx_workspace_bytes(const rsx_config* cfg) {
   b += 2 * (size_t)npix * R;                         // Ewald, Ewald_Avg (Table 1: 2 nx ny)
   b += (size_t)npix * geo_size(cfg->precision);
   b += (size_t)(cfg->nx + cfg->ny + cfg->nz) * Cs + sizeof(int);
-  if (uses_yz(cfg)) b += part_bytes(cfg) + 2 * (size_t)npix;  // fused y + z pass: bins, bin indices
+  if (uses_yz(cfg)) b += part_bytes(cfg);            // fused y + z pass: bins
+  if (uses_yz(cfg) || y_tuned(cfg)) b += 2 * (size_t)npix;  // lower bin of every pixel
   if (!uses_yz(cfg) || cfg->algorithm == 3)
     b += (size_t)image_batch(cfg) * npix * R;        // a batch of images
   return b;
@@ -941,13 +958,14 @@ int rsx_create(const rsx_config* cfg, rsx_context** out) {
     delete c;
     return rc;
   }
-  if ((cfg->nx == 1024 || cfg->ny == 1024 || (cfg->ny == 2048 && uses_yz(cfg))) &&
+  if ((cfg->nx == 1024 || cfg->ny == 1024 ||
+       (cfg->ny == 2048 && (uses_yz(cfg) || y_tuned(cfg)))) &&
       (rc = upload_tw4(c))) {
     free_all(c);
     delete c;
     return rc;
   }
-  if (cfg->nx == 2048 && angle_batch_cap(cfg) && (rc = upload_tw2k(c))) {
+  if (cfg->nx == 2048 && cfg->precision == 32 && cfg->algorithm != 3 && (rc = upload_tw2k(c))) {
     free_all(c);
     delete c;
     return rc;
@@ -976,8 +994,9 @@ int rsx_create(const rsx_config* cfg, rsx_context** out) {
       c->has_tmap_ftz = make_tmap(c, c->ft, 5LL * cfg->nz, &c->tmap_ftz, box,
                                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
   }
-  if (uses_yz(cfg) && ((e = cudaMalloc(&c->part, part_bytes(cfg))) != cudaSuccess ||
-                       (e = cudaMalloc((void**)&c->b0idx, (size_t)c->npix * 2)) != cudaSuccess)) {
+  if ((uses_yz(cfg) && (e = cudaMalloc(&c->part, part_bytes(cfg))) != cudaSuccess) ||
+      ((uses_yz(cfg) || y_tuned(cfg)) &&
+       (e = cudaMalloc((void**)&c->b0idx, (size_t)c->npix * 2)) != cudaSuccess)) {
     rc = cuda_fail(e, "y + z pass bins");
     free_all(c);
     delete c;
@@ -1287,104 +1306,89 @@ int run_energy_angles_batched(rsx_context* c, int ie, double start, double inc, 
   return RSX_OK;
 }
 
-// All angles of one energy on the z-first path (plan from zfirst_plan):
-// per batch of up to kz angles, the polarisation + z-FFT pass keeps the ns
-// q_z planes of every angle (packed: angle k, field f, plane s at
-// ((k * 3 + f) * ns + s) * nx * ny), one launch x-transforms all their rows,
-// then per angle the fused y-FFT pass picks each pixel's two bins from the
-// planes, the image and the rotation follow as on the other paths.
-int run_energy_zfirst(rsx_context* c, int ie, double start, double inc, int nang, int rotation,
-                      const ZPlan& zp, cudaStream_t s) {
-  const rsx_config& g = c->cfg;
-  int rc = ensure_geo<float>(c, ie, s);
-  if (rc) return rc;
-  CUtensorMap tm_m;
-  if (!make_tmap_m(c, &tm_m)) return fail(RSX_ERR_CUDA, "morphology tensor map");
-  const PolParams<float> pp = make_params<float>(c, ie, 0.0, 0);
-  const double ref = -(double)(g.n_components - 1) / (4.0 * kPi) * (double)c->N;
-  const long long fstride = (long long)zp.ns * c->npix, kstride = 3 * fstride;
-  const void* twx = g.nx == 1024 ? c->tw4 : g.nx == 2048 ? c->tw2k : c->twx;
-  const unsigned box = g.ny == 512 ? 32 : g.ny == 2048 ? 8 : 16;
-  const rsx::YzSel sel = {zp.kb, g.nz};
-  // the angles spread evenly over the fewest passes of at most kz
-  const int npass = (nang + zp.kz - 1) / zp.kz, per = (nang + npass - 1) / npass;
-  for (int a0 = 0; a0 < nang; a0 += per) {
-    const int nk = nang - a0 < per ? nang - a0 : per;
-    rsx::XAngles ang;
-    memset(&ang, 0, sizeof(ang));
-    ang.n = nk;
-    double alpha[rsx::kMaxXAngles];
-    for (int k = 0; k < nk; ++k) {
-      alpha[k] = rotation ? (start + inc * (a0 + k)) * (kPi / 180.0) : 0.0;
-      ang.ce[k] = (float)cos(alpha[k]);
-      ang.se[k] = (float)sin(alpha[k]);
-    }
-    {
-      PhaseTimer pt(c, RSX_PHASE_POL_FFTX, s);
-      RSX_CK(rsx::launch_pol_zfft_multi(&tm_m, g.nx, g.ny, g.nz, pp, ang, c->p, kstride, fstride,
-                                        zp.kb, zp.ns, c->twz, c->err, c->n_sm, c->wait_polls, s),
-             "polarisation + z-FFT kernel");
-    }
-    {
-      PhaseTimer pt(c, RSX_PHASE_FFTX, s);
-      RSX_CK(rsx::launch_xfft_rows(c->p, g.nx, (long long)nk * 3 * zp.ns * g.ny, twx, s),
-             "x-FFT kernel");
-    }
-    for (int k = 0; k < nk; ++k) {
-      float dc[3] = {(float)ref, 0.f, 0.f};
-      if (g.frame != RSX_FRAME_LITERAL) {
-        dc[0] = (float)(ref * cos(alpha[k]));
-        dc[1] = (float)(ref * sin(alpha[k]));
-      }
-      CUtensorMap tm;
-      if (!make_tmap(c, (char*)c->p + (size_t)k * kstride * sizeof(float2), 3LL * zp.ns, &tm, box,
-                     CU_TENSOR_MAP_L2_PROMOTION_L2_128B))
-        return fail(RSX_ERR_CUDA, "q_z plane tensor map");
-      long long L = 0;
-      {
-        PhaseTimer pt(c, RSX_PHASE_FFTY, s);
-        RSX_CK(fused_yz(c, &tm, 3, &L, s, sel, zp.ns), "y-FFT + bin selection kernel");
-      }
-      {
-        PhaseTimer pt(c, RSX_PHASE_EWALD, s);
-        RSX_CK(rsx::launch_ewald_bins(c->part, g.nx, g.ny, zp.ns, L, (const Geo<float>*)c->geo,
-                                      dc[0], dc[1], dc[2], (float*)c->img, s),
-               "Ewald kernel");
-      }
-      PhaseTimer pt(c, RSX_PHASE_ROTATE, s);
-      RSX_CK(rsx::launch_rotate_acc<float>(c->img, c->acc, g.nx, g.ny, alpha[k], rotation != 0, s),
-             "rotation kernel");
-    }
-  }
-  return RSX_OK;
-}
-
-// x-FFT of nrows contiguous rows of the planes in p, in place.
+// x-FFT of the rows of nfields x ns planes in p, in place.
 template <typename R>
-cudaError_t planes_x_fft(rsx_context* c, long long nrows, cudaStream_t s) {
+cudaError_t planes_x_fft(rsx_context* c, const ZPlan& zp, long long nfields, const rsx::XMask& xm,
+                         cudaStream_t s) {
   const rsx_config& g = c->cfg;
   if (g.nx == 1) return cudaSuccess;
   if (sizeof(R) == 4 && (g.nx == 512 || (g.nx == 1024 && c->tw4) || (g.nx == 2048 && c->tw2k)))
-    return rsx::launch_xfft_rows(c->p, g.nx, nrows,
-                                 g.nx == 1024 ? c->tw4 : g.nx == 2048 ? c->tw2k : c->twx, s);
+    return rsx::launch_x_planes(c->p, g.nx, g.ny, zp.ns, nfields, xm,
+                                g.nx == 1024 ? c->tw4 : g.nx == 2048 ? c->tw2k : c->twx, s);
+  const long long nrows = nfields * zp.ns * g.ny;
   if (g.nx == 1024 && c->tw4) return rsx::launch_row_fft4s<R>(c->p, nrows, c->tw4, s);
   return rsx::launch_row_fft<R>(c->p, g.nx, nrows, c->twx, s);
 }
 
-// y-FFT of nplanes contiguous [ny][nx] planes in p, in place.
+// y-FFT of nfields x ns contiguous [ny][nx] planes in p, in place; on the
+// tuned sizes only what the image reads is transformed and stored.
 template <typename R>
-cudaError_t planes_y_fft(rsx_context* c, long long nplanes, cudaStream_t s) {
+cudaError_t planes_y_fft(rsx_context* c, const ZPlan& zp, long long nfields,
+                         const rsx::YRuns& runs, cudaStream_t s) {
   const rsx_config& g = c->cfg;
-  const rsx::ColBatches bt = {nplanes, 1, c->npix, 0, 0};
+  if (g.ny == 1) return cudaSuccess;
+  if (sizeof(R) == 4 && y_tuned(&g) && c->b0idx && zp.ns < g.nz && c->n_sm > 0) {
+    CUtensorMap tm;
+    if (!make_tmap(c, c->p, nfields * zp.ns, &tm, 16384u / g.ny, CU_TENSOR_MAP_L2_PROMOTION_L2_128B))
+      return cudaErrorUnknown;
+    return rsx::launch_y_planes(&tm, c->p, g.nx, g.ny, g.nz, zp.kb, zp.ns, nfields, runs, c->b0idx,
+                                g.ny == 512 ? c->twy : c->tw4, g.ny == 2048 ? c->twy : nullptr,
+                                c->err, c->n_sm, c->wait_polls, s);
+  }
+  const rsx::ColBatches bt = {nfields * zp.ns, 1, c->npix, 0, 0};
   if (g.ny == 1024 && g.nx % 8 == 0 && c->tw4)
     return rsx::launch_col_fft4s<R>(c->p, g.nx, g.nx, bt, c->tw4, s);
   return rsx::launch_col_fft<R>(c->p, g.ny, g.nx, g.nx, bt, c->twy, s);
 }
 
-// All angles of one energy on the general planes path (plan from
-// planes_plan): per batch of angles one launch each for p and its pruned z
-// transform, the x-FFT and the y-FFT of every kept plane, then the images
-// and the rotation into the average, n_img angles at a time.
+// The runs of planes that each 16-column group's pixels read, and per plane
+// the groups of nx / 32 columns some run meets.  A column's bins run from
+// the one at q_y = 0 down to the one at the largest |q_y| still on the sphere;
+// the bounds are wide enough for any rounding, as in lowest_bin.
+void plane_runs(const rsx_config& g, double k, const ZPlan& zp, rsx::YRuns* runs,
+                rsx::XMask* xm) {
+  memset(runs, 0, sizeof(*runs));
+  memset(xm, zp.ns < g.nz ? 0 : 0xff, sizeof(*xm));
+  if (zp.ns >= g.nz || g.nx % 16 || g.nx > 4096) {
+    memset(xm, 0xff, sizeof(*xm));
+    return;
+  }
+  const double two_pi = 2.0 * kPi, dqx = two_pi / (g.nx * g.voxel_nm),
+               dqy = two_pi / (g.ny * g.voxel_nm), dqz = two_pi / (g.nz * g.voxel_nm);
+  const double edge = 1e-12 * k * k, qy = dqy * (g.ny / 2);
+  const int blo = 2 - zp.ns;
+  runs->n = g.nx / 16;
+  for (int cg = 0; cg < runs->n; ++cg) {
+    int fmin = g.nx, fmax = 0;
+    for (int i = 0; i < 16; ++i) {
+      const int mx = cg * 16 + i, f = mx < g.nx / 2 ? mx : g.nx - mx;
+      fmin = f < fmin ? f : fmin;
+      fmax = f > fmax ? f : fmax;
+    }
+    const double top = k * k - dqx * fmin * dqx * fmin;
+    const double low = k * k - dqx * fmax * dqx * fmax - qy * qy;
+    int len = 0;
+    if (top >= -edge) {
+      const double th = (-k + sqrt(top > 0.0 ? top : 0.0)) / dqz;
+      const double tl = (low > edge ? -k + sqrt(low) : -k) / dqz;
+      int hi = (int)floor(th + 1e-9 * (1.0 + fabs(th))) + 1 - blo;
+      int lo = (int)floor(tl - 1e-9 * (1.0 + fabs(tl))) - blo;
+      lo = lo < 0 ? 0 : lo;
+      hi = hi > zp.ns - 1 ? zp.ns - 1 : hi;
+      runs->first[cg] = (unsigned char)lo;
+      len = hi >= lo ? hi - lo + 1 : 0;
+      for (int z = lo; z <= hi; ++z) xm->m[z] |= 1u << (cg * 16 / ((g.nx + 31) / 32));
+    }
+    runs->start[cg + 1] = (unsigned short)(runs->start[cg] + len);
+  }
+}
+
+// All angles of one energy on the planes path (plan from planes_plan): per
+// batch of up to kz angles, the polarisation + z-transform pass keeps the ns
+// q_z planes of every angle (angle k, field f, plane s at
+// ((k * 3 + f) * ns + s) * nx * ny of p), one launch each x- and
+// y-transforms them, then the images and the rotation into the average
+// follow, n_img angles at a time.
 template <typename R>
 int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang, int rotation,
                       const ZPlan& zp, cudaStream_t s) {
@@ -1394,6 +1398,12 @@ int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang
   if (g.algorithm == 2 && (rc = ensure_nt<R>(c, ie, s))) return rc;
   const PolParams<R> pp = make_params<R>(c, ie, 0.0, 0);
   const double ref = -(double)(g.n_components - 1) / (4.0 * kPi) * (double)c->N;
+  rsx::YRuns runs;
+  rsx::XMask xm;
+  plane_runs(g, wavenumber(c->energies[ie]), zp, &runs, &xm);
+  CUtensorMap tm_m;
+  if (zp.zfft && !make_tmap_m(c, &tm_m)) return fail(RSX_ERR_CUDA, "morphology tensor map");
+  // the angles spread evenly over the fewest passes of at most kz
   const int npass = (nang + zp.kz - 1) / zp.kz, per = (nang + npass - 1) / npass;
   for (int a0 = 0; a0 < nang; a0 += per) {
     const int nk = nang - a0 < per ? nang - a0 : per;
@@ -1406,17 +1416,35 @@ int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang
     }
     {
       PhaseTimer pt(c, RSX_PHASE_POL_FFTX, s);
-      RSX_CK(rsx::launch_pol_planes<R>(c->M, g.algorithm == 2 ? c->nt : nullptr, c->dir, c->npix,
-                                       g.nz, pp, ab, c->p, zp.kb, zp.ns, c->twz, s),
-             "polarisation + z-transform kernel");
+      cudaError_t e;
+      if constexpr (sizeof(R) == 4) {
+        if (zp.zfft) {
+          rsx::XAngles ang;
+          memset(&ang, 0, sizeof(ang));
+          ang.n = nk;
+          memcpy(ang.ce, ab.ce, nk * sizeof(float));
+          memcpy(ang.se, ab.se, nk * sizeof(float));
+          const long long fstride = (long long)zp.ns * c->npix;
+          e = rsx::launch_pol_zfft_multi(&tm_m, g.nx, g.ny, g.nz, pp, ang, c->p, 3 * fstride,
+                                         fstride, zp.kb, zp.ns, c->twz, c->err, c->n_sm,
+                                         c->wait_polls, s);
+        } else {
+          e = rsx::launch_pol_planes<R>(c->M, g.algorithm == 2 ? c->nt : nullptr, c->dir, c->npix,
+                                        g.nz, pp, ab, c->p, zp.kb, zp.ns, c->twz, s);
+        }
+      } else {
+        e = rsx::launch_pol_planes<R>(c->M, g.algorithm == 2 ? c->nt : nullptr, c->dir, c->npix,
+                                      g.nz, pp, ab, c->p, zp.kb, zp.ns, c->twz, s);
+      }
+      RSX_CK(e, "polarisation + z-transform kernel");
     }
     {
       PhaseTimer pt(c, RSX_PHASE_FFTX, s);
-      RSX_CK(planes_x_fft<R>(c, (long long)nk * 3 * zp.ns * g.ny, s), "x-FFT kernel");
+      RSX_CK(planes_x_fft<R>(c, zp, 3LL * nk, xm, s), "x-FFT kernel");
     }
     if (g.ny > 1) {
       PhaseTimer pt(c, RSX_PHASE_FFTY, s);
-      RSX_CK(planes_y_fft<R>(c, (long long)nk * 3 * zp.ns, s), "y-FFT kernel");
+      RSX_CK(planes_y_fft<R>(c, zp, 3LL * nk, runs, s), "y-FFT kernel");
     }
     for (int i0 = 0; i0 < nk; i0 += c->n_img) {
       const int ni = nk - i0 < c->n_img ? nk - i0 : c->n_img;
@@ -1449,16 +1477,14 @@ int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang
 template <typename R>
 int run_energy_angles(rsx_context* c, int ie, double start, double inc, int nang, int rotation,
                       cudaStream_t s) {
+  ZPlan zp;
+  if (planes_plan(c, ie, &zp))
+    return run_energy_planes<R>(c, ie, start, inc, nang, rotation, zp, s);
   if constexpr (sizeof(R) == 4) {
-    ZPlan zp;
-    if (zfirst_plan(c, ie, &zp)) return run_energy_zfirst(c, ie, start, inc, nang, rotation, zp, s);
     if ((c->kx > 1 || c->cfg.nx == 2048) && x_multi_cap(&c->cfg) && c->n_sm > 0 &&
         ((uintptr_t)c->M & 15) == 0)
       return run_energy_angles_batched(c, ie, start, inc, nang, rotation, s);
   }
-  ZPlan pl;
-  if (planes_plan(c, ie, &pl))
-    return run_energy_planes<R>(c, ie, start, inc, nang, rotation, pl, s);
   for (int a = 0; a < nang; ++a) {
     const double alpha = rotation ? (start + inc * a) * (kPi / 180.0) : 0.0;
     int rc = scatter_angle<R>(c, ie, alpha, c->img, s);

@@ -1124,43 +1124,6 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_zfft_multi(
   }
 }
 
-// x-FFT of contiguous rows of NX complex in place (the kept q_z planes of
-// the z-first path): one warp per row, the row staged in shared memory in
-// the layout xfft_row<NX> takes (2048 points: halves at 0 and 1056; every
-// copy 16-byte aligned: rows of 8 NX bytes, FS and NTW even), then
-// xfft_row's four-step transform writes it back.  tw_g: the table xfft_row
-// uses (1024: W1024^(n1 k2) as [32][32]; 2048: that, then W2048^n, n < 1024;
-// 512: W512^j).
-template <int NX, int W>
-__global__ void __launch_bounds__(32 * W) k_xfft_rows(float2* __restrict__ data, long long nrows,
-                                                      const float2* __restrict__ tw_g) {
-  using C = float2;
-  constexpr int FS = NX == 2048 ? 2 * 1056 : (NX / 32) * 33;
-  constexpr int NTW = NX == 2048 ? 2048 : NX == 1024 ? 1024 : 512;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* tw = reinterpret_cast<C*>(smem_raw);
-  C* F = tw + NTW + (threadIdx.x >> 5) * FS;
-  const int lane = threadIdx.x & 31;
-  const long long row = (long long)blockIdx.x * W + (threadIdx.x >> 5);
-  C* r = data + (size_t)row * NX;
-  // the row goes to shared memory by asynchronous 16-byte copies (a lane
-  // keeps all NX / 64 of its copies in flight, no registers held), issued
-  // before the twiddle table's loads so that the two overlap
-  if (row < nrows) {
-#pragma unroll
-    for (int j = 0; j < NX / 64; ++j) {
-      const int n = 2 * (lane + 32 * j);
-      cp_async_pair(F + (NX == 2048 && n >= 1024 ? n + 32 : n), r + n);
-    }
-  }
-  for (int i = threadIdx.x; i < NTW; i += 32 * W) tw[i] = tw_g[i];
-  __syncthreads();
-  if (row >= nrows) return;
-  cp_async_wait_all();
-  __syncwarp();
-  xfft_row<NX>(F, tw, r, lane, [] {});
-}
-
 // y pass: a tile of TX adjacent columns of one batch.  Thread (n1, col)
 // loads rows n1 + 32 n2 straight from global memory (32 independent loads),
 // transforms over n2 in registers, applies the twiddles and writes row k2 of
@@ -1816,13 +1779,7 @@ __device__ __forceinline__ void yz2k_load(const float2* xb, int r0, int c4, bool
 // from columns 0-3, odd from 4-7), so the rest of the pass is unchanged;
 // virtual pixel (row, col) is the real pixel (2 row + col / 4, 4 ti + col mod 4).
 // tw2k: W2048^j (j < 64 used).
-//
-// SEL: the z-first path's planes instead of z-slices.  A field holds nz = ns
-// planes (any count), plane s being bin (kb + s) mod (zmask + 1) of the z
-// transform, already x-transformed; each pixel's two bins are planes
-// sb = (b0 - kb) mod (zmask + 1) and sb + 1, so a step selects instead of
-// accumulating: A0 = Y(sb), A1 = Y(sb + 1) (twz unused).
-template <bool Y2K, bool SEL>
+template <bool Y2K>
 __global__ void __launch_bounds__(512, 1) k_yz_tma(const __grid_constant__ CUtensorMap tmap, int nx,
                                                    int nz, int nf, int ntiles, int L, int T,
                                                    const Geo<float>* __restrict__ geo,
@@ -1831,7 +1788,7 @@ __global__ void __launch_bounds__(512, 1) k_yz_tma(const __grid_constant__ CUten
                                                    const float2* __restrict__ tw2k,
                                                    const unsigned short* __restrict__ b0idx,
                                                    float4* __restrict__ part, int* __restrict__ err,
-                                                   unsigned poll, int kb, int zmask) {
+                                                   unsigned poll) {
   using C = float2;
   constexpr int TX = 8, TILE = 1024 * TX, STR = 33 * TX;
   constexpr int GRP = Y2K ? 4 : 2, LGRP = Y2K ? 2 : 1;  // blocks reading one line in lockstep
@@ -1843,9 +1800,6 @@ __global__ void __launch_bounds__(512, 1) k_yz_tma(const __grid_constant__ CUten
   C* twz = tw4 + 1024;                       // [nz]
   unsigned short* btab = reinterpret_cast<unsigned short*>(twz + nz);  // [1024][TX]
   unsigned long long* bar = reinterpret_cast<unsigned long long*>(btab + TILE);
-  // SEL: each thread's 16 plane indices as bytes, [512][16] over the unused
-  // twz (16-byte aligned), read as one 16-byte word per step
-  unsigned char* btab8 = reinterpret_cast<unsigned char*>(twz);
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int col = lane & 7, hw = w >> 3;
   const int q = (w & 7) * 4 + (lane >> 3);  // n1 in stage 1, k2 in stage 2
@@ -1865,18 +1819,12 @@ __global__ void __launch_bounds__(512, 1) k_yz_tma(const __grid_constant__ CUten
     fence_proxy_async();
   }
   for (int i = t; i < 1024; i += 512) tw4[i] = tw4_g[i];
-  if constexpr (!SEL)
-    for (int i = t; i < nz; i += 512) twz[i] = twz_g[i];
+  for (int i = t; i < nz; i += 512) twz[i] = twz_g[i];
   __syncthreads();
-  // step st -> (work item, slice or plane z)
+  // step st -> (work item, slice z)
   auto split = [&](int st, int& item, int& z) {
-    if constexpr (SEL) {
-      item = st / nz;
-      z = st - item * nz;
-    } else {
-      item = st >> lognz;
-      z = st & (nz - 1);
-    }
+    item = st >> lognz;
+    z = st & (nz - 1);
   };
   auto issue = [&](int st, int b) {
     int item, z;
@@ -1908,16 +1856,7 @@ __global__ void __launch_bounds__(512, 1) k_yz_tma(const __grid_constant__ CUten
       for (int e = t; e < TILE; e += 512) {
         const size_t pixel = Y2K ? (size_t)(2 * (e >> 3) + ((e & 7) >> 2)) * nx + ti * 4 + (e & 3)
                                  : (size_t)(e >> 3) * nx + ti * TX + (e & 7);
-        const int bin = b0idx[pixel];
-        if constexpr (SEL) {
-          // virtual pixel (row, col) belongs to the stage-3 thread
-          // (q, hw, col) with row = q + 512 hw + 32 k: byte k of its word
-          const int row = e >> 3, rem = row & 511, qq = rem & 31;
-          const int owner = ((row >> 9) * 8 + (qq >> 2)) * 32 + ((qq & 3) << 3) + (e & 7);
-          btab8[owner * 16 + (rem >> 5)] = (unsigned char)((bin - kb) & zmask);
-        } else {
-          btab[e] = (unsigned short)bin;
-        }
+        btab[e] = b0idx[pixel];
       }
 #pragma unroll
       for (int k = 0; k < 16; ++k) acc0[k] = acc1[k] = make_float2(0.f, 0.f);
@@ -1976,36 +1915,19 @@ __global__ void __launch_bounds__(512, 1) k_yz_tma(const __grid_constant__ CUten
     }
     __syncthreads();  // halves swapped; every stage-2 read of tr is done
     {
-      const C wz = SEL ? make_float2(1.f, 0.f) : twz[z];
-      uint4 sb4 = make_uint4(0u, 0u, 0u, 0u);
-      float2* sel0 = nullptr;  // SEL: slot 0 of this thread's pixel column, as float2 pairs
-      if constexpr (SEL) {
-        sb4 = reinterpret_cast<const uint4*>(btab8)[t];
-        sel0 = reinterpret_cast<float2*>(
-            part + (size_t)(item >> loghalf) * npix +
-            (Y2K ? (size_t)(col >> 2) * nx + ti * 4 + (col & 3) : (size_t)ti * TX + col));
-      }
+      const C wz = twz[z];
 #pragma unroll
       for (int k = 0; k < 16; ++k) {
         const C mine = v[out_pos<16>(k)];
         const C other = xb[(16 * (1 - hw) + k) * 256 + q * TX + col];
         const C y = hw ? csub(other, mine) : cadd(mine, other);  // X[k2 + 32 (16 hw + k)]
         const int row = q + 512 * hw + 32 * k;
-        if constexpr (SEL) {
-          // each pixel's bins come from one plane each: stored as they pass
-          const unsigned wd = k < 4 ? sb4.x : k < 8 ? sb4.y : k < 12 ? sb4.z : sb4.w;
-          const int sb = (int)((wd >> (8 * (k & 3))) & 0xffu);
-          float2* d = sel0 + 2 * (size_t)row * (Y2K ? 2 * nx : nx);
-          if (sb == z) d[0] = y;
-          if (sb + 1 == z) d[1] = y;
-        } else {
-          const int b0 = btab[row * TX + col];
-          const C qq = cmul(y, twz[(b0 * z) & (nz - 1)]);
-          acc0[k] = cadd(acc0[k], qq);
-          acc1[k] = cadd(acc1[k], cmul(qq, wz));
-        }
+        const int b0 = btab[row * TX + col];
+        const C qq = cmul(y, twz[(b0 * z) & (nz - 1)]);
+        acc0[k] = cadd(acc0[k], qq);
+        acc1[k] = cadd(acc1[k], cmul(qq, wz));
       }
-      if (!SEL && (z == nz - 1 || st == s1 - 1)) {  // segment end: slot 0 if it began at z = 0
+      if (z == nz - 1 || st == s1 - 1) {  // segment end: slot 0 if it began at z = 0
         // slot: this segment's place among the item's segments (0 if it
         // began at z = 0); L >= nz / 3 keeps it below kYzSlots
         const int item_start = st - z;
@@ -2038,9 +1960,7 @@ __global__ void __launch_bounds__(512, 1) k_yz_tma(const __grid_constant__ CUten
 //           registers, which leaves it the 16 pixels k2 + 32 k1 (no swap);
 // then the two q_z bins of those pixels are accumulated across z as in
 // k_yz_tma.  The consumed input buffer is refilled (slice + 2) right after
-// stage 1.  Waits are bounded as in k_col_fft4s_tma.  SEL: the z-first
-// path's planes, as in k_yz_tma.
-template <bool SEL>
+// stage 1.  Waits are bounded as in k_col_fft4s_tma.
 __global__ void __launch_bounds__(512, 1) k_yz512_tma(const __grid_constant__ CUtensorMap tmap,
                                                       int nx, int nz, int nf, int ntiles, int L,
                                                       int T, const Geo<float>* __restrict__ geo,
@@ -2048,8 +1968,7 @@ __global__ void __launch_bounds__(512, 1) k_yz512_tma(const __grid_constant__ CU
                                                       const float2* __restrict__ twy_g,
                                                       const unsigned short* __restrict__ b0idx,
                                                       float4* __restrict__ part,
-                                                      int* __restrict__ err, unsigned poll,
-                                                      int kb, int zmask) {
+                                                      int* __restrict__ err, unsigned poll) {
   using C = float2;
   constexpr int TX = 16, NY = 512, TILE = NY * TX, STR = 33 * 8;
   constexpr unsigned kPoll = 1u << 22;
@@ -2073,18 +1992,12 @@ __global__ void __launch_bounds__(512, 1) k_yz512_tma(const __grid_constant__ CU
     fence_proxy_async();
   }
   for (int i = t; i < NY; i += 512) twy[i] = twy_g[i];
-  if constexpr (!SEL)
-    for (int i = t; i < nz; i += 512) twz[i] = twz_g[i];
+  for (int i = t; i < nz; i += 512) twz[i] = twz_g[i];
   __syncthreads();
-  // step st -> (work item, slice or plane z)
+  // step st -> (work item, slice z)
   auto split = [&](int st, int& item, int& z) {
-    if constexpr (SEL) {
-      item = st / nz;
-      z = st - item * nz;
-    } else {
-      item = st >> lognz;
-      z = st & (nz - 1);
-    }
+    item = st >> lognz;
+    z = st & (nz - 1);
   };
   auto issue = [&](int st, int b) {
     int item, z;
@@ -2109,8 +2022,7 @@ __global__ void __launch_bounds__(512, 1) k_yz512_tma(const __grid_constant__ CU
     if (z == 0 || st == s0) {  // a new segment: this tile's bins, zero accumulators
       __syncthreads();  // the previous step's reads of the bins are done
       for (int e = t; e < TILE; e += 512) {
-        const int bin = b0idx[(size_t)(e >> 4) * nx + ti * TX + (e & 15)];
-        btab[e] = (unsigned short)(SEL ? (bin - kb) & zmask : bin);
+        btab[e] = b0idx[(size_t)(e >> 4) * nx + ti * TX + (e & 15)];
       }
 #pragma unroll
       for (int k = 0; k < 16; ++k) acc0[k] = acc1[k] = make_float2(0.f, 0.f);
@@ -2154,26 +2066,16 @@ __global__ void __launch_bounds__(512, 1) k_yz512_tma(const __grid_constant__ CU
         v[n1] = cmul(make_float2(fmaf(sg, o.x, e.x), fmaf(sg, o.y, e.y)), twy[n1 * k2]);
       }
       dft_reg<16>(v);
-      const C wz = SEL ? make_float2(1.f, 0.f) : twz[z];
-      float2* sel0 = nullptr;  // SEL: slot 0 of this thread's pixel column, as float2 pairs
-      if constexpr (SEL)
-        sel0 = reinterpret_cast<float2*>(part + (size_t)(item / ntiles) * npix + (size_t)ti * TX + col);
+      const C wz = twz[z];
 #pragma unroll
       for (int k1 = 0; k1 < 16; ++k1) {
         const int row = k2 + 32 * k1;
         const int b0 = btab[row * TX + col];
-        if constexpr (SEL) {
-          // each pixel's bins come from one plane each: stored as they pass
-          float2* d = sel0 + 2 * (size_t)row * nx;
-          if (b0 == z) d[0] = v[out_pos<16>(k1)];
-          if (b0 + 1 == z) d[1] = v[out_pos<16>(k1)];
-        } else {
-          const C qq = cmul(v[out_pos<16>(k1)], twz[(b0 * z) & (nz - 1)]);
-          acc0[k1] = cadd(acc0[k1], qq);
-          acc1[k1] = cadd(acc1[k1], cmul(qq, wz));
-        }
+        const C qq = cmul(v[out_pos<16>(k1)], twz[(b0 * z) & (nz - 1)]);
+        acc0[k1] = cadd(acc0[k1], qq);
+        acc1[k1] = cadd(acc1[k1], cmul(qq, wz));
       }
-      if (!SEL && (z == nz - 1 || st == s1 - 1)) {  // segment end: slot 0 if it began at z = 0
+      if (z == nz - 1 || st == s1 - 1) {  // segment end: slot 0 if it began at z = 0
         // slot: this segment's place among the item's segments (0 if it
         // began at z = 0); L >= nz / 3 keeps it below kYzSlots
         const int item_start = st - z;
@@ -3012,38 +2914,15 @@ cudaError_t launch_pol_zfft_multi(const void* tmap, int nx, int ny, int nz,
                                   long long kstride, long long fstride, int kb, int ns,
                                   const void* twz, int* err, int n_sm, unsigned poll,
                                   cudaStream_t s) {
-  if (!zfirst_fusable(nx, ny, nz)) return cudaErrorInvalidValue;
   if (nz == 128)
     return pol_zfft_impl<4>(tmap, nx, ny, pp, ang, out, kstride, fstride, kb, ns, twz, err, n_sm,
                             poll, s);
   if (nz == 64)
     return pol_zfft_impl<2>(tmap, nx, ny, pp, ang, out, kstride, fstride, kb, ns, twz, err, n_sm,
                             poll, s);
+  if (nz != 32) return cudaErrorInvalidValue;
   return pol_zfft_impl<1>(tmap, nx, ny, pp, ang, out, kstride, fstride, kb, ns, twz, err, n_sm,
                           poll, s);
-}
-
-template <int NX, int W>
-static cudaError_t xfft_rows_impl(void* data, long long nrows, const void* tw, cudaStream_t s) {
-  constexpr int FS = NX == 2048 ? 2 * 1056 : (NX / 32) * 33;
-  constexpr int NTW = NX == 2048 ? 2048 : NX == 1024 ? 1024 : 512;
-  const size_t smem = ((size_t)NTW + (size_t)W * FS) * sizeof(float2);
-  auto kern = k_xfft_rows<NX, W>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  kern<<<grid1(nrows, W), 32 * W, smem, s>>>((float2*)data, nrows, (const float2*)tw);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_xfft_rows(void* data, int nx, long long nrows, const void* tw, cudaStream_t s) {
-  if (nrows <= 0) return cudaSuccess;
-  if (!tw || ((uintptr_t)data & 15)) return cudaErrorInvalidValue;  // 16-byte row copies
-  // 8 warps (2 blocks per SM) for 512- and 1024-point rows; 2048-point rows
-  // stage 17 KB per warp: 4 warps (2 blocks per SM)
-  if (nx == 1024) return xfft_rows_impl<1024, 8>(data, nrows, tw, s);
-  if (nx == 2048) return xfft_rows_impl<2048, 4>(data, nrows, tw, s);
-  if (nx == 512) return xfft_rows_impl<512, 8>(data, nrows, tw, s);
-  return cudaErrorInvalidValue;
 }
 
 bool yz_fusable(int nx, int ny, int nz) {
@@ -3055,19 +2934,11 @@ bool yz_fusable(int nx, int ny, int nz) {
          nz >= (ny == 2048 ? 4 : 1) && nz <= 1024 && (nz & (nz - 1)) == 0;
 }
 
-// sel.nzfull > 0: the z-first path's planes (nz = their count per field).
-static bool yz_sel_ok(int nx, int nz, const YzSel& sel) {
-  return nx >= 16 && (nx & (nx - 1)) == 0 && nz >= 1 && nz <= sel.nzfull && sel.nzfull <= 1024 &&
-         (sel.nzfull & (sel.nzfull - 1)) == 0 && sel.kb >= 0 && sel.kb < sel.nzfull;
-}
-
 cudaError_t launch_yz512_tma(const void* tmap, int nx, int nz, int nf, const Geo<float>* geo,
                              const void* twz, const void* twy, const unsigned short* b0idx,
                              void* part, int* err, int n_sm, unsigned poll, long long* L_out,
-                             cudaStream_t s, YzSel sel) {
-  const bool is_sel = sel.nzfull > 0;
-  if (!(is_sel ? yz_sel_ok(nx, nz, sel) : yz_fusable(nx, 512, nz)) || n_sm <= 0 ||
-      (nf != 3 && nf != 5))
+                             cudaStream_t s) {
+  if (!yz_fusable(nx, 512, nz) || n_sm <= 0 || (nf != 3 && nf != 5))
     return cudaErrorInvalidValue;
   const long long ntiles = nx / 16, items = nf * ntiles, T = items * nz;
   // equal step ranges over as many blocks as SMs, but at least nz / 3 steps
@@ -3075,27 +2946,23 @@ cudaError_t launch_yz512_tma(const void* tmap, int nx, int nz, int nf, const Geo
   const long long L0 = (T + n_sm - 1) / n_sm, Lmin = (nz + kYzSlots - 2) / (kYzSlots - 1);
   const long long L = L0 > Lmin ? L0 : Lmin;
   const long long grid = (T + L - 1) / L;
-  // SEL: every bin is stored once, in slot 0 (k_ewald_bins adds no other slot)
-  *L_out = is_sel ? T : L;
+  *L_out = L;
   const size_t smem = (2 * 8192 + 32 * 33 * 8 + 512 + (size_t)nz) * sizeof(float2) +
                       8192 * sizeof(unsigned short) + 2 * 8;
-  auto kern = is_sel ? k_yz512_tma<true> : k_yz512_tma<false>;
+  auto kern = k_yz512_tma;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)grid, 512, smem, s>>>(*(const CUtensorMap*)tmap, nx, nz, nf, (int)ntiles, (int)L,
                                          (int)T, geo, (const float2*)twz, (const float2*)twy, b0idx,
-                                         (float4*)part, err, poll, sel.kb, sel.nzfull - 1);
+                                         (float4*)part, err, poll);
   return cudaGetLastError();
 }
 
 cudaError_t launch_yz_tma(const void* tmap, int nx, int ny, int nz, int nf, const Geo<float>* geo,
                           const void* twz, const void* tw4, const void* tw2k,
                           const unsigned short* b0idx, void* part, int* err, int n_sm,
-                          unsigned poll, long long* L_out, cudaStream_t s, YzSel sel) {
-  const bool is_sel = sel.nzfull > 0;
-  if (!(is_sel ? yz_sel_ok(nx, nz, sel) && (ny == 1024 || ny == 2048) : yz_fusable(nx, ny, nz)) ||
-      ny == 512 || n_sm <= 0)
-    return cudaErrorInvalidValue;
+                          unsigned poll, long long* L_out, cudaStream_t s) {
+  if (!yz_fusable(nx, ny, nz) || ny == 512 || n_sm <= 0) return cudaErrorInvalidValue;
   if (nf != 3 && nf != 5) return cudaErrorInvalidValue;
   // 1024 rows: pairs of 8-column tiles; 2048 rows: quads of 4-column tiles
   const bool y2k = ny == 2048;
@@ -3109,19 +2976,17 @@ cudaError_t launch_yz_tma(const void* tmap, int nx, int ny, int nz, int nf, cons
   const long long L0 = (T + P0 - 1) / P0, Lmin = (nz + kYzSlots - 2) / (kYzSlots - 1);
   const long long L = L0 > Lmin ? L0 : Lmin;
   const long long groups = (T + L - 1) / L;
-  // SEL: every bin is stored once, in slot 0 (k_ewald_bins adds no other slot)
-  *L_out = is_sel ? T : L;
+  *L_out = L;
   const size_t smem = (2 * 8192 + 32 * 33 * 8 + 1024 + (size_t)nz) * sizeof(float2) +
                       8192 * sizeof(unsigned short) + 2 * 8;
-  auto kern = y2k ? (is_sel ? k_yz_tma<true, true> : k_yz_tma<true, false>)
-                  : (is_sel ? k_yz_tma<false, true> : k_yz_tma<false, false>);
+  auto kern = y2k ? k_yz_tma<true> : k_yz_tma<false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)(grp * groups), 512, smem, s>>>(*(const CUtensorMap*)tmap, nx, nz, nf,
                                                     (int)ntiles, (int)L, (int)T, geo,
                                                     (const float2*)twz, (const float2*)tw4,
                                                     (const float2*)tw2k, b0idx, (float4*)part,
-                                                    err, poll, sel.kb, sel.nzfull - 1);
+                                                    err, poll);
   return cudaGetLastError();
 }
 

@@ -192,18 +192,16 @@ cudaError_t launch_pol_fft4s_tma_multi(const void* M, int nx, int ny, int nz,
 // out + k * kstride + f * fstride + s * nx * ny as an [ny][nx] complex plane
 // (not yet x- or y-transformed).  tmap: a CUtensorMap over the morphology
 // viewed as [c nz][ny][4 nx] floats with (128 / nz) x 1 x nz boxes (see
-// make_tmap_m); twz: exp(-2 pi i j / nz), j < nz.  zfirst_fusable says
-// whether the shape qualifies (nz = 32, 64 or 128; nx and ny = 512, 1024 or
-// 2048).  One persistent CTA per SM (n_sm).
+// make_tmap_m); twz: exp(-2 pi i j / nz), j < nz.  nz = 32, 64 or 128, nx a
+// multiple of 1024 / nz.  zfirst_fusable: the shapes whose lateral passes
+// are tuned too (nx and ny = 512, 1024 or 2048).  One persistent CTA per SM
+// (n_sm).
 bool zfirst_fusable(int nx, int ny, int nz);
 cudaError_t launch_pol_zfft_multi(const void* tmap, int nx, int ny, int nz,
                                   const PolParams<float>& pp, const XAngles& ang, void* out,
                                   long long kstride, long long fstride, int kb, int ns,
                                   const void* twz, int* err, int n_sm, unsigned poll,
                                   cudaStream_t s);
-// In-place x-FFT of nrows contiguous rows of nx = 512, 1024 or 2048 complex
-// (FP32; tw: twx for 512, tw4 for 1024, the 2048-point table for 2048).
-cudaError_t launch_xfft_rows(void* data, int nx, long long nrows, const void* tw, cudaStream_t s);
 // The same pipeline for Algorithm 2: p = N_t e from the five stored entries
 // of N_t ([5][N] complex float, 16-byte aligned; the reference constant
 // left out as k_nt_all stores it).
@@ -223,23 +221,16 @@ bool yz_fusable(int nx, int ny, int nz);
 // this many blocks (their step ranges hold at least nz / (kYzSlots - 1)).
 constexpr int kYzSlots = 4;
 // b0idx: each pixel's lower q_z bin (launch_geometry's packed output).
-// sel: the z-first path's planes instead of z-slices when nzfull > 0: nz is
-// then the plane count per field (any value up to nzfull), plane s holds bin
-// (kb + s) mod nzfull, and each pixel takes its two bins from planes
-// (b0 - kb) mod nzfull and the one after.
-struct YzSel {
-  int kb = 0, nzfull = 0;
-};
 cudaError_t launch_yz_tma(const void* tmap, int nx, int ny, int nz, int nf, const Geo<float>* geo,
                           const void* twz, const void* tw4, const void* tw2k,
                           const unsigned short* b0idx, void* part, int* err, int n_sm,
-                          unsigned poll, long long* L_out, cudaStream_t s, YzSel sel = YzSel());
+                          unsigned poll, long long* L_out, cudaStream_t s);
 // The same for ny = 512 (16-column tiles, tensor map boxes of 32 floats x
 // 256 rows; twy the 512-point twiddle table).
 cudaError_t launch_yz512_tma(const void* tmap, int nx, int nz, int nf, const Geo<float>* geo,
                              const void* twz, const void* twy, const unsigned short* b0idx,
                              void* part, int* err, int n_sm, unsigned poll, long long* L_out,
-                             cudaStream_t s, YzSel sel = YzSel());
+                             cudaStream_t s);
 // The linearity path's per-energy bins (k_zbins5 layout) from launch_yz_tma
 // run over the five FFT'd N_t entries (nf = 5); dc = -(c-1)/(4 pi) N.
 cudaError_t launch_bins5_from_part(const void* part, int nx, int ny, int nz, long long L,
@@ -325,6 +316,35 @@ template <typename R>
 cudaError_t launch_pol_planes(const void* M, const void* nt, const void* dir, long long npix,
                               int nz, const PolParams<R>& pp, const AngleBatch<R>& ang, void* out,
                               int kb, int ns, const void* twz, cudaStream_t s);
+// The lateral transforms of the planes for tuned sizes (FP32), in place.
+// YRuns: per 16-column group cg < n the run of planes its pixels read:
+// first[cg] .. first[cg] + (start[cg + 1] - start[cg]) - 1 (start: prefix
+// sums).  XMask: per plane a bit for each group of nx / 32 columns that some
+// run meets.
+struct YRuns {
+  int n;
+  unsigned char first[256];
+  unsigned short start[257];
+};
+struct XMask {
+  unsigned m[256];
+};
+// y_planes_ok: ny = 512, 1024 or 2048 and nx a multiple of 16 (up to 4096).
+// launch_y_planes: the y-FFT of nfields x ns planes at p (ns < nz), storing
+// each pixel only in the planes of its two bins; tmap: a tensor map over the
+// planes as [nfields ns][ny][2 nx] floats with (16384 / ny) x 256 x 1 boxes;
+// tw: W512^j (512 rows) or W1024^(n1 k2) as [32][32]; twy: W2048^j (2048
+// rows); b0idx as launch_geometry packs it.  One persistent CTA per SM.
+// launch_x_planes: the x-FFT of their rows, nx = 512, 1024 or 2048 (tw:
+// W512^j, the [32][32] table, or that and W2048^n), storing only the column
+// groups of mask.
+bool y_planes_ok(int nx, int ny);
+cudaError_t launch_y_planes(const void* tmap, void* p, int nx, int ny, int nz, int kb, int ns,
+                            long long nfields, const YRuns& runs, const unsigned short* b0idx,
+                            const void* tw, const void* twy, int* err, int n_sm, unsigned poll,
+                            cudaStream_t s);
+cudaError_t launch_x_planes(void* data, int nx, int ny, int ns, long long nfields,
+                            const XMask& mask, const void* tw, cudaStream_t s);
 template <typename R>
 cudaError_t launch_plane_images(const void* planes, int nx, int ny, int nz, int kb, int ns,
                                 const Geo<R>* geo, const ImageDc<R>& dc, void* imgs,

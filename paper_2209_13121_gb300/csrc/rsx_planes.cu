@@ -10,6 +10,8 @@
 //                   the detector image, for every angle of the batch.
 // The rotation and average follow as on the other paths.  The 3-D DFT is
 // separable, so the values are the full transform's up to rounding order.
+#include <cuda.h>  // CUtensorMap (the type only)
+
 #include "rsx_device.cuh"
 #include "rsx_kernels.h"
 #include "rsx_pol.cuh"
@@ -30,7 +32,12 @@ constexpr int kPlThreads = 256, kPlSlots = 2, kPlPairs = kPlThreads * kPlSlots;
 // D = p(z) - p(nz - z),
 //   X(k) = sum_{z = 0}^{nz/2} cos(t) S - i sin(t) D,  t = 2 pi k z / nz
 // (z = 0 and, for even nz, z = nz/2 stand alone with D = 0), which halves the
-// multiplies: 2 ns fused multiply-adds per voxel and field.  At the kept
+// multiplies: 2 ns fused multiply-adds per voxel and field.  p(0) is taken off
+// the whole column first and nz p(0) returned to bin 0 (the other bins of a
+// constant are 0): summed as it stands, a column's mean would leave its
+// rounding in every bin, where the first stages of an FFT cancel it (one
+// material, 45 x 40 x 40, unrotated image against 64 bits away from q = 0:
+// 3.9e-6 with it, 2.1e-6 without; transforming every slice first 1.4e-6).  At the kept
 // fraction of the bins (ns / nz ~ 0.28 at 5 nm and 300 eV) that is 14 per
 // voxel and field at nz = 16 and 28 at nz = 45, against ~10 to 25 for an FFT
 // that would need a plan for every nz.
@@ -172,8 +179,12 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
       for (int i = 0; i < SB; ++i) x[i] = RT<R>::mk(R(0), R(0));
       const F* b = buf + ((size_t)a * H1 * 3 + f) * PX + px;
       const C* w = tw + g * SBP;
-      for (int z = 0; z < H1; ++z) {
-        const F v = b[z * 3 * PX];
+      const C p0 = b[0].s;  // taken off the column: its bin 0 gets nz p0 back
+      for (int z = 1; z < H1; ++z) {
+        F v = b[z * 3 * PX];
+        const R n = 2 * z == nz ? R(1) : R(2);
+        v.s.x = fma(-n, p0.x, v.s.x);
+        v.s.y = fma(-n, p0.y, v.s.y);
         C wv[SBP];
 #pragma unroll
         for (int i = 0; i < SBP; ++i) wv[i] = w[z * NSP + i];
@@ -184,9 +195,15 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
         }
       }
       C* o = out + (size_t)(a0 + a) * kstride + (size_t)f * fstride + pix0 + px;
+      const int zero = (kb == 0 ? 0 : nz - kb) - g * SB;  // the group's place of bin 0
 #pragma unroll
-      for (int i = 0; i < SB; ++i)
+      for (int i = 0; i < SB; ++i) {
+        if (i == zero) {
+          x[i].x = fma(R(nz), p0.x, x[i].x);
+          x[i].y = fma(R(nz), p0.y, x[i].y);
+        }
         if (g * SB + i < ns) o[(size_t)(g * SB + i) * npix] = x[i];
+      }
     }
   }
 }
@@ -238,6 +255,365 @@ __global__ void __launch_bounds__(256) k_plane_images(const typename RT<R>::C* _
       val = ewald_value<R>(g, v0, v1);
     }
     dst[(size_t)a * npix] = val;
+  }
+}
+
+// --------------------------------------------------- y pass of the planes
+// In-place y-FFT of the kept planes (FP32, ny = 512, 1024 or 2048, nx a
+// multiple of 16) that stores only what the image reads: a pixel's value in a
+// plane is kept when that plane is one of the pixel's two bins.
+//
+// The planes a column meets: the bins of its pixels run from the one at the
+// largest |q_y| up to the one at q_y = 0, so a 16-column group needs one run
+// of planes (YRuns, bounds from the host).  Summed over the groups that is
+// ~52 % of the planes (1024 x 1024 x 128 at 5 nm and 270 eV); the rest is
+// never read here.
+//
+// A step is one (angle, field, 16-column group, plane): TPG = ny / 512 tiles
+// of 8192 elements (a group's 128-byte lines are read by one block, tile
+// after tile).  The steps are cut into one contiguous range per persistent
+// block of two 256-thread groups; thread group g takes the block's tiles
+// i = g, g + 2, ...  Three tile buffers rotate: while two tiles are
+// transformed the next is in flight.  A tile arrives by tensor copies; each
+// thread holds 32 of its elements in registers, transforms them, and the
+// tile is transposed through the buffer it came in (three 256-thread barriers
+// a tile; one shared write and two reads per element, where the
+// split-halves form this replaces took three and four).
+//   ny = 1024 = 32 x 32: 8 columns; thread (n1, col) does the 32-point DFT over n2
+//       (n = n1 + 32 n2), W1024^(n1 k2), then thread (k2, col) the one over
+//       n1: rows k2 + 32 k1.
+//   ny = 2048: 4 columns; threads 0-127 the even outputs, 128-255 the odd
+//       ones (a radix-2 decimation in frequency as the tile is read:
+//       a = x[n] + x[n + 1024], b = (x[n] - x[n + 1024]) W2048^n), each a
+//       1024-point transform as above: rows 2 (k2 + 32 k1) + odd.
+//   ny = 512 = 16 x 32: 16 columns; thread (n1, col) does the 32-point DFT
+//       over n2 (n = n1 + 16 n2), W512^(n1 k2), then two 16-point DFTs, k2
+//       and k2 + 16: rows k2 + 32 k1.
+// A thread's pixels' plane indices are packed as bytes in registers, loaded
+// when the column group changes.  Waits are bounded; on a timeout the block
+// sets *err and its abort flag, both groups leave their loops, and thread 0
+// waits (bounded) for the copies in flight.
+template <int NY> struct YTile {
+  static constexpr int TX = 8192 / NY, TPG = 16 / TX;
+  static constexpr int BUF = NY == 512 ? 8192 : 8448;  // elements: the tile, or its padded transpose
+  static constexpr int NTW = NY == 2048 ? 1024 + 1024 : NY;
+  static constexpr int NQ = NY == 2048 ? 2 : 1;  // tiles of a step one thread group sees
+};
+constexpr int kYBufs = 3;
+
+// v[n] *= tw[n * stride] for n = 1..31
+template <int STRIDE>
+__device__ __forceinline__ void tw_rows(float2* v, const float2* tw) {
+#pragma unroll
+  for (int n = 1; n < 32; ++n) v[n] = cmul(v[n], tw[n * STRIDE]);
+}
+
+template <int NY>
+__global__ void __launch_bounds__(512, 1) k_y_planes(
+    const __grid_constant__ CUtensorMap tmap, const __grid_constant__ YRuns runs, int nx, int nz,
+    int kb, int ns, int L, int T, const unsigned short* __restrict__ b0idx,
+    const float2* __restrict__ tw_g, const float2* __restrict__ twy_g, float2* __restrict__ p,
+    int* __restrict__ err, unsigned poll) {
+  using C = float2;
+  using Y = YTile<NY>;
+  constexpr int TX = Y::TX, TPG = Y::TPG, BUF = Y::BUF, NQ = Y::NQ;
+  constexpr unsigned kPoll = 1u << 22;
+  extern __shared__ __align__(128) unsigned char smem_a128[];
+  C* bufs = reinterpret_cast<C*>(smem_a128);  // [kYBufs][BUF]
+  C* tw = bufs + kYBufs * BUF;                 // [NTW]
+  unsigned long long* bar = reinterpret_cast<unsigned long long*>(tw + Y::NTW);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar + kYBufs);
+  volatile int* issued = abort_flag + 1;  // [kYBufs] loads issued into each buffer
+  const int t = threadIdx.x & 255, g = threadIdx.x >> 8;
+  const int s0 = (int)blockIdx.x * L;
+  const int s1 = s0 + L < T ? s0 + L : T;
+  if (s0 >= s1) return;
+  const int ntile = (s1 - s0) * TPG;
+  const int S = runs.start[runs.n];
+  const size_t npix = (size_t)NY * nx;
+
+  // step -> (angle and field af, column group cg, plane z); next() advances
+  struct Step {
+    int af, cg, z;
+  };
+  auto locate = [&](int st) {
+    Step q;
+    q.af = st / S;
+    const int r = st - q.af * S;
+    int lo = 0, hi = runs.n - 1;  // the last group with start <= r that has steps
+    while (lo < hi) {
+      const int m = (lo + hi + 1) >> 1;
+      if (runs.start[m] <= r) lo = m;
+      else hi = m - 1;
+    }
+    q.cg = lo;
+    q.z = runs.first[lo] + (r - runs.start[lo]);
+    return q;
+  };
+  auto next = [&](Step& q) {
+    if (q.z - runs.first[q.cg] + 1 < runs.start[q.cg + 1] - runs.start[q.cg]) {
+      ++q.z;
+      return;
+    }
+    do {
+      if (++q.cg == runs.n) q.cg = 0, ++q.af;
+    } while (runs.start[q.cg + 1] == runs.start[q.cg]);
+    q.z = runs.first[q.cg];
+  };
+  auto issue = [&](const Step& q, int i) {  // tile i of the block (one thread)
+    const int b = i % kYBufs, x = q.cg * 32 + (i % TPG) * (2 * TX);
+    mbar_expect_tx(&bar[b], 8192 * sizeof(C));
+#pragma unroll
+    for (int k = 0; k < NY / 256; ++k)
+      tma_load_3d(bufs + b * BUF + k * 256 * TX, &tmap, x, k * 256, q.af * ns + q.z, &bar[b]);
+    __threadfence_block();  // the count follows the barrier's arrival
+    issued[b] = issued[b] + 1;
+  };
+
+  if (threadIdx.x == 0) {
+    for (int b = 0; b < kYBufs; ++b) {
+      mbar_init(&bar[b], 1);
+      issued[b] = 0;
+    }
+    *abort_flag = 0;
+    fence_proxy_async();
+  }
+  // W1024^(n1 k2) as [32][32] (1024 and 2048 rows; then W2048^n, n < 1024), or W512^j
+  for (int i = threadIdx.x; i < (NY == 512 ? 512 : 1024); i += 512) tw[i] = tw_g[i];
+  if constexpr (NY == 2048)
+    for (int i = threadIdx.x; i < 1024; i += 512) tw[1024 + i] = twy_g[i];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    Step q = locate(s0);
+    for (int i = 0; i < kYBufs && i < ntile; ++i) {
+      issue(q, i);
+      if ((i + 1) % TPG == 0 && i + 1 < ntile) next(q);
+    }
+  }
+
+  // this thread's place: c its column; stage 1 line n1, stage 2 line k2
+  const int c = t & (TX - 1), hi = t / TX;
+  const int odd = NY == 2048 ? hi >> 5 : 0;    // warp-uniform
+  const int ln = NY == 2048 ? hi & 31 : hi;    // n1 in stage 1, k2 in stage 2
+  Step q = locate(s0), ahead = q;  // this group's tile; the tile kYBufs later (thread t = 0)
+  int qi = 0, ai = 0;              // their step numbers, relative to s0
+  int last_af = -1, last_cg = -1;
+  uint4 sb[NQ][2];  // plane indices of this thread's 32 pixels, as bytes
+  for (int i = g; i < ntile; i += 2) {
+    while (qi < i / TPG) next(q), ++qi;
+    const int b = i % kYBufs, x0 = q.cg * 16 + (i % TPG) * TX;
+    if (q.cg != last_cg || q.af != last_af) {
+      last_cg = q.cg;
+      last_af = q.af;
+#pragma unroll
+      for (int h = 0; h < NQ; ++h) {
+        // 2048 rows: the group's tiles are quarters g (h = 0) and g + 2
+        const int col = NY == 2048 ? q.cg * 16 + (g + 2 * h) * TX + c : x0 + c;
+        unsigned w[8];
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+          const int row = NY == 512 ? (k & 15) * 32 + ln + (k >> 4) * 16
+                          : NY == 2048 ? 2 * (ln + 32 * k) + odd
+                                       : ln + 32 * k;
+          int d = (int)b0idx[(size_t)row * nx + col] - kb;
+          if (d < 0) d += nz;
+          w[k >> 2] = (k & 3) ? w[k >> 2] | (unsigned)d << (8 * (k & 3)) : (unsigned)d;
+        }
+        sb[h][0] = make_uint4(w[0], w[1], w[2], w[3]);
+        sb[h][1] = make_uint4(w[4], w[5], w[6], w[7]);
+      }
+    }
+    // The other thread group issues this tile once it has read tile
+    // i - kYBufs from the same buffer; until then the barrier may still be in
+    // that tile's phase, where this tile's parity would read as complete.
+    bool ok = false;
+    for (unsigned n = 0; n < poll; ++n) {
+      if (issued[b] > i / kYBufs &&
+          (ok = mbar_try_wait(&bar[b], (unsigned)((i / kYBufs) & 1))))
+        break;
+      if (*abort_flag) break;
+    }
+    C* const in = bufs + b * BUF;
+    C v[32];
+    if (ok) {
+      if constexpr (NY == 2048) {
+#pragma unroll
+        for (int n2 = 0; n2 < 32; ++n2) {
+          const int n = ln + 32 * n2;
+          const C x1 = in[n * TX + c], x2 = in[(n + 1024) * TX + c];
+          v[n2] = odd ? cmul(csub(x1, x2), tw[1024 + n]) : cadd(x1, x2);
+        }
+      } else {
+#pragma unroll
+        for (int n2 = 0; n2 < 32; ++n2) v[n2] = in[(ln + (NY / 32) * n2) * TX + c];
+      }
+    }
+    if (named_bar_or(1 + g, 256, !ok)) {  // the tile has been read (or not all of it came)
+      if (t == 0) {
+        atomicOr(err, 1);
+        *abort_flag = 1;
+      }
+      break;
+    }
+    dft32(v);
+    if constexpr (NY == 512) {
+#pragma unroll
+      for (int k2 = 1; k2 < 32; ++k2) v[k2] = cmul(v[k2], tw[ln * k2]);
+#pragma unroll
+      for (int k2 = 0; k2 < 32; ++k2) in[k2 * 256 + t] = v[k2];  // t = n1 16 + c
+    } else {
+      tw_rows<32>(v, tw + ln);
+      C* tr = in + (NY == 2048 ? odd * 32 * 33 * TX : 0) + ln * TX + c;
+#pragma unroll
+      for (int k2 = 0; k2 < 32; ++k2) tr[k2 * 33 * TX] = v[k2];
+    }
+    named_bar_sync(1 + g, 256);
+    if constexpr (NY == 512) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int n1 = 0; n1 < 16; ++n1) v[16 * h + n1] = in[(ln + 16 * h) * 256 + n1 * 16 + c];
+    } else {
+      const C* tr = in + (NY == 2048 ? odd * 32 * 33 * TX : 0) + ln * 33 * TX + c;
+#pragma unroll
+      for (int n1 = 0; n1 < 32; ++n1) v[n1] = tr[n1 * TX];
+    }
+    named_bar_sync(1 + g, 256);  // the buffer is free
+    if (t == 0 && i + kYBufs < ntile) {
+      while (ai < (i + kYBufs) / TPG) next(ahead), ++ai;
+      fence_proxy_async();
+      issue(ahead, i + kYBufs);
+    }
+    if constexpr (NY == 512) {
+      dft_reg<16>(v);
+      dft_reg<16>(v + 16);
+    } else {
+      dft32(v);
+    }
+    C* o = p + ((size_t)q.af * ns + q.z) * npix + x0 + c;
+    const uint4 sa = NQ == 2 && (i % TPG) >= 2 ? sb[NQ - 1][0] : sb[0][0];
+    const uint4 sc = NQ == 2 && (i % TPG) >= 2 ? sb[NQ - 1][1] : sb[0][1];
+    const unsigned w[8] = {sa.x, sa.y, sa.z, sa.w, sc.x, sc.y, sc.z, sc.w};
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+      const int d = q.z - (int)((w[k >> 2] >> (8 * (k & 3))) & 0xffu);
+      if ((unsigned)d <= 1u) {
+        const int row = NY == 512 ? (k & 15) * 32 + ln + (k >> 4) * 16
+                        : NY == 2048 ? 2 * (ln + 32 * k) + odd
+                                     : ln + 32 * k;
+        o[(size_t)row * nx] = NY == 512 ? v[(k & 16) + out_pos<16>(k & 15)] : v[k];
+      }
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && *abort_flag)
+    for (int b = 0; b < kYBufs; ++b)
+      if (issued[b] > 0) mbar_wait_bounded(&bar[b], (unsigned)((issued[b] - 1) & 1), kPoll);
+}
+
+// --------------------------------------------------- x pass of the planes
+// x-FFT of the planes' rows in place (FP32, nx = NX = 512, 1024 or 2048), one
+// warp per row, storing only the column groups (NX / 32 columns each) that
+// the y pass reads from the row's plane (mask.m[plane], a bit per group;
+// ~53 % of them at 1024 x 1024 x 128, 5 nm, 270 eV).  HBM-bound: the row goes to
+// shared memory by asynchronous 16-byte copies (a lane keeps all NX / 64 of
+// its copies in flight, no registers held), issued before the twiddle
+// table's loads so that the two overlap.
+//   NX = 1024: four-step 32 x 32 in registers with one padded transpose; 512:
+//   16 x 32, the 32-point half split over lane pairs; 2048: a radix-2
+//   decimation in frequency as the row is read, then two 1024-point
+//   transforms, kept in registers (64 complex a lane) so that the even and
+//   odd outputs leave as one 16-byte store.
+// tw_g: W512^j; W1024^(n1 k2) as [32][32]; for 2048 that, then W2048^n, n < 1024.
+template <int NX> struct XRow {
+  static constexpr int FS = NX == 2048 ? 2 * 1056 : (NX / 32) * 33;
+  static constexpr int NTW = NX;
+  static constexpr int W = NX == 2048 ? 4 : 8;  // warps per block, two blocks per SM
+};
+
+// The first half of a 1024-point transform up to and including the
+// transpose: v[n2] in, the second stage's inputs out.
+__device__ __forceinline__ void fft1024_half(float2* v, float2* F, const float2* tw4, int lane) {
+  dft32(v);
+  tw_rows<32>(v, tw4 + lane);
+  __syncwarp();
+#pragma unroll
+  for (int k2 = 0; k2 < 32; ++k2) F[k2 * 33 + lane] = v[k2];
+  __syncwarp();
+#pragma unroll
+  for (int n1 = 0; n1 < 32; ++n1) v[n1] = F[lane * 33 + n1];
+}
+
+template <int NX>
+__global__ void __launch_bounds__(32 * XRow<NX>::W, 2) k_x_planes(
+    float2* __restrict__ data, long long nrows, int ny, int ns, const __grid_constant__ XMask mask,
+    const float2* __restrict__ tw_g) {
+  using C = float2;
+  constexpr int FS = XRow<NX>::FS, NTW = XRow<NX>::NTW, W = XRow<NX>::W;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* tw = reinterpret_cast<C*>(smem_raw);
+  C* F = tw + NTW + (threadIdx.x >> 5) * FS;
+  const int lane = threadIdx.x & 31;
+  const long long row = (long long)blockIdx.x * W + (threadIdx.x >> 5);
+  const unsigned m = row < nrows ? mask.m[(int)((row / ny) % ns)] : 0u;
+  C* r = data + (size_t)row * NX;
+  if (m) {
+#pragma unroll
+    for (int j = 0; j < NX / 64; ++j) {
+      const int n = 2 * (lane + 32 * j);
+      cp_async_pair(F + (NX == 2048 && n >= 1024 ? n + 32 : n), r + n);
+    }
+  }
+  for (int i = threadIdx.x; i < NTW; i += 32 * W) tw[i] = tw_g[i];
+  __syncthreads();
+  if (!m) return;
+  cp_async_wait_all();
+  __syncwarp();
+  C v[32];
+  if constexpr (NX == 1024) {
+#pragma unroll
+    for (int n2 = 0; n2 < 32; ++n2) v[n2] = F[lane + 32 * n2];
+    fft1024_half(v, F, tw, lane);
+    dft32(v);
+#pragma unroll
+    for (int k1 = 0; k1 < 32; ++k1)
+      if (m >> k1 & 1u) r[lane + 32 * k1] = v[k1];
+  } else if constexpr (NX == 2048) {
+    C u[32];
+#pragma unroll
+    for (int n2 = 0; n2 < 32; ++n2) {
+      const int n = lane + 32 * n2;
+      const C a = F[n], b = F[1056 + n];
+      v[n2] = cadd(a, b);
+      u[n2] = cmul(csub(a, b), tw[1024 + n]);
+    }
+    fft1024_half(v, F, tw, lane);
+    fft1024_half(u, F + 1056, tw, lane);
+    dft32(v);
+    dft32(u);
+#pragma unroll
+    for (int k1 = 0; k1 < 32; ++k1)
+      if (m >> k1 & 1u)
+        reinterpret_cast<float4*>(r)[lane + 32 * k1] = make_float4(v[k1].x, v[k1].y, u[k1].x, u[k1].y);
+  } else {
+#pragma unroll
+    for (int n2 = 0; n2 < 16; ++n2) v[n2] = F[lane + 32 * n2];
+    dft_reg<16>(v);
+    C u[16];
+#pragma unroll
+    for (int k2 = 0; k2 < 16; ++k2) u[k2] = cmul(v[out_pos<16>(k2)], tw[lane * k2]);
+    __syncwarp();
+#pragma unroll
+    for (int k2 = 0; k2 < 16; ++k2) F[k2 * 33 + lane] = u[k2];
+    __syncwarp();
+    const int k2 = lane & 15, h = lane >> 4;
+#pragma unroll
+    for (int n = 0; n < 16; ++n) v[n] = F[k2 * 33 + 2 * n + h];
+    dft32_pair(v, u, h);
+    const unsigned mh = m >> (16 * h);
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      if (mh >> k & 1u) r[k2 + 256 * h + 16 * k] = u[k];
   }
 }
 
@@ -326,6 +702,78 @@ cudaError_t launch_plane_images(const void* planes, int nx, int ny, int nz, int 
     k_plane_images<R, 1><<<dim3(gx, dc.n), 256, 0, s>>>((const C*)planes, nx, ny, nz, kb, ns, geo,
                                                         dc, (R*)imgs);
   return cudaGetLastError();
+}
+
+bool y_planes_ok(int nx, int ny) {
+  return (ny == 512 || ny == 1024 || ny == 2048) && nx >= 16 && nx <= 4096 && nx % 16 == 0;
+}
+
+template <int NY>
+static cudaError_t y_planes_impl(const void* tmap, void* p, int nx, int nz, int kb, int ns,
+                                 long long nfields, const YRuns& runs,
+                                 const unsigned short* b0idx, const void* tw, const void* twy,
+                                 int* err, int n_sm, unsigned poll, cudaStream_t s) {
+  using Y = YTile<NY>;
+  const long long T = nfields * runs.start[runs.n];
+  if (T <= 0) return cudaSuccess;
+  if (n_sm <= 0 || T > (1 << 30) || (NY == 2048 && !twy) || !tw || !b0idx)
+    return cudaErrorInvalidValue;
+  const long long L = (T + n_sm - 1) / n_sm;
+  const size_t smem = (size_t)(kYBufs * Y::BUF + Y::NTW) * sizeof(float2) + kYBufs * 8 +
+                      (1 + kYBufs) * sizeof(int);
+  auto kern = k_y_planes<NY>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<(unsigned)((T + L - 1) / L), 512, smem, s>>>(
+      *(const CUtensorMap*)tmap, runs, nx, nz, kb, ns, (int)L, (int)T, b0idx, (const float2*)tw,
+      (const float2*)twy, (float2*)p, err, poll);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_y_planes(const void* tmap, void* p, int nx, int ny, int nz, int kb, int ns,
+                            long long nfields, const YRuns& runs, const unsigned short* b0idx,
+                            const void* tw, const void* twy, int* err, int n_sm, unsigned poll,
+                            cudaStream_t s) {
+  if (!y_planes_ok(nx, ny) || ns < 1 || ns >= nz || nz > kMaxPlanesNz || kb < 0 || kb >= nz ||
+      runs.n != nx / 16)
+    return cudaErrorInvalidValue;
+  for (int i = 0; i < runs.n; ++i)
+    if (runs.start[i + 1] < runs.start[i] ||
+        runs.first[i] + (runs.start[i + 1] - runs.start[i]) > ns)
+      return cudaErrorInvalidValue;
+  if (ny == 512)
+    return y_planes_impl<512>(tmap, p, nx, nz, kb, ns, nfields, runs, b0idx, tw, twy, err, n_sm,
+                              poll, s);
+  if (ny == 1024)
+    return y_planes_impl<1024>(tmap, p, nx, nz, kb, ns, nfields, runs, b0idx, tw, twy, err, n_sm,
+                               poll, s);
+  return y_planes_impl<2048>(tmap, p, nx, nz, kb, ns, nfields, runs, b0idx, tw, twy, err, n_sm,
+                             poll, s);
+}
+
+template <int NX>
+static cudaError_t x_planes_impl(void* data, long long nrows, int ny, int ns, const XMask& mask,
+                                 const void* tw, cudaStream_t s) {
+  using X = XRow<NX>;
+  const size_t smem = ((size_t)X::NTW + (size_t)X::W * X::FS) * sizeof(float2);
+  auto kern = k_x_planes<NX>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<(unsigned)((nrows + X::W - 1) / X::W), 32 * X::W, smem, s>>>(
+      (float2*)data, nrows, ny, ns, mask, (const float2*)tw);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_x_planes(void* data, int nx, int ny, int ns, long long nfields,
+                            const XMask& mask, const void* tw, cudaStream_t s) {
+  const long long nrows = nfields * ns * ny;
+  if (nrows <= 0) return cudaSuccess;
+  // 16-byte row copies
+  if (!tw || ((uintptr_t)data & 15) || ns < 1 || ns > kMaxPlanesNz) return cudaErrorInvalidValue;
+  if (nx == 1024) return x_planes_impl<1024>(data, nrows, ny, ns, mask, tw, s);
+  if (nx == 2048) return x_planes_impl<2048>(data, nrows, ny, ns, mask, tw, s);
+  if (nx == 512) return x_planes_impl<512>(data, nrows, ny, ns, mask, tw, s);
+  return cudaErrorInvalidValue;
 }
 
 #define RSX_INST(R)                                                                               \

@@ -83,3 +83,25 @@ def test_more_angles_than_one_batch_holds(rsx):
         ctx.set_morphology(M)
         ctx.set_optical_constants(E, K)
         _close(ctx.run((0.0, 1.0, 180.0)), ref, 32)
+
+
+@pytest.mark.parametrize("shape", [(16, 512, 32), (16, 1024, 32), (16, 2048, 16)],
+                         ids=["512", "1024", "2048"])
+def test_y_pass_timeout_is_reported_and_recoverable(rsx, shape):
+    """With a wait bound of zero polls the y pass of the planes gives up
+    cleanly: the run reports it, leaves its host output alone, and with the
+    default bound restored gives a fresh context's result bit for bit."""
+    nz, ny, nx = shape
+    M = torch.from_numpy(synth.morphology_random(shape, 2, seed=15, dtype=np.float32)).cuda()
+    K = synth.optical_constants([285.0], 2, seed=16)
+    with rsx.Context(nx, ny, nz, 2, 5.0) as ctx:
+        ctx.set_morphology(M)
+        ctx.set_optical_constants([285.0], K)
+        ref = ctx.run((0.0, 30.0, 150.0))
+        out = np.full((1, ny, nx), 7.0, dtype=np.float32)
+        ctx.set_wait_limit(0)
+        with pytest.raises(rsx.RsxError) as e:
+            ctx.run((0.0, 30.0, 150.0), out=out)
+        assert e.value.code == rsx.RSX_ERR_CUDA and np.all(out == 7.0)
+        ctx.set_wait_limit()
+        np.testing.assert_array_equal(ctx.run((0.0, 30.0, 150.0)), ref)
