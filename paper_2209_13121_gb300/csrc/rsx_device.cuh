@@ -274,6 +274,63 @@ template <typename C> __host__ __device__ __forceinline__ void dft32(C* v) {
   dft32_combine<0>(v, e, o);
 }
 
+// acc + a * exp(-2 pi i E / 32) for a compile-time E: four fused
+// multiply-adds, or two additions where the factor is a power of -i.
+template <int E, typename C> __host__ __device__ __forceinline__ C cadd_w32(C acc, C a) {
+  using R = decltype(a.x);
+  constexpr int e = E & 31;
+  if constexpr (e == 0) return cadd(acc, a);
+  else if constexpr (e == 8) return cadd(acc, cmul_mi(a));
+  else if constexpr (e == 16) return csub(acc, a);
+  else if constexpr (e == 24) return csub(acc, cmul_mi(a));
+  else {
+    constexpr double q[9] = {1.0, 0.98078528040323044913, 0.92387953251128675613,
+                             0.83146961230254523708, 0.70710678118654752440,
+                             0.55557023301960222474, 0.38268343236508977173,
+                             0.19509032201612826785, 0.0};  // cos(pi j / 16)
+    constexpr int m = e & 15;
+    constexpr double sg = e < 16 ? 1.0 : -1.0;
+    constexpr double cs = sg * (m <= 8 ? q[m] : -q[16 - m]);
+    constexpr double sn = sg * (m <= 8 ? q[8 - m] : q[m - 8]);
+    acc.x = acc.x + a.x * R(cs) + a.y * R(sn);
+    acc.y = acc.y + a.y * R(cs) - a.x * R(sn);
+    return acc;
+  }
+}
+
+// The first outputs of a 32-point forward DFT of v, in order, each passed to
+// out(K, X[K]) for K = 0, 1, ... while K < count (count <= 16).  With
+// n = n1 + 4 m: four 8-point DFTs over m, then each output on its own,
+//   X[a + 8 b] = sum_n1 W32^(n1 (a + 8 b)) Y_n1[a],
+// 12 fused multiply-adds per output: cheaper than the whole transform
+// (~440 operations) up to 16 outputs (224 + 12 each).
+template <int K, typename C, typename Out>
+__device__ __forceinline__ void dft32_first_step(const C* v, int count, Out& out) {
+  if constexpr (K < 16) {
+    if (K >= count) return;  // uniform
+    constexpr int a = 4 * out_pos<8>(K & 7);
+    C x = v[a];
+    x = cadd_w32<K>(x, v[a + 1]);
+    x = cadd_w32<2 * K>(x, v[a + 2]);
+    x = cadd_w32<3 * K>(x, v[a + 3]);
+    out(K, x);
+    dft32_first_step<K + 1>(v, count, out);
+  }
+}
+template <typename C, typename Out>
+__device__ __forceinline__ void dft32_first(C* v, int count, Out out) {
+#pragma unroll
+  for (int n1 = 0; n1 < 4; ++n1) {
+    C y[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) y[m] = v[n1 + 4 * m];
+    dft_reg<8>(y);
+#pragma unroll
+    for (int m = 0; m < 8; ++m) v[n1 + 4 * m] = y[m];
+  }
+  dft32_first_step<0>(v, count, out);
+}
+
 // v[out_pos<16>(K)] *= W32^K for K = 0..15: the odd half of a 32-point DFT
 // after its 16-point DFT (compile-time twiddles).
 template <int K, typename C> __device__ __forceinline__ void w32_outputs(C* v) {
