@@ -101,7 +101,8 @@ typedef struct rsx_context rsx_context;
  * ny = 2048), the two q_z bins per
  * pixel of the fused y-FFT + z pass (up to 4 partial slots of 3 x 2 x 16
  * bytes per pixel; 5 x 2 x 16 for Algorithm 3).  For Algorithms 1 and 2 with
- * nz <= 255 the p workspace is at least the lesser of 32 angles' p and 96 MB,
+ * nz <= 255 the p workspace is at least the lesser of 32 angles' p and 96 MB
+ * (FP64: 1 GB),
  * and a batch of images (at most 64, 64 MB or one) is held.  *out
  * receives the handle.  Errors: RSX_ERR_INVALID (sizes, precision,
  * algorithm), RSX_ERR_OOM. */

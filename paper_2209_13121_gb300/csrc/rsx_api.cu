@@ -764,7 +764,8 @@ static bool planes_cfg(const rsx_config* cfg) {
 static long long p_elems(const rsx_config* cfg) {
   const long long one = 3LL * cfg->nx * cfg->ny * cfg->nz, base = one * angle_batch_of(cfg);
   if (!planes_cfg(cfg)) return base;
-  const long long pool = (96LL << 20) / (long long)complex_size(cfg->precision);
+  const long long pool = ((cfg->precision == 32 ? 96LL : 1024LL) << 20) /
+                         (long long)complex_size(cfg->precision);
   const long long want = 32 * one < pool ? 32 * one : pool;
   return want > base ? want : base;
 }
@@ -818,7 +819,7 @@ static bool planes_plan(const rsx_context* c, int ie, ZPlan* zp) {
   zp->zfft = g.precision == 32 && g.algorithm == 1 && (g.nz == 32 || g.nz == 64 || g.nz == 128) &&
              g.nx % (1024 / g.nz) == 0 && c->n_sm > 0 && ((uintptr_t)c->M & 15) == 0 &&
              c->npix * g.nz >= 2048LL * c->n_sm;
-  if (!zp->zfft && !rsx::pol_planes_fits(g.precision, g.nz, zp->ns)) return false;
+  if (!zp->zfft && !rsx::pol_planes_fits(g.precision, g.nz, zp->kb, zp->ns)) return false;
   const long long kz = c->p_cap / (3LL * zp->ns * c->npix);
   const int cap = zp->zfft ? rsx::kMaxXAngles : rsx::kMaxAngleBatch;
   zp->kz = kz < cap ? (int)kz : cap;

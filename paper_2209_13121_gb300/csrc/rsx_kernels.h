@@ -311,7 +311,7 @@ template <typename R> struct ImageDc {
   int n;
   R x[kMaxAngleBatch], y[kMaxAngleBatch];
 };
-bool pol_planes_fits(int precision, int nz, int ns);
+bool pol_planes_fits(int precision, int nz, int kb, int ns);
 template <typename R>
 cudaError_t launch_pol_planes(const void* M, const void* nt, const void* dir, long long npix,
                               int nz, const PolParams<R>& pp, const AngleBatch<R>& ang, void* out,

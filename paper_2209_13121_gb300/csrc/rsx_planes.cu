@@ -19,37 +19,42 @@
 namespace rsx {
 namespace {
 
-// A voxel pair's field after the fold below: sum and difference.
+// A field at a fold's voxels: sum and difference.
 template <typename C> struct Folded {
   C s, d;
 };
 
-constexpr int kPlThreads = 256, kPlSlots = 2, kPlPairs = kPlThreads * kPlSlots;
+constexpr int kPlThreads = 256, kPlVoxels = 4;  // voxels a thread holds
+
+// it / d for it < 2^11 and d <= 512, with magic(d): exact while it d < 2^20
+__host__ __device__ constexpr unsigned magic(unsigned d) { return (1u << 20) / d + 1; }
+__device__ __forceinline__ int div_by(int it, unsigned m) { return (int)(((unsigned)it * m) >> 20); }
 
 // A block owns PX adjacent pixels (flat index y nx + x) by the whole stack.
-// The z transform is evaluated as a sum over the bins that are kept, with the
-// voxels z and nz - z folded first: with S = p(z) + p(nz - z) and
-// D = p(z) - p(nz - z),
-//   X(k) = sum_{z = 0}^{nz/2} cos(t) S - i sin(t) D,  t = 2 pi k z / nz
-// (z = 0 and, for even nz, z = nz/2 stand alone with D = 0), which halves the
-// multiplies: 2 ns fused multiply-adds per voxel and field.  p(0) is taken off
-// the whole column first and nz p(0) returned to bin 0 (the other bins of a
-// constant are 0): summed as it stands, a column's mean would leave its
-// rounding in every bin, where the first stages of an FFT cancel it (one
-// material, 45 x 40 x 40, unrotated image against 64 bits away from q = 0:
-// 3.9e-6 with it, 2.1e-6 without; transforming every slice first 1.4e-6).  At the kept
-// fraction of the bins (ns / nz ~ 0.28 at 5 nm and 300 eV) that is 14 per
-// voxel and field at nz = 16 and 28 at nz = 45, against ~10 to 25 for an FFT
-// that would need a plan for every nz.
-// A thread keeps the sums of its kPlSlots voxel pairs in registers for all
-// angles.  Per step of A angles: every thread forms p of its voxels for each
-// angle and stores S and D (three fields) to shared memory; then the block's
-// threads take (angle, field, group of SB bins, pixel) items, a pixel's
-// S and D read once per SB bins (with SB = 8, 32 fused multiply-adds per
-// 16-byte shared read of S and D and 4 broadcast reads of the twiddles).
+// The z transform is evaluated as a sum over the bins that are kept, the
+// voxels folded first.  Odd nz: with S = p(z) + p(nz - z), D = p(z) - p(nz - z),
+//   X(k) = sum_{z <= nz/2} cos(t) S - i sin(t) D,  t = 2 pi k z / nz
+// (z = 0 alone).  EVEN nz, L = nz / 2: the even bins see a(z) = p(z) +
+// p(z + L) and the odd ones b(z) = p(z) - p(z + L), z < L, each folded once
+// more: S = a(z) + a(L - z), D = a(z) - a(L - z), or S = b(z) - b(L - z),
+// D = b(z) + b(L - z), in the same sum over z <= L/2 (z = 0 and L/2 alone).
+// So a kept bin takes 2 fused multiply-adds per voxel and field for odd nz
+// and 1 for even: ns of them, 7 at nz = 16 and 28 at nz = 45 (5 nm, 270 eV),
+// against ~10 to 25 for an FFT that would need a plan for every nz.  Before
+// the sum its z = 0 term is taken off the even bins' whole column and
+// returned to bin 0 (the other bins of a constant are 0): summed as it
+// stands, a column's mean would leave its rounding in every bin, where the
+// first stages of an FFT cancel it (one material, 45 x 40 x 40, unrotated
+// image against 64 bits away from q = 0: 3.9e-6 with it, 2.1e-6 without;
+// transforming every slice first 1.4e-6).
+// A thread keeps the angle-independent sums of its 4 voxels (one quad, or
+// two pairs) in registers for all angles.  Per step of A angles: every thread
+// forms p of its voxels for each angle and stores the folds (three fields) to
+// shared memory; then the block's threads take (angle, field, group of SB
+// bins of one parity, pixel) items.
 // SRC 0: morphology (dir: FP64's cached director); 1: Algorithm 2's N_t.
 // twt: exp(-2 pi i j / nz), j < nz.
-template <typename R, int SRC, int SB>
+template <typename R, int SRC, int SB, bool EVEN>
 __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_planes(
     const typename RT<R>::V4* __restrict__ M, const typename RT<R>::C* __restrict__ nt,
     const R* __restrict__ dir, long long npix, int nz, int PX, int A, int kb, int ns,
@@ -58,64 +63,66 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
   using C = typename RT<R>::C;
   using F = Folded<C>;
   constexpr int SBP = (SB + 1) & ~1;  // twiddles of a group, padded to pairs
+  constexpr int NP = EVEN ? 2 : 1;    // parities of the bins
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int t = threadIdx.x;
-  const int H1 = nz / 2 + 1, G = (ns + SB - 1) / SB, NSP = G * SBP;
-  F* buf = reinterpret_cast<F*>(smem_raw);        // [A][H1][3][PX]
-  C* tw = reinterpret_cast<C*>(buf + (size_t)A * H1 * 3 * PX);  // [H1][NSP]
+  const int L = EVEN ? nz / 2 : nz, H = L / 2 + 1;  // terms of the folded sum
+  const int odd0 = kb & 1;                          // parity of plane 0's bin
+  const int n0 = EVEN ? (ns + 1 - odd0) / 2 : ns;   // kept bins of parity 0
+  const int G0 = (n0 + SB - 1) / SB, G = G0 + (EVEN ? (ns - n0 + SB - 1) / SB : 0);
+  const int NSP = G * SBP;
+  F* buf = reinterpret_cast<F*>(smem_raw);                        // [A][NP][H][3][PX]
+  C* tw = reinterpret_cast<C*>(buf + (size_t)A * NP * H * 3 * PX);  // [H][NSP]
   const long long N = npix * nz;
   const long long pix0 = (long long)blockIdx.x * PX;
   const int npx = npix - pix0 < PX ? (int)(npix - pix0) : PX;
-  for (int i = t; nz > 1 && i < H1 * NSP; i += kPlThreads) {  // (nz = 1 has no shared memory)
-    const int z = i / NSP, r = i - z * NSP, g = r / SBP, b = g * SB + (r - g * SBP);
+  // bin i of group g: plane first(g) + NP i
+  auto first = [&](int g) {
+    return !EVEN ? g * SB : g < G0 ? odd0 + 2 * g * SB : 1 - odd0 + 2 * (g - G0) * SB;
+  };
+  for (int i = t; nz > 1 && i < H * NSP; i += kPlThreads) {  // (nz = 1 has no shared memory)
+    const int z = i / NSP, r = i - z * NSP, g = r / SBP, b = first(g) + NP * (r - g * SBP);
     tw[i] = twz[(int)(((long long)(kb + b) * z) % nz)];
   }
 
-  // this thread's voxel pairs: the sums of Eq. (polarization), divided by 4 pi
-  TAcc<R> acc[kPlSlots][2];
-  int at[kPlSlots];    // shared-memory place of the pair (field 0, angle 0); -1: none
-  bool two[kPlSlots];  // the pair has a second voxel, nz - z
+  // this thread's voxels: the sums of Eq. (polarization), divided by 4 pi.
+  // EVEN: z, z + L, L - z, nz - z of one pixel; else z, nz - z of two
+  TAcc<R> acc[kPlVoxels];
+  int at[2];     // shared-memory place of each fold (field 0, angle 0); -1: none
+  bool two[2];   // its second half exists (z is not alone)
 #pragma unroll
-  for (int sl = 0; sl < kPlSlots; ++sl) {
-    const int q = t + sl * kPlThreads, z = q / PX, px = q - z * PX;
-    at[sl] = z < H1 && px < npx ? (z * 3) * PX + px : -1;
-    two[sl] = at[sl] >= 0 && z > 0 && 2 * z < nz;
-    tacc_zero(acc[sl][0]);
-    tacc_zero(acc[sl][1]);
-    if (at[sl] < 0) continue;
-    const size_t i0 = (size_t)z * npix + pix0 + px, i1 = (size_t)(nz - z) * npix + pix0 + px;
-    if constexpr (SRC == 1) {
+  for (int sl = 0; sl < 2; ++sl) {
+    const int q = EVEN ? t : t + sl * kPlThreads, z = q / PX, px = q - z * PX;
+    const bool in = z < H && px < npx;
+    at[sl] = in ? z * 3 * PX + px : -1;
+    two[sl] = in && z > 0 && 2 * z != L;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (h && !two[sl]) break;
-        acc[sl][h].aw = R(0);
+    for (int h = 0; h < 2; ++h) {
+      TAcc<R>& a = acc[2 * sl + h];
+      tacc_zero(a);
+      // EVEN: slot 0 holds z and z + L, slot 1 L - z and nz - z
+      const int zv = EVEN ? (sl ? L - z : z) + (h ? L : 0) : h ? nz - z : z;
+      const bool have = EVEN ? (sl ? two[sl] : in) : h ? two[sl] : in;
+      if (!have) continue;
+      const size_t i = (size_t)(EVEN && sl && h ? nz - z : zv) * npix + pix0 + px;
+      if constexpr (SRC == 1) {
 #pragma unroll
         for (int e = 0; e < 5; ++e) {
-          const C v = ld_stream(nt + (size_t)e * N + (h ? i1 : i0));
-          acc[sl][h].t[e][0] = v.x;
-          acc[sl][h].t[e][1] = v.y;
+          const C v = ld_stream(nt + (size_t)e * N + i);
+          a.t[e][0] = v.x;
+          a.t[e][1] = v.y;
         }
-      }
-    } else {
-      for (int j = 0; j < pp.c; ++j) {
-        const typename RT<R>::V4* Mj = M + (size_t)j * N;
-        const typename RT<R>::V4 m0 = ld_stream(Mj + i0);
-        typename RT<R>::V4 m1 = m0;
-        if (two[sl]) m1 = ld_stream(Mj + i1);
-        if (dir) {
-          const R* dj = dir + (size_t)j * 3 * N;
-          tacc_add_d(acc[sl][0], (R)m0.x, (R)m0.y, dj[i0], dj[N + i0], dj[2 * N + i0], pp, j);
-          if (two[sl])
-            tacc_add_d(acc[sl][1], (R)m1.x, (R)m1.y, dj[i1], dj[N + i1], dj[2 * N + i1], pp, j);
-        } else {
-          tacc_add(acc[sl][0], (R)m0.x, (R)m0.y, (R)m0.z, (R)m0.w, pp, j);
-          if (two[sl]) tacc_add(acc[sl][1], (R)m1.x, (R)m1.y, (R)m1.z, (R)m1.w, pp, j);
+      } else {
+        for (int j = 0; j < pp.c; ++j) {
+          const typename RT<R>::V4 m = ld_stream(M + (size_t)j * N + i);
+          if (dir) {
+            const R* dj = dir + (size_t)j * 3 * N + i;
+            tacc_add_d(a, (R)m.x, (R)m.y, dj[0], dj[N], dj[2 * N], pp, j);
+          } else {
+            tacc_add(a, (R)m.x, (R)m.y, (R)m.z, (R)m.w, pp, j);
+          }
         }
-      }
-      const R inv = R(1.0 / kFourPi);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        TAcc<R>& a = acc[sl][h];
+        const R inv = R(1.0 / kFourPi);
         a.aw = ((a.aw - R(1)) + a.as[0]) * inv;
         a.as[1] *= inv;
 #pragma unroll
@@ -132,10 +139,11 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
   if (nz == 1) {  // no z transform: the pixel's p is its plane
     for (int k = 0; k < ang.n; ++k) {
 #pragma unroll
-      for (int sl = 0; sl < kPlSlots; ++sl) {
+      for (int sl = 0; sl < 2; ++sl) {
         if (at[sl] < 0) continue;
         C p[3];
-        p_from_tacc(acc[sl][0].aw, acc[sl][0].as[1], acc[sl][0].t, ang.ce[k], ang.se[k], literal, p);
+        p_from_tacc(acc[2 * sl].aw, acc[2 * sl].as[1], acc[2 * sl].t, ang.ce[k], ang.se[k], literal,
+                    p);
         C* o = out + k * kstride + pix0 + at[sl];
         o[0] = p[0];
         o[fstride] = p[1];
@@ -144,45 +152,70 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
     }
     return;
   }
+  const unsigned mpx = magic(PX), mg = magic(G), m3 = magic(3);
+  const int s_bin0 = kb == 0 ? 0 : nz - kb;  // bin 0's plane
   for (int a0 = 0; a0 < ang.n; a0 += A) {
     const int na = ang.n - a0 < A ? ang.n - a0 : A;
     if (a0 > 0) __syncthreads();  // the previous step's reads are done
     for (int a = 0; a < na; ++a) {
       const R ce = ang.ce[a0 + a], se = ang.se[a0 + a];
-      F* ba = buf + (size_t)a * H1 * 3 * PX;
+      F* ba = buf + (size_t)a * NP * H * 3 * PX;
+      if constexpr (EVEN) {
+        if (at[0] < 0) continue;
+        C p[4][3];
 #pragma unroll
-      for (int sl = 0; sl < kPlSlots; ++sl) {
-        if (at[sl] < 0) continue;
-        C p[3], q[3];
-        p_from_tacc(acc[sl][0].aw, acc[sl][0].as[1], acc[sl][0].t, ce, se, literal, p);
-        p_from_tacc(acc[sl][1].aw, acc[sl][1].as[1], acc[sl][1].t, ce, se, literal, q);
+        for (int v = 0; v < 4; ++v)
+          p_from_tacc(acc[v].aw, acc[v].as[1], acc[v].t, ce, se, literal, p[v]);
 #pragma unroll
-        for (int f = 0; f < 3; ++f) {
+        for (int f = 0; f < 3; ++f) {  // (a voxel that does not exist has p = 0)
+          const C a1 = cadd(p[0][f], p[1][f]), b1 = csub(p[0][f], p[1][f]);
+          const C a2 = cadd(p[2][f], p[3][f]), b2 = csub(p[2][f], p[3][f]);
           F v;
-          v.s = two[sl] ? cadd(p[f], q[f]) : p[f];
-          v.d = two[sl] ? csub(p[f], q[f]) : RT<R>::mk(R(0), R(0));
-          ba[at[sl] + f * PX] = v;
+          v.s = cadd(a1, a2);
+          v.d = csub(a1, a2);
+          ba[at[0] + f * PX] = v;
+          v.s = csub(b1, b2);
+          v.d = cadd(b1, b2);
+          ba[at[0] + (H * 3 + f) * PX] = v;
+        }
+      } else {
+#pragma unroll
+        for (int sl = 0; sl < 2; ++sl) {
+          if (at[sl] < 0) continue;
+          C p[3], q[3];
+          p_from_tacc(acc[2 * sl].aw, acc[2 * sl].as[1], acc[2 * sl].t, ce, se, literal, p);
+          p_from_tacc(acc[2 * sl + 1].aw, acc[2 * sl + 1].as[1], acc[2 * sl + 1].t, ce, se, literal,
+                      q);
+#pragma unroll
+          for (int f = 0; f < 3; ++f) {
+            F v;
+            v.s = cadd(p[f], q[f]);
+            v.d = csub(p[f], q[f]);
+            ba[at[sl] + f * PX] = v;
+          }
         }
       }
     }
     __syncthreads();
     const int items = na * 3 * G * PX;
     for (int it = t; it < items; it += kPlThreads) {
-      int r = it / PX;
+      int r = div_by(it, mpx);
       const int px = it - r * PX;
-      const int g = r % G;
-      r /= G;
-      const int f = r % 3, a = r / 3;
+      int q = div_by(r, mg);
+      const int g = r - q * G, a = div_by(q, m3), f = q - 3 * a;
       if (px >= npx) continue;
+      const int par = EVEN && g >= G0;
+      const F* b = buf + ((size_t)(a * NP + par) * H * 3 + f) * PX + px;
+      const C* w = tw + g * SBP;
+      // z = 0: the even bins' base (see above), the odd bins' first term
+      const C p0 = b[0].s;
       C x[SB];
 #pragma unroll
-      for (int i = 0; i < SB; ++i) x[i] = RT<R>::mk(R(0), R(0));
-      const F* b = buf + ((size_t)a * H1 * 3 + f) * PX + px;
-      const C* w = tw + g * SBP;
-      const C p0 = b[0].s;  // taken off the column: its bin 0 gets nz p0 back
-      for (int z = 1; z < H1; ++z) {
+      for (int i = 0; i < SB; ++i) x[i] = par ? p0 : RT<R>::mk(R(0), R(0));
+      const R once = par ? R(0) : R(1), twice = par ? R(0) : R(2);
+      for (int z = 1; z < H; ++z) {
         F v = b[z * 3 * PX];
-        const R n = 2 * z == nz ? R(1) : R(2);
+        const R n = 2 * z == L ? once : twice;
         v.s.x = fma(-n, p0.x, v.s.x);
         v.s.y = fma(-n, p0.y, v.s.y);
         C wv[SBP];
@@ -194,15 +227,162 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
           x[i].y = fma(wv[i].x, v.s.y, fma(wv[i].y, v.d.x, x[i].y));
         }
       }
-      C* o = out + (size_t)(a0 + a) * kstride + (size_t)f * fstride + pix0 + px;
-      const int zero = (kb == 0 ? 0 : nz - kb) - g * SB;  // the group's place of bin 0
+      const int s0 = first(g);
+      C* o = out + (size_t)(a0 + a) * kstride + (size_t)f * fstride + (size_t)s0 * npix + pix0 + px;
 #pragma unroll
       for (int i = 0; i < SB; ++i) {
-        if (i == zero) {
-          x[i].x = fma(R(nz), p0.x, x[i].x);
-          x[i].y = fma(R(nz), p0.y, x[i].y);
+        if (s0 + NP * i == s_bin0) {
+          x[i].x = fma(R(L), p0.x, x[i].x);
+          x[i].y = fma(R(L), p0.y, x[i].y);
         }
-        if (g * SB + i < ns) o[(size_t)(g * SB + i) * npix] = x[i];
+        if (s0 + NP * i < ns) o[(size_t)(NP * i) * npix] = x[i];
+      }
+    }
+  }
+}
+
+// The same pass for nz = 4 Q, Q = 2, 4, 8, 16 or 32, by a decimation in
+// frequency: z = n2 + Q n1, and plane s = 4 s2 + s1 holds bin kb + s:
+//   X(kb + s) = sum_n2 W_Q^(n2 s2) W_nz^(n2 (kb + s1)) sum_n1 x[n2 + Q n1] W_4^(n1 (kb + s1)).
+// A block owns PX = 256 / Q pixels; thread (n2, pixel) holds the
+// angle-independent sums of its four voxels n1 in registers for all angles.
+// Per step of A angles it forms their p, does the 4-point transform over n1
+// and the twiddles (its own four, in registers) and stores u[s1][n2] of the
+// three fields to shared memory (thread order: contiguous); then the threads
+// take (angle, field, s1, pixel) items: a Q-point transform over n2 in
+// registers, whose first outputs s2 go straight to their planes (Q = 32: only
+// the kept ones are evaluated).  ~75 instructions per voxel and angle at
+// nz = 16, where the folded sums above took 160 at 64 % issue (1024 x 1024 x 16,
+// c = 3, two energies of 91 angles: the pass 19.0 ms, 13.4 so; Algorithm 2 at
+// 1024 x 1024 x 32, 37 angles: 16.5 and 13.2).
+template <typename R, int Q> struct PlFft {
+  static constexpr int PX = kPlThreads / Q;
+  // u's stride between s1: padded where a half-warp spans two of them
+  static constexpr int KS = kPlThreads + (PX * (int)sizeof(typename RT<R>::C) < 128 ? PX : 0);
+  // angles per step: the items (12 PX per angle) fill the block
+  static constexpr int A = sizeof(R) == 8 ? (Q >= 8 ? 2 : 1) : Q >= 16 ? 4 : Q == 8 ? 2 : 1;
+};
+
+template <typename R, int SRC, int Q>
+__global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_planes_fft(
+    const typename RT<R>::V4* __restrict__ M, const typename RT<R>::C* __restrict__ nt,
+    const R* __restrict__ dir, long long npix, int kb, int ns,
+    const __grid_constant__ PolParams<R> pp, const __grid_constant__ AngleBatch<R> ang,
+    typename RT<R>::C* __restrict__ out, const typename RT<R>::C* __restrict__ twz) {
+  using C = typename RT<R>::C;
+  using P = PlFft<R, Q>;
+  constexpr int NZ = 4 * Q, PX = P::PX, KS = P::KS, A = P::A;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* buf = reinterpret_cast<C*>(smem_raw);  // [A][3][4][KS]
+  const int t = threadIdx.x, px = t % PX, n2 = t / PX;
+  const long long N = npix * NZ;
+  const long long pix0 = (long long)blockIdx.x * PX;
+  const int npx = npix - pix0 < PX ? (int)(npix - pix0) : PX;
+  TAcc<R> acc[4];
+  C w[4];
+#pragma unroll
+  for (int n1 = 0; n1 < 4; ++n1) {
+    w[n1] = twz[(n2 * (kb + n1)) % NZ];
+    TAcc<R>& a = acc[n1];
+    tacc_zero(a);
+    const size_t i = (size_t)(n2 + Q * n1) * npix + pix0 + px;
+    if (px < npx) {
+      if constexpr (SRC == 1) {
+#pragma unroll
+        for (int e = 0; e < 5; ++e) {
+          const C v = ld_stream(nt + (size_t)e * N + i);
+          a.t[e][0] = v.x;
+          a.t[e][1] = v.y;
+        }
+      }
+    }
+  }
+  if constexpr (SRC == 0) {
+    if (px < npx) {
+      const size_t i = (size_t)n2 * npix + pix0 + px, step = (size_t)Q * npix;
+      for (int j = 0; j < pp.c; ++j) {
+        const typename RT<R>::V4* Mj = M + (size_t)j * N + i;
+        typename RT<R>::V4 m[4];
+#pragma unroll
+        for (int n1 = 0; n1 < 4; ++n1) m[n1] = ld_stream(Mj + n1 * step);
+        const R* dj = dir + (size_t)j * 3 * N + i;
+#pragma unroll
+        for (int n1 = 0; n1 < 4; ++n1) {
+          if (dir)
+            tacc_add_d(acc[n1], (R)m[n1].x, (R)m[n1].y, dj[n1 * step], dj[N + n1 * step],
+                       dj[2 * N + n1 * step], pp, j);
+          else
+            tacc_add(acc[n1], (R)m[n1].x, (R)m[n1].y, (R)m[n1].z, (R)m[n1].w, pp, j);
+        }
+      }
+      const R inv = R(1.0 / kFourPi);
+#pragma unroll
+      for (int n1 = 0; n1 < 4; ++n1) {
+        TAcc<R>& a = acc[n1];
+        a.aw = ((a.aw - R(1)) + a.as[0]) * inv;
+        a.as[1] *= inv;
+#pragma unroll
+        for (int e = 0; e < 5; ++e) {
+          a.t[e][0] *= inv;
+          a.t[e][1] *= inv;
+        }
+      }
+    }
+  }
+  const bool literal = pp.literal != 0;
+  const size_t fstride = (size_t)ns * npix, kstride = 3 * fstride;
+  const int rot = kb & 3;  // s1 = 0 takes output kb mod 4 of the 4-point transform
+  for (int a0 = 0; a0 < ang.n; a0 += A) {
+    const int na = ang.n - a0 < A ? ang.n - a0 : A;
+    if (a0 > 0) __syncthreads();  // the previous step's reads are done
+    for (int a = 0; a < na; ++a) {
+      const R ce = ang.ce[a0 + a], se = ang.se[a0 + a];
+      C p[4][3];
+#pragma unroll
+      for (int n1 = 0; n1 < 4; ++n1)
+        p_from_tacc(acc[n1].aw, acc[n1].as[1], acc[n1].t, ce, se, literal, p[n1]);
+      C* b = buf + a * 3 * 4 * KS + t;
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        dft4(p[0][f], p[1][f], p[2][f], p[3][f]);
+        // output k1 goes to s1 = (k1 - kb) mod 4 (uniform)
+#pragma unroll
+        for (int s1 = 0; s1 < 4; ++s1) {
+          const C v = rot == 0   ? p[s1][f]
+                      : rot == 1 ? p[(s1 + 1) & 3][f]
+                      : rot == 2 ? p[(s1 + 2) & 3][f]
+                                 : p[(s1 + 3) & 3][f];
+          b[(f * 4 + s1) * KS] = cmul(v, w[s1]);
+        }
+      }
+    }
+    __syncthreads();
+    const int items = na * 12 * PX;
+    for (int it = t; it < items; it += kPlThreads) {
+      const int q = it % PX, r = it / PX, s1 = r & 3, af = r >> 2;  // af = 3 a + f
+      if (q >= npx) continue;
+      const C* b = buf + r * KS + q;
+      C v[Q];
+#pragma unroll
+      for (int n = 0; n < Q; ++n) v[n] = b[n * PX];
+      C* o = out + (size_t)(3 * a0 + af) * fstride + (size_t)s1 * npix + pix0 + q;
+      const int mine = (ns - s1 + 3) >> 2;  // kept s2 of this s1
+      if constexpr (Q == 32) {
+        if (ns <= 64) {
+          dft32_first(v, (ns + 3) >> 2, [&](int s2, C x) {
+            if (s2 < mine) o[(size_t)(4 * s2) * npix] = x;
+          });
+        } else {
+          dft32(v);
+#pragma unroll
+          for (int s2 = 0; s2 < 32; ++s2)
+            if (s2 < mine) o[(size_t)(4 * s2) * npix] = v[s2];
+        }
+      } else {
+        dft_reg<Q>(v);
+#pragma unroll
+        for (int s2 = 0; s2 < Q; ++s2)
+          if (s2 < mine) o[(size_t)(4 * s2) * npix] = v[out_pos<Q>(s2)];
       }
     }
   }
@@ -617,36 +797,50 @@ __global__ void __launch_bounds__(32 * XRow<NX>::W, 2) k_x_planes(
   }
 }
 
-// Groups of at most 8 bins, as even as they come.
-int bins_per_group(int ns) {
-  const int G = (ns + 7) / 8, SB = (ns + G - 1) / G;
-  return SB < 2 ? 2 : SB;
+// The pass's shape for a stack: terms of the folded sum, bins of the larger
+// parity, groups of at most 8 bins of one parity, as even as they come.
+struct PlShape {
+  int np, H, SB, G;
+};
+PlShape pl_shape(int nz, int kb, int ns) {
+  PlShape p;
+  const bool even = nz % 2 == 0;
+  p.np = even ? 2 : 1;
+  p.H = (even ? nz / 2 : nz) / 2 + 1;
+  const int n0 = even ? (ns + 1 - (kb & 1)) / 2 : ns, n1 = ns - n0, most = n0 > n1 ? n0 : n1;
+  const int g = (most + 7) / 8;
+  p.SB = (most + g - 1) / g;
+  if (p.SB < 2) p.SB = 2;
+  p.G = (n0 + p.SB - 1) / p.SB + (even ? (n1 + p.SB - 1) / p.SB : 0);
+  return p;
 }
 
-template <typename R, int SRC, int SB>
+template <typename R, int SRC, int SB, bool EVEN>
 cudaError_t pol_planes_sb(const void* M, const void* nt, const void* dir, long long npix, int nz,
                           const PolParams<R>& pp, const AngleBatch<R>& ang, void* out, int kb,
                           int ns, const void* twz, cudaStream_t s) {
   using C = typename RT<R>::C;
   using F = Folded<C>;
-  const int H1 = nz / 2 + 1, G = (ns + SB - 1) / SB, NSP = G * ((SB + 1) & ~1);
-  // pixels of a block: all pair slots in use, whole 32-byte sectors per plane row
+  const PlShape sh = pl_shape(nz, kb, ns);
+  // pixels of a block: its threads' folds in use, whole 32-byte sectors per plane row
   constexpr int unit = 32 / (int)sizeof(C);
-  const int PX = kPlPairs / H1 / unit * unit;
+  const int PX = (EVEN ? kPlThreads : 2 * kPlThreads) / sh.H / unit * unit;
   if (PX < unit) return cudaErrorInvalidValue;
   // angles per step: up to 4 within ~100 KB (two FP32 blocks per SM), the
   // fewest idle threads in the last round of the items
-  const size_t per = (size_t)H1 * 3 * PX * sizeof(F), twb = (size_t)H1 * NSP * sizeof(C);
+  const size_t per = (size_t)sh.np * sh.H * 3 * PX * sizeof(F),
+               twb = (size_t)sh.H * sh.G * ((SB + 1) & ~1) * sizeof(C);
   int A = 1;
   double best = 0.0;
   for (int a = 1; a <= 4 && a <= ang.n; ++a) {
-    if (a > 1 && a * per + twb > 104 * 1024) break;
-    const int items = a * 3 * G * PX, rounds = (items + kPlThreads - 1) / kPlThreads;
+    const int items = a * 3 * sh.G * PX, rounds = (items + kPlThreads - 1) / kPlThreads;
+    if (a > 1 && (a * per + twb > 104 * 1024 || items >= 2048)) break;
     const double eff = (double)items / (rounds * kPlThreads) + 0.02 * a;
     if (eff > best) best = eff, A = a;
   }
+  if (3 * sh.G * PX >= 2048 || A * 3 * sh.G >= 2048) return cudaErrorInvalidValue;  // div_by's range
   const size_t smem = nz == 1 ? 0 : A * per + twb;
-  auto kern = k_pol_planes<R, SRC, SB>;
+  auto kern = k_pol_planes<R, SRC, SB, EVEN>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)((npix + PX - 1) / PX), kPlThreads, smem, s>>>(
@@ -655,25 +849,55 @@ cudaError_t pol_planes_sb(const void* M, const void* nt, const void* dir, long l
   return cudaGetLastError();
 }
 
-template <typename R, int SRC>
+template <typename R, int SRC, int Q>
+cudaError_t pol_planes_fft(const void* M, const void* nt, const void* dir, long long npix,
+                           const PolParams<R>& pp, const AngleBatch<R>& ang, void* out, int kb,
+                           int ns, const void* twz, cudaStream_t s) {
+  using C = typename RT<R>::C;
+  using P = PlFft<R, Q>;
+  const size_t smem = (size_t)P::A * 12 * P::KS * sizeof(C);
+  auto kern = k_pol_planes_fft<R, SRC, Q>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<(unsigned)((npix + P::PX - 1) / P::PX), kPlThreads, smem, s>>>(
+      (const typename RT<R>::V4*)M, (const C*)nt, (const R*)dir, npix, kb, ns, pp, ang, (C*)out,
+      (const C*)twz);
+  return cudaGetLastError();
+}
+
+template <typename R, int SRC, bool EVEN>
 cudaError_t pol_planes_src(const void* M, const void* nt, const void* dir, long long npix, int nz,
                            const PolParams<R>& pp, const AngleBatch<R>& ang, void* out, int kb,
                            int ns, const void* twz, cudaStream_t s) {
+  if constexpr (EVEN) {
+    // FP64 at nz = 128 would not fit its registers (64 of data, 96 of sums)
+    switch (nz) {
+      case 8: return pol_planes_fft<R, SRC, 2>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, s);
+      case 16: return pol_planes_fft<R, SRC, 4>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, s);
+      case 32: return pol_planes_fft<R, SRC, 8>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, s);
+      case 64: return pol_planes_fft<R, SRC, 16>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, s);
+      case 128:
+        if constexpr (sizeof(R) == 4)
+          return pol_planes_fft<R, SRC, 32>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, s);
+        break;
+      default: break;
+    }
+  }
 #define RSX_PL(B) \
-  case B: return pol_planes_sb<R, SRC, B>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, s);
-  switch (bins_per_group(ns)) {
-    RSX_PL(3) RSX_PL(4) RSX_PL(5) RSX_PL(6) RSX_PL(7) RSX_PL(8)
-    default: return pol_planes_sb<R, SRC, 2>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, s);
+  case B: return pol_planes_sb<R, SRC, B, EVEN>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, s);
+  switch (pl_shape(nz, kb, ns).SB) {
+    RSX_PL(2) RSX_PL(3) RSX_PL(4) RSX_PL(5) RSX_PL(6) RSX_PL(7) RSX_PL(8)
+    default: return cudaErrorInvalidValue;
   }
 #undef RSX_PL
 }
 }  // namespace
 
-bool pol_planes_fits(int precision, int nz, int ns) {
+bool pol_planes_fits(int precision, int nz, int kb, int ns) {
   if (nz < 1 || nz > kMaxPlanesNz || ns < 1 || ns > nz) return false;
   const size_t cs = precision == 32 ? sizeof(float2) : sizeof(double2);
-  const int H1 = nz / 2 + 1, SB = bins_per_group(ns), G = (ns + SB - 1) / SB;
-  return (2 * 3 * (size_t)kPlPairs + (size_t)H1 * G * ((SB + 1) & ~1)) * cs <= 220 * 1024;
+  const PlShape sh = pl_shape(nz, kb, ns);
+  return (4 * 3 * (size_t)kPlThreads + (size_t)sh.H * sh.G * ((sh.SB + 1) & ~1)) * cs <= 220 * 1024;
 }
 
 template <typename R>
@@ -683,8 +907,11 @@ cudaError_t launch_pol_planes(const void* M, const void* nt, const void* dir, lo
   if (nz < 1 || nz > kMaxPlanesNz || ns < 1 || ns > nz || kb < 0 || kb >= nz || ang.n < 1 ||
       ang.n > kMaxAngleBatch)
     return cudaErrorInvalidValue;
-  return nt ? pol_planes_src<R, 1>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, s)
-            : pol_planes_src<R, 0>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, s);
+  if (nz % 2)
+    return nt ? pol_planes_src<R, 1, false>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, s)
+              : pol_planes_src<R, 0, false>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, s);
+  return nt ? pol_planes_src<R, 1, true>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, s)
+            : pol_planes_src<R, 0, true>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, s);
 }
 
 template <typename R>
