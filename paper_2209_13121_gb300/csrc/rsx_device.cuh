@@ -565,64 +565,186 @@ __device__ __forceinline__ void block_fft_ct(typename RT<R>::C* buf, const typen
 //   y[(j - k) RAD + k + r Ns] = V_r,
 // which leaves the spectrum in natural order after the last pass (the same
 // self-sorting scheme as the power-of-two passes above, with any radix).
-// x and y are different buffers.  tw[t] = exp(-2 pi i t / n); the twiddle
-// index r k n / (Ns RAD) stays below n.
+// x and y are different buffers, element i at x[i * es].  tw[t] =
+// exp(-2 pi i t / n); the twiddle index r k n / (Ns RAD) stays below n.
 // ---------------------------------------------------------------------------
 
-// RAD-point forward DFT by its definition, natural order in and out, with
-// W_RAD^q = tw[q * tstep] (tstep = n / RAD).
-template <int RAD, typename C>
-__device__ __forceinline__ void dft_def(C* v, const C* tw, int tstep) {
-  C out[RAD];
-#pragma unroll
-  for (int r = 0; r < RAD; ++r) {
-    out[r] = v[0];
-#pragma unroll
-    for (int m = 1; m < RAD; ++m) out[r] = cadd(out[r], cmul(v[m], tw[((r * m) % RAD) * tstep]));
+// Unsigned division by a run-time constant: it / d for it < 2^20, d < 2^12,
+// by one multiplication (mul = ceil(2^32 / d); exact while it < 2^32 / d).
+struct FastDiv {
+  unsigned d, mul;
+};
+__device__ __forceinline__ int fast_div(int it, FastDiv f) {
+  return f.d == 1 ? it : (int)__umulhi((unsigned)it, f.mul);
+}
+
+template <int P> struct OddRoots;
+template <> struct OddRoots<3> {  // cos and sin of 2 pi j / 3
+  static __host__ __device__ constexpr double c(int j) {
+    constexpr double t[] = {
+        1, -0.49999999999999977796, -0.50000000000000044409};
+    return t[j];
   }
+  static __host__ __device__ constexpr double s(int j) {
+    constexpr double t[] = {
+        0, 0.86602540378443870761, -0.86602540378443837454};
+    return t[j];
+  }
+};
+template <> struct OddRoots<5> {  // cos and sin of 2 pi j / 5
+  static __host__ __device__ constexpr double c(int j) {
+    constexpr double t[] = {
+        1, 0.30901699437494745126, -0.80901699437494734024, -0.80901699437494756229,
+        0.30901699437494722922};
+    return t[j];
+  }
+  static __host__ __device__ constexpr double s(int j) {
+    constexpr double t[] = {
+        0, 0.95105651629515353118, 0.58778525229247324813, -0.58778525229247302608,
+        -0.9510565162951536422};
+    return t[j];
+  }
+};
+template <> struct OddRoots<7> {  // cos and sin of 2 pi j / 7
+  static __host__ __device__ constexpr double c(int j) {
+    constexpr double t[] = {
+        1, 0.62348980185873359439, -0.22252093395631433737, -0.90096886790241903498,
+        -0.900968867902419146, -0.22252093395631458717, 0.62348980185873337234};
+    return t[j];
+  }
+  static __host__ __device__ constexpr double s(int j) {
+    constexpr double t[] = {
+        0, 0.78183148246802980363, 0.97492791218182361934, 0.43388373911755823142,
+        -0.43388373911755800938, -0.97492791218182361934, -0.78183148246802991466};
+    return t[j];
+  }
+};
+template <> struct OddRoots<11> {  // cos and sin of 2 pi j / 11
+  static __host__ __device__ constexpr double c(int j) {
+    constexpr double t[] = {
+        1, 0.84125353283118120551, 0.41541501300188643508, -0.1423148382732850048,
+        -0.65486073394528498959, -0.95949297361449736865, -0.95949297361449747967,
+        -0.65486073394528521163, -0.14231483827328522684, 0.41541501300188604651,
+        0.84125353283118120551};
+    return t[j];
+  }
+  static __host__ __device__ constexpr double s(int j) {
+    constexpr double t[] = {
+        0, 0.54064081745559755543, 0.90963199535451833011, 0.98982144188093279524,
+        0.7557495743542582689, 0.28173255684142967104, -0.28173255684142939348,
+        -0.75574957435425815788, -0.98982144188093268422, -0.90963199535451855215,
+        -0.54064081745559744441};
+    return t[j];
+  }
+};
+template <> struct OddRoots<13> {  // cos and sin of 2 pi j / 13
+  static __host__ __device__ constexpr double c(int j) {
+    constexpr double t[] = {
+        1, 0.88545602565320991051, 0.56806474673115592289, 0.12053668025532300601,
+        -0.35460488704253545489, -0.74851074817110119231, -0.9709418174260520118,
+        -0.97094181742605212282, -0.74851074817110130333, -0.35460488704253589898,
+        0.12053668025532320029, 0.56806474673115481266, 0.88545602565321002153};
+    return t[j];
+  }
+  static __host__ __device__ constexpr double s(int j) {
+    constexpr double t[] = {
+        0, 0.46472317204376850652, 0.82298386589365635224, 0.99270887409805397272,
+        0.93501624268541483342, 0.66312265824079519305, 0.23931566428755768339,
+        -0.23931566428755743359, -0.66312265824079497101, -0.9350162426854147224,
+        -0.99270887409805397272, -0.82298386589365701838, -0.4647231720437683955};
+    return t[j];
+  }
+};
+
+// P-point forward DFT for an odd prime P, natural order in and out: with
+// t_m = v_m + v_(P-m), d_m = v_m - v_(P-m) (m <= H = (P - 1) / 2),
+//   X_k, X_(P-k) = v_0 + sum_m cos(2 pi k m / P) t_m  -+  i sum_m sin(2 pi k m / P) d_m.
+template <int P, int K, int M, typename C>
+__device__ __forceinline__ void dft_odd_sums(C& a, C& b, const C* tt, const C* dd) {
+  using R = decltype(a.x);
+  if constexpr (M <= (P - 1) / 2) {
+    constexpr R c = R(OddRoots<P>::c(K * M % P)), sn = R(OddRoots<P>::s(K * M % P));
+    a.x += c * tt[M - 1].x;
+    a.y += c * tt[M - 1].y;
+    b.x += sn * dd[M - 1].x;
+    b.y += sn * dd[M - 1].y;
+    dft_odd_sums<P, K, M + 1>(a, b, tt, dd);
+  }
+}
+template <int P, int K, typename C>
+__device__ __forceinline__ void dft_odd_outputs(C* v, C v0, const C* tt, const C* dd) {
+  using R = decltype(v0.x);
+  if constexpr (K <= (P - 1) / 2) {
+    C a = v0, b;
+    b.x = b.y = R(0);
+    dft_odd_sums<P, K, 1>(a, b, tt, dd);
+    v[K].x = a.x + b.y;  // a - i b
+    v[K].y = a.y - b.x;
+    v[P - K].x = a.x - b.y;
+    v[P - K].y = a.y + b.x;
+    dft_odd_outputs<P, K + 1>(v, v0, tt, dd);
+  }
+}
+template <int P, typename C> __device__ __forceinline__ void dft_odd(C* v) {
+  constexpr int H = (P - 1) / 2;
+  C tt[H], dd[H];
+  const C v0 = v[0];
 #pragma unroll
-  for (int r = 0; r < RAD; ++r) v[r] = out[r];
+  for (int m = 0; m < H; ++m) {
+    tt[m] = cadd(v[m + 1], v[P - 1 - m]);
+    dd[m] = csub(v[m + 1], v[P - 1 - m]);
+    v[0] = cadd(v[0], tt[m]);
+  }
+  dft_odd_outputs<P, 1>(v, v0, tt, dd);
 }
 
 // One butterfly of a pass with a radix known at compile time (2, 4, 8, 16
-// by the register DFTs, 3, 5, 7 by definition).
+// by the power-of-two register DFTs, 3, 5, 7, 11, 13 by dft_odd).
 template <int RAD, typename C>
-__device__ __forceinline__ void any_butterfly(const C* x, C* y, int j, int n, int Ns, const C* tw) {
-  const int nb = n / RAD, k = j % Ns, ts = n / (Ns * RAD);
+__device__ __forceinline__ void any_butterfly(const C* x, C* y, int es, int j, int nb, int Ns,
+                                              FastDiv dNs, int ts, const C* tw) {
+  const int k = j - fast_div(j, dNs) * Ns;
   C v[RAD];
+  const C* xj = x + j * es;
+  const int step = nb * es;
 #pragma unroll
-  for (int r = 0; r < RAD; ++r) v[r] = x[j + r * nb];
+  for (int r = 0; r < RAD; ++r) v[r] = xj[r * step];
   if (k) {
+    const int kt = k * ts;
 #pragma unroll
-    for (int r = 1; r < RAD; ++r) v[r] = cmul(v[r], tw[r * k * ts]);
+    for (int r = 1; r < RAD; ++r) v[r] = cmul(v[r], tw[r * kt]);
   }
-  const int o = (j - k) * RAD + k;
+  C* yo = y + ((j - k) * RAD + k) * es;
+  const int ws = Ns * es;
   if constexpr (RAD == 2 || RAD == 4 || RAD == 8 || RAD == 16) {
     dft_reg<RAD>(v);
 #pragma unroll
-    for (int r = 0; r < RAD; ++r) y[o + r * Ns] = v[out_pos<RAD>(r)];
+    for (int r = 0; r < RAD; ++r) yo[r * ws] = v[out_pos<RAD>(r)];
   } else {
-    dft_def<RAD>(v, tw, nb);
+    dft_odd<RAD>(v);
 #pragma unroll
-    for (int r = 0; r < RAD; ++r) y[o + r * Ns] = v[r];
+    for (int r = 0; r < RAD; ++r) yo[r * ws] = v[r];
   }
 }
 
-// Output r of one butterfly for any other radix (a prime above 7), summed
+// Output r of one butterfly for any other radix (a prime above 13), summed
 // straight from x (O(RAD) work; a pass spreads its outputs over threads);
 // the combined exponent of the pass twiddle and W_RAD^(r m) is reduced
 // modulo n.
 template <typename C>
-__device__ __forceinline__ void any_output_prime(const C* x, C* y, int j, int r, int rad, int n,
-                                                 int Ns, const C* tw) {
+__device__ __forceinline__ void any_output_prime(const C* x, C* y, int es, int j, int r, int rad,
+                                                 int n, int Ns, const C* tw) {
   const int nb = n / rad, k = j % Ns, ts = n / (Ns * rad);
   const int o = (j - k) * rad + k;
-  C acc = x[j];
+  C acc = x[j * es];
+  int e = 0;
+  const int de = (int)(((long long)k * ts + (long long)r * nb) % n);  // exponent of m = 1
   for (int m = 1; m < rad; ++m) {
-    const long long e = (long long)m * k * ts + (long long)((r * m) % rad) * nb;
-    acc = cadd(acc, cmul(x[j + m * nb], tw[(int)(e % n)]));
+    e += de;
+    if (e >= n) e -= n;
+    acc = cadd(acc, cmul(x[(j + m * nb) * es], tw[e]));
   }
-  y[o + r * Ns] = acc;
+  y[(o + r * Ns) * es] = acc;
 }
 
 }  // namespace rsx
