@@ -330,7 +330,7 @@ struct XMask {
   unsigned m[256];
 };
 // y_planes_ok: ny = 512, 1024 or 2048 and nx a multiple of 16 (up to 4096).
-// launch_y_planes: the y-FFT of nfields x ns planes at p (ns < nz), storing
+// launch_y_planes: the y-FFT of nfields x ns planes at p (ns < nz, or nz = 1), storing
 // each pixel only in the planes of its two bins; tmap: a tensor map over the
 // planes as [nfields ns][ny][2 nx] floats with (16384 / ny) x 256 x 1 boxes;
 // tw: W512^j (512 rows) or W1024^(n1 k2) as [32][32]; twy: W2048^j (2048

@@ -961,7 +961,8 @@ cudaError_t launch_y_planes(const void* tmap, void* p, int nx, int ny, int nz, i
                             long long nfields, const YRuns& runs, const unsigned short* b0idx,
                             const void* tw, const void* twy, int* err, int n_sm, unsigned poll,
                             cudaStream_t s) {
-  if (!y_planes_ok(nx, ny) || ns < 1 || ns >= nz || nz > kMaxPlanesNz || kb < 0 || kb >= nz ||
+  if (!y_planes_ok(nx, ny) || ns < 1 || (ns >= nz && nz > 1) || nz > kMaxPlanesNz || kb < 0 ||
+      kb >= nz ||
       runs.n != nx / 16)
     return cudaErrorInvalidValue;
   for (int i = 0; i < runs.n; ++i)
