@@ -2423,20 +2423,28 @@ __global__ void __launch_bounds__(256) k_bins5_from_part(const float4* __restric
   }
 }
 
-// Detector value of one pixel for e = (ce, se, 0) from the linearity
-// bins (Eq. (Ewald) with p~ = N_t~ e per bin; zero off the sphere).
+// The ten bin values of one pixel on the linearity path (five N_t entries,
+// two bins), [2][5].
 template <typename R>
-__device__ __forceinline__ R linear_pixel(const typename RT<R>::C* __restrict__ bins, long long npix,
-                                          long long pix, const Geo<R>& g, R ce, R se,
-                                          int literal) {
+__device__ __forceinline__ void load_bins(const typename RT<R>::C* __restrict__ bins,
+                                          long long npix, long long pix,
+                                          typename RT<R>::C (&t)[2][5]) {
+#pragma unroll
+  for (int b = 0; b < 2; ++b)
+#pragma unroll
+    for (int q = 0; q < 5; ++q) t[b][q] = bins[(size_t)(2 * q + b) * npix + pix];
+}
+
+// Detector value of one pixel for e = (ce, se, 0) from them (Eq. (Ewald)
+// with p~ = N_t~ e per bin).
+template <typename R>
+__device__ __forceinline__ R linear_pixel(const typename RT<R>::C (&tb)[2][5], const Geo<R>& g,
+                                          R ce, R se, int literal) {
   using C = typename RT<R>::C;
-  if (g.b0 < 0) return R(0);
   C pb[2][3];
 #pragma unroll
   for (int b = 0; b < 2; ++b) {
-    C t[5];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) t[q] = bins[(size_t)(2 * q + b) * npix + pix];
+    const C (&t)[5] = tb[b];
     // columns x = (xx, xy, xz) and y = (xy, yy, yz) of N_t, combined with e
     const C px = RT<R>::mk(ce * t[0].x + se * t[1].x, ce * t[0].y + se * t[1].y);
     const C py = RT<R>::mk(ce * t[1].x + se * t[2].x, ce * t[1].y + se * t[2].y);
@@ -2460,22 +2468,33 @@ __global__ void __launch_bounds__(256) k_ewald_linear(const typename RT<R>::C* _
   const long long npix = (long long)nx * ny;
   const long long pix = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (pix >= npix) return;
-  img[shifted_pixel(pix, nx, ny)] = linear_pixel<R>(bins, npix, pix, geo[pix], ce, se, literal);
+  const Geo<R> g = geo[pix];
+  R val = R(0);
+  if (g.b0 >= 0) {
+    typename RT<R>::C t[2][5];
+    load_bins<R>(bins, npix, pix, t);
+    val = linear_pixel<R>(t, g, ce, se, literal);
+  }
+  img[shifted_pixel(pix, nx, ny)] = val;
 }
 
-// The same for a batch of angles: imgs[a] for a = blockIdx.y.
-template <typename R>
-__global__ void __launch_bounds__(256) k_ewald_linear_many(const typename RT<R>::C* __restrict__ bins,
-                                                           int nx, int ny,
-                                                           const Geo<R>* __restrict__ geo,
-                                                           AngleBatch<R> ab, int literal,
-                                                           R* __restrict__ imgs) {
+// The images of a batch of angles.  A thread takes AP angles of one pixel:
+// the pixel's 80 bytes of bins (FP32) and its geometry are read once for
+// them instead of once per angle (1024 x 1024, 91 angles: 1.42 -> 0.33 ms).
+template <typename R, int AP>
+__global__ void __launch_bounds__(256) k_ewald_linear_many(
+    const typename RT<R>::C* __restrict__ bins, int nx, int ny, const Geo<R>* __restrict__ geo,
+    const __grid_constant__ AngleBatch<R> ab, int literal, R* __restrict__ imgs) {
   const long long npix = (long long)nx * ny;
   const long long pix = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (pix >= npix) return;
-  const int a = blockIdx.y;
-  imgs[(size_t)a * npix + shifted_pixel(pix, nx, ny)] =
-      linear_pixel<R>(bins, npix, pix, geo[pix], ab.ce[a], ab.se[a], literal);
+  const int a0 = blockIdx.y * AP, a1 = a0 + AP < ab.n ? a0 + AP : ab.n;
+  const Geo<R> g = geo[pix];
+  typename RT<R>::C t[2][5];
+  if (g.b0 >= 0) load_bins<R>(bins, npix, pix, t);
+  R* dst = imgs + shifted_pixel(pix, nx, ny);
+  for (int a = a0; a < a1; ++a)
+    dst[(size_t)a * npix] = g.b0 < 0 ? R(0) : linear_pixel<R>(t, g, ab.ce[a], ab.se[a], literal);
 }
 
 // ------------------------------------------------ Algorithm 3 (NrComputation)
@@ -3374,9 +3393,12 @@ cudaError_t launch_ewald_linear_many(const void* bins, int nx, int ny, const Geo
   if (ab.n <= 0) return cudaSuccess;
   if (ab.n > kMaxAngleBatch) return cudaErrorInvalidValue;
   const long long npix = (long long)nx * ny;
-  const dim3 grid(grid1(npix, 256), ab.n);
-  k_ewald_linear_many<R><<<grid, 256, 0, s>>>((const typename RT<R>::C*)bins, nx, ny, geo, ab,
-                                              literal ? 1 : 0, (R*)imgs);
+  // 16 angles per thread once one angle's pixels fill the chip
+  const bool big = npix >= (1 << 17);
+  const dim3 grid(grid1(npix, 256), big ? (ab.n + 15) / 16 : ab.n);
+  auto kern = big ? k_ewald_linear_many<R, 16> : k_ewald_linear_many<R, 1>;
+  kern<<<grid, 256, 0, s>>>((const typename RT<R>::C*)bins, nx, ny, geo, ab, literal ? 1 : 0,
+                            (R*)imgs);
   return cudaGetLastError();
 }
 
