@@ -358,6 +358,15 @@ cudaError_t launch_y_fft(rsx_context* c, void* data, long long ncomp, cudaStream
   return rsx::launch_col_fft<R>(data, g.ny, g.nx, g.nx, bt, c->twy, s);
 }
 
+// A plan of the planes path for one energy (see planes_plan): the kept run of
+// q_z bins kb .. kb + ns - 1 mod nz and the angles per batch.
+struct ZPlan {
+  int kb = 0, ns = 0, kz = 0;
+  bool zfft = false;  // p and its z transform by launch_pol_zfft_multi
+  bool film = false;  // nz = 1: p and its x-FFT by launch_pol_fft4s_tma_multi
+};
+bool lin_plan(const rsx_context* c, int ie, ZPlan* zp);
+
 // exp(-2 pi i t / n), t < n, in the context precision.
 int upload_twiddles(rsx_context* c, int n, void** dst) {
   const int prec = c->cfg.precision;
@@ -466,6 +475,126 @@ cudaError_t fused_yz(rsx_context* c, const CUtensorMap* map, int nf, long long* 
                             c->wait_polls, L, s);
 }
 
+// x-FFT of the rows of nfields x ns planes at data, in place.
+template <typename R>
+cudaError_t planes_x_fft(rsx_context* c, void* data, const ZPlan& zp, long long nfields,
+                         const rsx::XMask& xm, cudaStream_t s) {
+  const rsx_config& g = c->cfg;
+  if (g.nx == 1) return cudaSuccess;
+  if (sizeof(R) == 4 && (g.nx == 512 || (g.nx == 1024 && c->tw4) || (g.nx == 2048 && c->tw2k)))
+    return rsx::launch_x_planes(data, g.nx, g.ny, zp.ns, nfields, xm,
+                                g.nx == 1024 ? c->tw4 : g.nx == 2048 ? c->tw2k : c->twx, s);
+  const long long nrows = nfields * zp.ns * g.ny;
+  if (g.nx == 1024 && c->tw4) return rsx::launch_row_fft4s<R>(data, nrows, c->tw4, s);
+  return rsx::launch_row_fft<R>(data, g.nx, nrows, c->twx, s);
+}
+
+// (A film's whole plane is stored: 2048 rows then go 4 columns, 32 bytes, at a
+// time, 15.4 ms per two energies of 91 angles at 2048 x 2048; the 8-column
+// kernel 12.0.)
+// y-FFT of nfields x ns contiguous [ny][nx] planes at data, in place; on the
+// tuned sizes only what the image reads is transformed and stored.
+template <typename R>
+cudaError_t planes_y_fft(rsx_context* c, void* data, const ZPlan& zp, long long nfields,
+                         const rsx::YRuns& runs, cudaStream_t s) {
+  const rsx_config& g = c->cfg;
+  if (g.ny == 1) return cudaSuccess;
+  if (sizeof(R) == 4 && rsx::y_planes_ok(g.nx, g.ny) && c->b0idx && c->n_sm > 0 &&
+      (zp.ns < g.nz || (zp.film && g.ny != 2048))) {
+    CUtensorMap tm;
+    if (!make_tmap(c, data, nfields * zp.ns, &tm, 16384u / g.ny, CU_TENSOR_MAP_L2_PROMOTION_L2_128B))
+      return cudaErrorUnknown;
+    return rsx::launch_y_planes(&tm, data, g.nx, g.ny, g.nz, zp.kb, zp.ns, nfields, runs, c->b0idx,
+                                g.ny == 512 ? c->twy : c->tw4, g.ny == 2048 ? c->twy : nullptr,
+                                c->err, c->n_sm, c->wait_polls, s);
+  }
+  const rsx::ColBatches bt = {nfields * zp.ns, 1, c->npix, 0, 0};
+  if (g.ny == 1024 && g.nx % 8 == 0 && c->tw4)
+    return rsx::launch_col_fft4s<R>(data, g.nx, g.nx, bt, c->tw4, s);
+  return rsx::launch_col_fft<R>(data, g.ny, g.nx, g.nx, bt, c->twy, s);
+}
+
+// The runs of planes that each 16-column group's pixels read, and per plane
+// the groups of nx / 32 columns some run meets.  A column's bins run from
+// the one at q_y = 0 down to the one at the largest |q_y| still on the sphere;
+// the bounds are wide enough for any rounding, as in lowest_bin.
+void plane_runs(const rsx_config& g, double k, const ZPlan& zp, rsx::YRuns* runs,
+                rsx::XMask* xm) {
+  memset(runs, 0, sizeof(*runs));
+  memset(xm, zp.ns < g.nz ? 0 : 0xff, sizeof(*xm));
+  if (zp.film) {  // the one plane, everywhere
+    runs->n = g.nx / 16;
+    for (int cg = 0; cg <= runs->n; ++cg) runs->start[cg] = (unsigned short)cg;
+    return;
+  }
+  if (zp.ns >= g.nz || g.nx % 16 || g.nx > 4096) {
+    memset(xm, 0xff, sizeof(*xm));
+    return;
+  }
+  const double two_pi = 2.0 * kPi, dqx = two_pi / (g.nx * g.voxel_nm),
+               dqy = two_pi / (g.ny * g.voxel_nm), dqz = two_pi / (g.nz * g.voxel_nm);
+  const double edge = 1e-12 * k * k, qy = dqy * (g.ny / 2);
+  const int blo = 2 - zp.ns;
+  runs->n = g.nx / 16;
+  for (int cg = 0; cg < runs->n; ++cg) {
+    int fmin = g.nx, fmax = 0;
+    for (int i = 0; i < 16; ++i) {
+      const int mx = cg * 16 + i, f = mx < g.nx / 2 ? mx : g.nx - mx;
+      fmin = f < fmin ? f : fmin;
+      fmax = f > fmax ? f : fmax;
+    }
+    const double top = k * k - dqx * fmin * dqx * fmin;
+    const double low = k * k - dqx * fmax * dqx * fmax - qy * qy;
+    int len = 0;
+    if (top >= -edge) {
+      const double th = (-k + sqrt(top > 0.0 ? top : 0.0)) / dqz;
+      const double tl = (low > edge ? -k + sqrt(low) : -k) / dqz;
+      int hi = (int)floor(th + 1e-9 * (1.0 + fabs(th))) + 1 - blo;
+      int lo = (int)floor(tl - 1e-9 * (1.0 + fabs(tl))) - blo;
+      lo = lo < 0 ? 0 : lo;
+      hi = hi > zp.ns - 1 ? zp.ns - 1 : hi;
+      runs->first[cg] = (unsigned char)lo;
+      len = hi >= lo ? hi - lo + 1 : 0;
+      for (int z = lo; z <= hi; ++z) xm->m[z] |= 1u << (cg * 16 / ((g.nx + 31) / 32));
+    }
+    runs->start[cg + 1] = (unsigned short)(runs->start[cg] + len);
+  }
+}
+
+// The same for stacks the z-first form serves: N_t's entries z-transformed
+// as they are formed (from the device morphology; from N_t where that was
+// streamed from the host) and only the kept planes transformed laterally.
+template <typename R>
+int lin_planes_bins(rsx_context* c, int ie, const ZPlan& zp, cudaStream_t s) {
+  const rsx_config& g = c->cfg;
+  int rc;
+  if (c->M_host && (rc = ensure_nt<R>(c, ie, s))) return rc;
+  rsx::YRuns runs;
+  rsx::XMask xm;
+  plane_runs(g, wavenumber(c->energies[ie]), zp, &runs, &xm);
+  {
+    PhaseTimer pt(c, RSX_PHASE_NT, s);
+    RSX_CK(rsx::launch_lin_planes<R>(c->M, c->M_host ? c->nt : nullptr, c->npix, g.nz,
+                                     make_params<R>(c, ie, 0.0, 0), c->ft, zp.kb, zp.ns, c->twz, s),
+           "N_t + z-FFT kernel");
+  }
+  {
+    PhaseTimer pt(c, RSX_PHASE_FFTX, s);
+    RSX_CK(planes_x_fft<R>(c, c->ft, zp, 5, xm, s), "x-FFT kernel");
+  }
+  {
+    PhaseTimer pt(c, RSX_PHASE_FFTY, s);
+    RSX_CK(planes_y_fft<R>(c, c->ft, zp, 5, runs, s), "y-FFT kernel");
+  }
+  const double dc = -(double)(g.n_components - 1) / (4.0 * kPi) * (double)c->N;
+  PhaseTimer pt(c, RSX_PHASE_EWALD, s);
+  RSX_CK(rsx::launch_bins5_planes<R>(c->ft, g.nx, g.ny, g.nz, zp.kb, zp.ns, (const Geo<R>*)c->geo,
+                                     dc, c->bins5, s),
+         "q_z bins kernel");
+  c->bins_energy = ie;
+  return RSX_OK;
+}
+
 // Linearity fast path, once per energy: FFT (x and y) of N_t's five
 // entries, then their two q_z bins per pixel.
 template <typename R>
@@ -474,6 +603,8 @@ int ensure_bins(rsx_context* c, int ie, cudaStream_t s) {
   const rsx_config& g = c->cfg;
   int rc = ensure_geo<R>(c, ie, s);
   if (rc) return rc;
+  ZPlan zp;
+  if (lin_plan(c, ie, &zp)) return lin_planes_bins<R>(c, ie, zp, s);
   if ((rc = ensure_nt<R>(c, ie, s))) return rc;
   {
     PhaseTimer pt(c, RSX_PHASE_POL_FFTX, s);
@@ -704,11 +835,6 @@ static int angle_batch_of(const rsx_config* cfg) {
 // wide enough for any such difference: a pixel within 1e-12 k^2 of the
 // sphere's edge counts as on it (at q_z = -k, its lowest possible value),
 // and a t within 1e-9 above an integer also takes the bin below.
-struct ZPlan {
-  int kb = 0, ns = 0, kz = 0;
-  bool zfft = false;  // p and its z transform by launch_pol_zfft_multi
-  bool film = false;  // nz = 1: p and its x-FFT by launch_pol_fft4s_tma_multi
-};
 
 static int lowest_bin(const rsx_config& g, double k) {
   const double two_pi = 2.0 * kPi;
@@ -780,6 +906,19 @@ static int image_batch(const rsx_config* cfg) {
   const long long n = uses_yz(cfg) ? (long long)part_bytes(cfg) / img : (64LL << 20) / img;
   return n < 1 ? 1 : n > rsx::kMaxAngleBatch ? rsx::kMaxAngleBatch : (int)n;
 }
+
+namespace {
+// The linearity path's plan: while at most 3/4 of the bins are kept, on
+// stacks its z-first pass takes.
+bool lin_plan(const rsx_context* c, int ie, ZPlan* zp) {
+  const rsx_config& g = c->cfg;
+  if (g.algorithm != 3 || !rsx::lin_planes_fits(g.precision, g.nz)) return false;
+  const int blo = lowest_bin(g, wavenumber(c->energies[ie]));
+  zp->ns = 2 - blo;
+  zp->kb = ((blo % g.nz) + g.nz) % g.nz;
+  return 4 * zp->ns <= 3 * g.nz;
+}
+}  // namespace
 
 static bool zfirst_plan(const rsx_context* c, int ie, ZPlan* zp) {
   const rsx_config& g = c->cfg;
@@ -973,7 +1112,7 @@ int rsx_create(const rsx_config* cfg, rsx_context** out) {
     delete c;
     return rc;
   }
-  if (cfg->nx == 2048 && cfg->precision == 32 && cfg->algorithm != 3 && (rc = upload_tw2k(c))) {
+  if (cfg->nx == 2048 && cfg->precision == 32 && (rc = upload_tw2k(c))) {
     free_all(c);
     delete c;
     return rc;
@@ -1314,92 +1453,6 @@ int run_energy_angles_batched(rsx_context* c, int ie, double start, double inc, 
   return RSX_OK;
 }
 
-// x-FFT of the rows of nfields x ns planes in p, in place.
-template <typename R>
-cudaError_t planes_x_fft(rsx_context* c, const ZPlan& zp, long long nfields, const rsx::XMask& xm,
-                         cudaStream_t s) {
-  const rsx_config& g = c->cfg;
-  if (g.nx == 1) return cudaSuccess;
-  if (sizeof(R) == 4 && (g.nx == 512 || (g.nx == 1024 && c->tw4) || (g.nx == 2048 && c->tw2k)))
-    return rsx::launch_x_planes(c->p, g.nx, g.ny, zp.ns, nfields, xm,
-                                g.nx == 1024 ? c->tw4 : g.nx == 2048 ? c->tw2k : c->twx, s);
-  const long long nrows = nfields * zp.ns * g.ny;
-  if (g.nx == 1024 && c->tw4) return rsx::launch_row_fft4s<R>(c->p, nrows, c->tw4, s);
-  return rsx::launch_row_fft<R>(c->p, g.nx, nrows, c->twx, s);
-}
-
-// (A film's whole plane is stored: 2048 rows then go 4 columns, 32 bytes, at a
-// time, 15.4 ms per two energies of 91 angles at 2048 x 2048; the 8-column
-// kernel 12.0.)
-// y-FFT of nfields x ns contiguous [ny][nx] planes in p, in place; on the
-// tuned sizes only what the image reads is transformed and stored.
-template <typename R>
-cudaError_t planes_y_fft(rsx_context* c, const ZPlan& zp, long long nfields,
-                         const rsx::YRuns& runs, cudaStream_t s) {
-  const rsx_config& g = c->cfg;
-  if (g.ny == 1) return cudaSuccess;
-  if (sizeof(R) == 4 && y_tuned(&g) && c->b0idx && c->n_sm > 0 &&
-      (zp.ns < g.nz || (zp.film && g.ny != 2048))) {
-    CUtensorMap tm;
-    if (!make_tmap(c, c->p, nfields * zp.ns, &tm, 16384u / g.ny, CU_TENSOR_MAP_L2_PROMOTION_L2_128B))
-      return cudaErrorUnknown;
-    return rsx::launch_y_planes(&tm, c->p, g.nx, g.ny, g.nz, zp.kb, zp.ns, nfields, runs, c->b0idx,
-                                g.ny == 512 ? c->twy : c->tw4, g.ny == 2048 ? c->twy : nullptr,
-                                c->err, c->n_sm, c->wait_polls, s);
-  }
-  const rsx::ColBatches bt = {nfields * zp.ns, 1, c->npix, 0, 0};
-  if (g.ny == 1024 && g.nx % 8 == 0 && c->tw4)
-    return rsx::launch_col_fft4s<R>(c->p, g.nx, g.nx, bt, c->tw4, s);
-  return rsx::launch_col_fft<R>(c->p, g.ny, g.nx, g.nx, bt, c->twy, s);
-}
-
-// The runs of planes that each 16-column group's pixels read, and per plane
-// the groups of nx / 32 columns some run meets.  A column's bins run from
-// the one at q_y = 0 down to the one at the largest |q_y| still on the sphere;
-// the bounds are wide enough for any rounding, as in lowest_bin.
-void plane_runs(const rsx_config& g, double k, const ZPlan& zp, rsx::YRuns* runs,
-                rsx::XMask* xm) {
-  memset(runs, 0, sizeof(*runs));
-  memset(xm, zp.ns < g.nz ? 0 : 0xff, sizeof(*xm));
-  if (zp.film) {  // the one plane, everywhere
-    runs->n = g.nx / 16;
-    for (int cg = 0; cg <= runs->n; ++cg) runs->start[cg] = (unsigned short)cg;
-    return;
-  }
-  if (zp.ns >= g.nz || g.nx % 16 || g.nx > 4096) {
-    memset(xm, 0xff, sizeof(*xm));
-    return;
-  }
-  const double two_pi = 2.0 * kPi, dqx = two_pi / (g.nx * g.voxel_nm),
-               dqy = two_pi / (g.ny * g.voxel_nm), dqz = two_pi / (g.nz * g.voxel_nm);
-  const double edge = 1e-12 * k * k, qy = dqy * (g.ny / 2);
-  const int blo = 2 - zp.ns;
-  runs->n = g.nx / 16;
-  for (int cg = 0; cg < runs->n; ++cg) {
-    int fmin = g.nx, fmax = 0;
-    for (int i = 0; i < 16; ++i) {
-      const int mx = cg * 16 + i, f = mx < g.nx / 2 ? mx : g.nx - mx;
-      fmin = f < fmin ? f : fmin;
-      fmax = f > fmax ? f : fmax;
-    }
-    const double top = k * k - dqx * fmin * dqx * fmin;
-    const double low = k * k - dqx * fmax * dqx * fmax - qy * qy;
-    int len = 0;
-    if (top >= -edge) {
-      const double th = (-k + sqrt(top > 0.0 ? top : 0.0)) / dqz;
-      const double tl = (low > edge ? -k + sqrt(low) : -k) / dqz;
-      int hi = (int)floor(th + 1e-9 * (1.0 + fabs(th))) + 1 - blo;
-      int lo = (int)floor(tl - 1e-9 * (1.0 + fabs(tl))) - blo;
-      lo = lo < 0 ? 0 : lo;
-      hi = hi > zp.ns - 1 ? zp.ns - 1 : hi;
-      runs->first[cg] = (unsigned char)lo;
-      len = hi >= lo ? hi - lo + 1 : 0;
-      for (int z = lo; z <= hi; ++z) xm->m[z] |= 1u << (cg * 16 / ((g.nx + 31) / 32));
-    }
-    runs->start[cg + 1] = (unsigned short)(runs->start[cg] + len);
-  }
-}
-
 // All angles of one energy on the planes path (plan from planes_plan): per
 // batch of up to kz angles, the polarisation + z-transform pass keeps the ns
 // q_z planes of every angle (angle k, field f, plane s at
@@ -1462,11 +1515,11 @@ int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang
     }
     if (!zp.film) {
       PhaseTimer pt(c, RSX_PHASE_FFTX, s);
-      RSX_CK(planes_x_fft<R>(c, zp, 3LL * nk, xm, s), "x-FFT kernel");
+      RSX_CK(planes_x_fft<R>(c, c->p, zp, 3LL * nk, xm, s), "x-FFT kernel");
     }
     if (g.ny > 1) {
       PhaseTimer pt(c, RSX_PHASE_FFTY, s);
-      RSX_CK(planes_y_fft<R>(c, zp, 3LL * nk, runs, s), "y-FFT kernel");
+      RSX_CK(planes_y_fft<R>(c, c->p, zp, 3LL * nk, runs, s), "y-FFT kernel");
     }
     for (int i0 = 0; i0 < nk; i0 += c->n_img) {
       const int ni = nk - i0 < c->n_img ? nk - i0 : c->n_img;

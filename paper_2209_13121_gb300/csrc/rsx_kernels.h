@@ -316,6 +316,19 @@ template <typename R>
 cudaError_t launch_pol_planes(const void* M, const void* nt, const void* dir, long long npix,
                               int nz, const PolParams<R>& pp, const AngleBatch<R>& ang, void* out,
                               int kb, int ns, const void* twz, cudaStream_t s);
+// The linearity path on the planes: N_t's five entries (from M, or nt),
+// z-transformed, the ns kept bins of entry e at out + (e * ns + s) * npix
+// (lin_planes_fits: nz = 8 .. 64 a power of two, 128 in FP32), and, from the
+// transformed planes, the bins ([5][2][npix]) its images combine;
+// dc = -(c-1)/(4 pi) N.
+bool lin_planes_fits(int precision, int nz);
+template <typename R>
+cudaError_t launch_lin_planes(const void* M, const void* nt, long long npix, int nz,
+                              const PolParams<R>& pp, void* out, int kb, int ns, const void* twz,
+                              cudaStream_t s);
+template <typename R>
+cudaError_t launch_bins5_planes(const void* planes, int nx, int ny, int nz, int kb, int ns,
+                                const Geo<R>* geo, double dc, void* bins, cudaStream_t s);
 // The lateral transforms of the planes for tuned sizes (FP32), in place.
 // YRuns: per 16-column group cg < n the run of planes its pixels read:
 // first[cg] .. first[cg] + (start[cg + 1] - start[cg]) - 1 (start: prefix

@@ -11,6 +11,7 @@
 // The rotation and average follow as on the other paths.  The 3-D DFT is
 // separable, so the values are the full transform's up to rounding order.
 #include <cuda.h>  // CUtensorMap (the type only)
+#include <string.h>
 
 #include "rsx_device.cuh"
 #include "rsx_kernels.h"
@@ -255,6 +256,8 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
 // nz = 16, where the folded sums above took 160 at 64 % issue (1024 x 1024 x 16,
 // c = 3, two energies of 91 angles: the pass 19.0 ms, 13.4 so; Algorithm 2 at
 // 1024 x 1024 x 32, 37 angles: 16.5 and 13.2).
+// NF = 3: the fields of p of every angle.  NF = 5: the linearity path's five
+// entries of N_t (xx, xy, yy, xz, yz, the constant left out), once.
 template <typename R, int Q> struct PlFft {
   static constexpr int PX = kPlThreads / Q;
   // u's stride between s1: padded where a half-warp spans two of them
@@ -263,7 +266,7 @@ template <typename R, int Q> struct PlFft {
   static constexpr int A = sizeof(R) == 8 ? (Q >= 8 ? 2 : 1) : Q >= 16 ? 4 : Q == 8 ? 2 : 1;
 };
 
-template <typename R, int SRC, int Q>
+template <typename R, int SRC, int Q, int NF>
 __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_planes_fft(
     const typename RT<R>::V4* __restrict__ M, const typename RT<R>::C* __restrict__ nt,
     const R* __restrict__ dir, long long npix, int kb, int ns,
@@ -271,9 +274,9 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
     typename RT<R>::C* __restrict__ out, const typename RT<R>::C* __restrict__ twz) {
   using C = typename RT<R>::C;
   using P = PlFft<R, Q>;
-  constexpr int NZ = 4 * Q, PX = P::PX, KS = P::KS, A = P::A;
+  constexpr int NZ = 4 * Q, PX = P::PX, KS = P::KS, A = NF == 3 ? P::A : 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);  // [A][3][4][KS]
+  C* buf = reinterpret_cast<C*>(smem_raw);  // [A][NF][4][KS]
   const int t = threadIdx.x, px = t % PX, n2 = t / PX;
   const long long N = npix * NZ;
   const long long pix0 = (long long)blockIdx.x * PX;
@@ -330,20 +333,32 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
     }
   }
   const bool literal = pp.literal != 0;
-  const size_t fstride = (size_t)ns * npix, kstride = 3 * fstride;
+  const size_t fstride = (size_t)ns * npix;
   const int rot = kb & 3;  // s1 = 0 takes output kb mod 4 of the 4-point transform
-  for (int a0 = 0; a0 < ang.n; a0 += A) {
-    const int na = ang.n - a0 < A ? ang.n - a0 : A;
+  const int nang = NF == 3 ? ang.n : 1;
+  for (int a0 = 0; a0 < nang; a0 += A) {
+    const int na = nang - a0 < A ? nang - a0 : A;
     if (a0 > 0) __syncthreads();  // the previous step's reads are done
     for (int a = 0; a < na; ++a) {
-      const R ce = ang.ce[a0 + a], se = ang.se[a0 + a];
-      C p[4][3];
+      C p[4][NF];
+      if constexpr (NF == 3) {
+        const R ce = ang.ce[a0 + a], se = ang.se[a0 + a];
 #pragma unroll
-      for (int n1 = 0; n1 < 4; ++n1)
-        p_from_tacc(acc[n1].aw, acc[n1].as[1], acc[n1].t, ce, se, literal, p[n1]);
-      C* b = buf + a * 3 * 4 * KS + t;
+        for (int n1 = 0; n1 < 4; ++n1)
+          p_from_tacc(acc[n1].aw, acc[n1].as[1], acc[n1].t, ce, se, literal, p[n1]);
+      } else {
 #pragma unroll
-      for (int f = 0; f < 3; ++f) {
+        for (int n1 = 0; n1 < 4; ++n1)
+#pragma unroll
+          for (int f = 0; f < NF; ++f) {
+            const bool diag = f == 0 || f == 2;
+            p[n1][f] = RT<R>::mk(acc[n1].t[f][0] + (diag ? acc[n1].aw : R(0)),
+                                 acc[n1].t[f][1] + (diag ? acc[n1].as[1] : R(0)));
+          }
+      }
+      C* b = buf + a * NF * 4 * KS + t;
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
         dft4(p[0][f], p[1][f], p[2][f], p[3][f]);
         // output k1 goes to s1 = (k1 - kb) mod 4 (uniform)
 #pragma unroll
@@ -357,15 +372,15 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
       }
     }
     __syncthreads();
-    const int items = na * 12 * PX;
+    const int items = na * 4 * NF * PX;
     for (int it = t; it < items; it += kPlThreads) {
-      const int q = it % PX, r = it / PX, s1 = r & 3, af = r >> 2;  // af = 3 a + f
+      const int q = it % PX, r = it / PX, s1 = r & 3, af = r >> 2;  // af = NF a + f
       if (q >= npx) continue;
       const C* b = buf + r * KS + q;
       C v[Q];
 #pragma unroll
       for (int n = 0; n < Q; ++n) v[n] = b[n * PX];
-      C* o = out + (size_t)(3 * a0 + af) * fstride + (size_t)s1 * npix + pix0 + q;
+      C* o = out + (size_t)(NF * a0 + af) * fstride + (size_t)s1 * npix + pix0 + q;
       const int mine = (ns - s1 + 3) >> 2;  // kept s2 of this s1
       if constexpr (Q == 32) {
         if (ns <= 64) {
@@ -849,14 +864,39 @@ cudaError_t pol_planes_sb(const void* M, const void* nt, const void* dir, long l
   return cudaGetLastError();
 }
 
-template <typename R, int SRC, int Q>
+// The linearity path's bins ([5][2][npix]) from the transformed planes of
+// N_t's entries: per pixel its two planes of each, the constant returned to
+// xx and yy at q = 0.
+template <typename R>
+__global__ void __launch_bounds__(256) k_bins5_planes(const typename RT<R>::C* __restrict__ planes,
+                                                      long long npix, int nz, int kb, int ns,
+                                                      const Geo<R>* __restrict__ geo, R dc,
+                                                      typename RT<R>::C* __restrict__ bins) {
+  const long long pix = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (pix >= npix) return;
+  const Geo<R> g = geo[pix];
+  if (g.b0 < 0) return;  // off the sphere: the bins are not read
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    const int bin = b ? g.b1 : g.b0;
+    const int s = bin < kb ? bin - kb + nz : bin - kb;
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      typename RT<R>::C v = planes[((size_t)q * ns + s) * npix + pix];
+      if (pix == 0 && bin == 0 && (q == 0 || q == 2)) v.x += dc;
+      bins[(size_t)(2 * q + b) * npix + pix] = v;
+    }
+  }
+}
+
+template <typename R, int SRC, int Q, int NF = 3>
 cudaError_t pol_planes_fft(const void* M, const void* nt, const void* dir, long long npix,
                            const PolParams<R>& pp, const AngleBatch<R>& ang, void* out, int kb,
                            int ns, const void* twz, cudaStream_t s) {
   using C = typename RT<R>::C;
   using P = PlFft<R, Q>;
-  const size_t smem = (size_t)P::A * 12 * P::KS * sizeof(C);
-  auto kern = k_pol_planes_fft<R, SRC, Q>;
+  const size_t smem = (size_t)(NF == 3 ? P::A : 1) * 4 * NF * P::KS * sizeof(C);
+  auto kern = k_pol_planes_fft<R, SRC, Q, NF>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)((npix + P::PX - 1) / P::PX), kPlThreads, smem, s>>>(
@@ -892,6 +932,43 @@ cudaError_t pol_planes_src(const void* M, const void* nt, const void* dir, long 
 #undef RSX_PL
 }
 }  // namespace
+
+bool lin_planes_fits(int precision, int nz) {
+  return nz == 8 || nz == 16 || nz == 32 || nz == 64 || (nz == 128 && precision == 32);
+}
+
+template <typename R>
+cudaError_t launch_lin_planes(const void* M, const void* nt, long long npix, int nz,
+                              const PolParams<R>& pp, void* out, int kb, int ns, const void* twz,
+                              cudaStream_t s) {
+  if (!lin_planes_fits(8 * (int)sizeof(R), nz) || ns < 1 || ns > nz || kb < 0 || kb >= nz)
+    return cudaErrorInvalidValue;
+  AngleBatch<R> none;
+  memset(&none, 0, sizeof(none));
+#define RSX_LIN(Q)                                                                                \
+  return nt ? pol_planes_fft<R, 1, Q, 5>(M, nt, nullptr, npix, pp, none, out, kb, ns, twz, s)     \
+            : pol_planes_fft<R, 0, Q, 5>(M, nt, nullptr, npix, pp, none, out, kb, ns, twz, s);
+  switch (nz) {
+    case 8: RSX_LIN(2)
+    case 16: RSX_LIN(4)
+    case 32: RSX_LIN(8)
+    case 64: RSX_LIN(16)
+    default: break;
+  }
+  if constexpr (sizeof(R) == 4) { RSX_LIN(32) }
+#undef RSX_LIN
+  return cudaErrorInvalidValue;
+}
+
+template <typename R>
+cudaError_t launch_bins5_planes(const void* planes, int nx, int ny, int nz, int kb, int ns,
+                                const Geo<R>* geo, double dc, void* bins, cudaStream_t s) {
+  using C = typename RT<R>::C;
+  const long long npix = (long long)nx * ny;
+  k_bins5_planes<R><<<(unsigned)((npix + 255) / 256), 256, 0, s>>>((const C*)planes, npix, nz, kb, ns,
+                                                                   geo, (R)dc, (C*)bins);
+  return cudaGetLastError();
+}
 
 bool pol_planes_fits(int precision, int nz, int kb, int ns) {
   if (nz < 1 || nz > kMaxPlanesNz || ns < 1 || ns > nz) return false;
@@ -1008,6 +1085,11 @@ cudaError_t launch_x_planes(void* data, int nx, int ny, int ns, long long nfield
   template cudaError_t launch_pol_planes<R>(const void*, const void*, const void*, long long, int, \
                                             const PolParams<R>&, const AngleBatch<R>&, void*, int, \
                                             int, const void*, cudaStream_t);                      \
+  template cudaError_t launch_lin_planes<R>(const void*, const void*, long long, int,             \
+                                            const PolParams<R>&, void*, int, int, const void*,    \
+                                            cudaStream_t);                                        \
+  template cudaError_t launch_bins5_planes<R>(const void*, int, int, int, int, int,               \
+                                              const Geo<R>*, double, void*, cudaStream_t);        \
   template cudaError_t launch_plane_images<R>(const void*, int, int, int, int, int,               \
                                               const Geo<R>*, const ImageDc<R>&, void*,            \
                                               cudaStream_t);

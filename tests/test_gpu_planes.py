@@ -73,6 +73,46 @@ def test_edges_match_oracle_and_the_general_path(rsx, shape, c, voxel, E, prec):
             _close(ctx.run(rotation=False)[0], img.cpu().numpy(), prec, r=1.5)
 
 
+# stacks the linearity path's z-first pass takes and their neighbours, the
+# tuned x and y passes, both sources of N_t
+LIN = [((7, 9, 10), 64), ((8, 12, 20), 32), ((16, 16, 32), 64), ((32, 10, 9), 32), ((64, 8, 8), 64),
+       ((64, 8, 12), 32), ((128, 6, 10), 32), ((128, 4, 6), 64), ((16, 512, 16), 32),
+       ((16, 1024, 16), 32), ((16, 4, 1024), 32), ((16, 3, 2048), 32)]
+
+
+@pytest.mark.parametrize("shape,prec", LIN, ids=["x".join(map(str, s)) + f"f{p}" for s, p in LIN])
+def test_linearity_path_planes(rsx, shape, prec):
+    nz, ny, nx = shape
+    E = [285.0, 300.0]
+    M = synth.morphology_random(shape, 2, seed=17, dtype=np.float32 if prec == 32 else np.float64)
+    K = synth.optical_constants(E, 2, seed=18)
+    for dev, frame in ((True, 0), (False, 1)):
+        ref = O.run_alg1(M, K, E, 5.0, angles_deg=(0.0, 40.0, 160.0),
+                         uT_mode="lab" if frame else "literal")
+        with rsx.Context(nx, ny, nz, 2, 5.0, precision=prec, algorithm=3, frame=frame) as ctx:
+            ctx.set_morphology(torch.from_numpy(M).cuda() if dev else M)
+            ctx.set_optical_constants(E, K)
+            _close(ctx.run((0.0, 40.0, 160.0)), ref, prec)
+
+
+FILMS = [(512, 512), (512, 1024), (1024, 512), (2048, 512), (512, 2048), (512, 2000)]
+
+
+@pytest.mark.parametrize("ny,nx", FILMS, ids=[f"{a}x{b}" for a, b in FILMS])
+def test_films_match_oracle(rsx, ny, nx):
+    """One slice: p x-transformed by the multi-angle pass straight into the
+    planes (rows of 512, 1024, 2048 points), each tuned column length, the
+    2048-row columns' own kernel, a partial batch of angles; and a row length
+    the multi-angle pass does not take."""
+    M = synth.morphology_random((1, ny, nx), 2, seed=19, dtype=np.float32)
+    K = synth.optical_constants([285.0], 2, seed=20)
+    ref = O.run_alg1(M, K, [285.0], 5.0, angles_deg=(0.0, 45.0, 180.0))
+    with rsx.Context(nx, ny, 1, 2, 5.0) as ctx:
+        ctx.set_morphology(torch.from_numpy(M).cuda())
+        ctx.set_optical_constants([285.0], K)
+        _close(ctx.run((0.0, 45.0, 180.0)), ref, 32)
+
+
 def test_more_angles_than_one_batch_holds(rsx):
     """181 angles in three or more batches of at most 64; two energies."""
     shape, c, E = (6, 12, 20), 2, [275.0, 300.0]
