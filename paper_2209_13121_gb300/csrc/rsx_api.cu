@@ -1405,12 +1405,10 @@ int run_energy_angles_batched(rsx_context* c, int ie, double start, double inc, 
     const int nk = nang - a0 < kx ? nang - a0 : kx;
     rsx::XAngles ang;
     memset(&ang, 0, sizeof(ang));
-    ang.n = nk;
     double alpha[rsx::kMaxXAngles];
     for (int k = 0; k < nk; ++k) {
       alpha[k] = rotation ? (start + inc * (a0 + k)) * (kPi / 180.0) : 0.0;
-      ang.ce[k] = (float)cos(alpha[k]);
-      ang.se[k] = (float)sin(alpha[k]);
+      rsx::add_angle(ang, alpha[k]);
     }
     {
       PhaseTimer pt(c, RSX_PHASE_POL_FFTX, s);
@@ -1491,9 +1489,7 @@ int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang
         if (zp.zfft || zp.film) {
           rsx::XAngles ang;
           memset(&ang, 0, sizeof(ang));
-          ang.n = nk;
-          memcpy(ang.ce, ab.ce, nk * sizeof(float));
-          memcpy(ang.se, ab.se, nk * sizeof(float));
+          for (int k = 0; k < nk; ++k) rsx::add_angle(ang, alpha[k]);
           const long long fstride = (long long)zp.ns * c->npix;
           e = zp.film
                   ? rsx::launch_pol_fft4s_tma_multi(

@@ -726,13 +726,11 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_fft4s_tma_mul
     fence_proxy_async();
   }
   for (int i = t; i < NTW; i += blockDim.x) tw4[i] = tw4_g[i];
-  __shared__ float ang_ce[KMAX], ang_se[KMAX];  // indexed by a run-time angle
+  __shared__ float4 ang_s[KMAX];  // cos a, sin a, cos 2a, sin 2a, indexed by a run-time angle
   if (t == 0) {
 #pragma unroll
-    for (int i = 0; i < KMAX; ++i) {  // constant indices: the parameters stay in place
-      ang_ce[i] = ang.ce[i];
-      ang_se[i] = ang.se[i];
-    }
+    for (int i = 0; i < KMAX; ++i)  // constant indices: the parameters stay in place
+      ang_s[i] = make_float4(ang.ce[i], ang.se[i], ang.c2[i], ang.s2[i]);
   }
   __syncthreads();
   const int nk = ang.n;
@@ -796,19 +794,9 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_fft4s_tma_mul
           for (int sl = 0; sl < SL; ++sl)
             tacc_add(acc[sl], cur[sl].x, cur[sl].y, cur[sl].z, cur[sl].w, pp, j);
         }
-        // (sum v^2 - 1) first, then the small optical part (FP32 accuracy);
-        // everything divided by 4 pi once per voxel
-        const float inv = float(1.0 / kFourPi);
+        PTen<float> pt10[SL];
 #pragma unroll
-        for (int sl = 0; sl < SL; ++sl) {
-          acc[sl].aw = ((acc[sl].aw - 1.f) + acc[sl].as[0]) * inv;
-          acc[sl].as[1] *= inv;
-#pragma unroll
-          for (int q = 0; q < 5; ++q) {
-            acc[sl].t[q][0] *= inv;
-            acc[sl].t[q][1] *= inv;
-          }
-        }
+        for (int sl = 0; sl < SL; ++sl) pten_of(pt10[sl], acc[sl], pp.literal != 0);
         // row buffer u = rr * nk + k holds angle k of row rr; with H > 1 all
         // nk buffers of the row stay open across its segments (nk <= NPB)
         for (int k = 0; k < nk; ++k) {
@@ -816,12 +804,12 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_fft4s_tma_mul
           if (h == 0 && u >= NPB) named_bar_sync(1 + NPB + i, NB);  // previous use done
           if (!failed) {
             C* Pi = P + i * 3 * FS + h * 1056;
-            const float ce = ang_ce[k], se = ang_se[k];
+            const float4 an = ang_s[k];
 #pragma unroll
             for (int sl = 0; sl < SL; ++sl) {
               const int e = pt + sl * TP;
               C out[3];
-              p_from_tacc(acc[sl].aw, acc[sl].as[1], acc[sl].t, ce, se, pp.literal != 0, out);
+              p_from_pten(pt10[sl], an.x, an.y, an.z, an.w, pp.literal != 0, out);
               Pi[e] = out[0];
               Pi[FS + e] = out[1];
               Pi[2 * FS + e] = out[2];
@@ -894,7 +882,8 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_fft4s_tma_mul
 //            as it has been read.  (The whole transform, written back to
 //            shared memory and copied out bin by bin: 59.8 ms per energy
 //            at 1024 x 1024 x 128, 91 angles, 53.4 so; 2048 x 2048 x 64
-//            121.7 and 109.0.)
+//            121.7 and 109.0; with the ten-real form of the sums, PTen,
+//            48.9 and 99.0.)
 // zf_pos(a, b) = 32 a + b, for R = 4 with b xor a (the low bits swizzled by
 // a); with LS = 130 (R = 4) or nz + 1 that keeps the polarisation stores and
 // stage 2's loads free of shared-memory bank conflicts (checked per
@@ -967,13 +956,11 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_zfft_multi(
   }
   for (int i = t; i < 32 * R; i += blockDim.x)
     twt[i] = twz_g[((i / R) * (kb + i % R)) & (NZ - 1)];
-  __shared__ float ang_ce[KMAX], ang_se[KMAX];  // indexed by a run-time angle
+  __shared__ float4 ang_s[KMAX];  // cos a, sin a, cos 2a, sin 2a, indexed by a run-time angle
   if (t == 0) {
 #pragma unroll
-    for (int i = 0; i < KMAX; ++i) {  // constant indices: the parameters stay in place
-      ang_ce[i] = ang.ce[i];
-      ang_se[i] = ang.se[i];
-    }
+    for (int i = 0; i < KMAX; ++i)  // constant indices: the parameters stay in place
+      ang_s[i] = make_float4(ang.ce[i], ang.se[i], ang.c2[i], ang.s2[i]);
   }
   __syncthreads();
   const int nk = ang.n;
@@ -1006,8 +993,9 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_zfft_multi(
 
   if (kind == 0) {  // polarisation warps; pt: this thread's index among them
     const int pt = ridx * 32 + lane;
-    bool failed = false;
-    int slot = 0, ph = 0;
+    const bool literal = pp.literal != 0;
+    bool failed = false, wrapped = false;
+    int slot = 0, ph = 0, i = 0;  // row buffer u is slot i = u mod NPB
     for (int rr = 0; rr < (int)nmine; ++rr) {
       TAcc<float> acc[SL];
 #pragma unroll
@@ -1033,27 +1021,18 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_zfft_multi(
         for (int sl = 0; sl < SL; ++sl)
           tacc_add(acc[sl], cur[sl].x, cur[sl].y, cur[sl].z, cur[sl].w, pp, j);
       }
-      const float inv = float(1.0 / kFourPi);
+      PTen<float> pt10[SL];
 #pragma unroll
-      for (int sl = 0; sl < SL; ++sl) {
-        acc[sl].aw = ((acc[sl].aw - 1.f) + acc[sl].as[0]) * inv;
-        acc[sl].as[1] *= inv;
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-          acc[sl].t[q][0] *= inv;
-          acc[sl].t[q][1] *= inv;
-        }
-      }
+      for (int sl = 0; sl < SL; ++sl) pten_of(pt10[sl], acc[sl], literal);
       for (int k = 0; k < nk; ++k) {
-        const int u = rr * nk + k, i = u % NPB;
-        if (u >= NPB) named_bar_sync(1 + NPB + i, NB);  // previous use done
+        if (wrapped) named_bar_sync(1 + NPB + i, NB);  // previous use done
         if (!failed) {
           C* Pi = P + i * 3 * FS;
-          const float ce = ang_ce[k], se = ang_se[k];
+          const float4 an = ang_s[k];
           C o[SL][3];
 #pragma unroll
           for (int sl = 0; sl < SL; ++sl)
-            p_from_tacc(acc[sl].aw, acc[sl].as[1], acc[sl].t, ce, se, pp.literal != 0, o[sl]);
+            p_from_pten(pt10[sl], an.x, an.y, an.z, an.w, literal, o[sl]);
           // stage 1 of the z transform: sl = g + (4 / R) n1 holds n1 of one n2
 #pragma unroll
           for (int f = 0; f < 3; ++f) {
@@ -1075,6 +1054,7 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_zfft_multi(
           }
         }
         named_bar_arrive(1 + i, NB);
+        if (++i == NPB) i = 0, wrapped = true;
       }
     }
     return;
@@ -1092,8 +1072,9 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_zfft_multi(
   for (int c = 0; c < R; ++c) at[c] = px * LS + zf_pos<R>(k1, c);
   const C* tw = twt + s1;
   const int mine = (ns - s1 + R - 1) / R, most = (ns + R - 1) / R;  // outputs of this lane, of any
+  int i = fg % NPB, rr = 0, k = fg;  // buffer u: slot i, tile rr, angle k
   for (int u = fg; u < U; u += FG) {
-    const int i = u % NPB;
+    for (; k >= nk; k -= nk) ++rr;
     named_bar_sync(1 + i, NB);
     const bool go = *abort_flag == 0;
     C v[32];
@@ -1108,7 +1089,6 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_zfft_multi(
     if (u + NPB < U) named_bar_arrive(1 + NPB + i, NB);
     if (go) {
       // tiles follow the pixels: tile XW is its first pixel y nx + x
-      const int rr = u / nk, k = u - rr * nk;
       C* o = out + (size_t)k * kstride + (size_t)f * fstride + (size_t)s1 * npix +
              (size_t)((blockIdx.x + rr * gridDim.x) * XW + px);
       if constexpr (ALL) {
@@ -1123,6 +1103,8 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_zfft_multi(
         });
       }
     }
+    k += FG;
+    if ((i += FG) >= NPB) i -= NPB;
   }
 }
 

@@ -42,7 +42,8 @@ constexpr unsigned kWaitPolls = 1u << 22;
 constexpr int kMaxAngleBatch = 64;
 template <typename R> struct AngleBatch {
   int n;
-  R ce[kMaxAngleBatch], se[kMaxAngleBatch];
+  R ce[kMaxAngleBatch], se[kMaxAngleBatch];  // cos a, sin a
+  R c2[kMaxAngleBatch], s2[kMaxAngleBatch];  // cos 2a, sin 2a
   long long cxx[kMaxAngleBatch], cxy[kMaxAngleBatch], cyx[kMaxAngleBatch], cyy[kMaxAngleBatch];
 };
 
@@ -63,6 +64,8 @@ inline void add_angle(AngleBatch<R>& ab, double alpha, int nx, int ny) {
   const int a = ab.n++;
   ab.ce[a] = (R)cos(alpha);
   ab.se[a] = (R)sin(alpha);
+  ab.c2[a] = (R)cos(2.0 * alpha);
+  ab.s2[a] = (R)sin(2.0 * alpha);
   ab.cxx[a] = c[0];
   ab.cxy[a] = c[1];
   ab.cyx[a] = c[2];
@@ -174,9 +177,17 @@ cudaError_t launch_pol_fft4s_tma(const void* M, int nx, int ny, int nz, const Po
 // up to 8) or z-first pass: cos and sin of each, n of them in use.
 constexpr int kMaxXAngles = 32;
 struct XAngles {
-  float ce[kMaxXAngles], se[kMaxXAngles];
+  float ce[kMaxXAngles], se[kMaxXAngles];  // cos a, sin a
+  float c2[kMaxXAngles], s2[kMaxXAngles];  // cos 2a, sin 2a
   int n;
 };
+inline void add_angle(XAngles& xa, double alpha) {
+  xa.ce[xa.n] = (float)cos(alpha);
+  xa.se[xa.n] = (float)sin(alpha);
+  xa.c2[xa.n] = (float)cos(2.0 * alpha);
+  xa.s2[xa.n] = (float)sin(2.0 * alpha);
+  ++xa.n;
+}
 // The Algorithm-1 x pass for ang.n angles per read of the morphology (FP32,
 // nx = 1024 or 512, M 16-byte aligned): angle k's three x-transformed fields
 // go to p + k * pstride (complex elements; pstride >= 3 N).  pp supplies the

@@ -88,7 +88,8 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
 
   // this thread's voxels: the sums of Eq. (polarization), divided by 4 pi.
   // EVEN: z, z + L, L - z, nz - z of one pixel; else z, nz - z of two
-  TAcc<R> acc[kPlVoxels];
+  const bool literal = pp.literal != 0;
+  PTen<R> ten[kPlVoxels];
   int at[2];     // shared-memory place of each fold (field 0, angle 0); -1: none
   bool two[2];   // its second half exists (z is not alone)
 #pragma unroll
@@ -99,21 +100,25 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
     two[sl] = in && z > 0 && 2 * z != L;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      TAcc<R>& a = acc[2 * sl + h];
-      tacc_zero(a);
+      pten_zero(ten[2 * sl + h]);
       // EVEN: slot 0 holds z and z + L, slot 1 L - z and nz - z
       const int zv = EVEN ? (sl ? L - z : z) + (h ? L : 0) : h ? nz - z : z;
       const bool have = EVEN ? (sl ? two[sl] : in) : h ? two[sl] : in;
       if (!have) continue;
       const size_t i = (size_t)(EVEN && sl && h ? nz - z : zv) * npix + pix0 + px;
       if constexpr (SRC == 1) {
+        const R none[2] = {R(0), R(0)};
+        R tt[5][2];
 #pragma unroll
         for (int e = 0; e < 5; ++e) {
           const C v = ld_stream(nt + (size_t)e * N + i);
-          a.t[e][0] = v.x;
-          a.t[e][1] = v.y;
+          tt[e][0] = v.x;
+          tt[e][1] = v.y;
         }
+        pten_of(ten[2 * sl + h], none, tt, literal);
       } else {
+        TAcc<R> a;
+        tacc_zero(a);
         for (int j = 0; j < pp.c; ++j) {
           const typename RT<R>::V4 m = ld_stream(M + (size_t)j * N + i);
           if (dir) {
@@ -123,19 +128,11 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
             tacc_add(a, (R)m.x, (R)m.y, (R)m.z, (R)m.w, pp, j);
           }
         }
-        const R inv = R(1.0 / kFourPi);
-        a.aw = ((a.aw - R(1)) + a.as[0]) * inv;
-        a.as[1] *= inv;
-#pragma unroll
-        for (int e = 0; e < 5; ++e) {
-          a.t[e][0] *= inv;
-          a.t[e][1] *= inv;
-        }
+        pten_of(ten[2 * sl + h], a, literal);
       }
     }
   }
 
-  const bool literal = pp.literal != 0;
   const size_t fstride = (size_t)ns * npix, kstride = 3 * fstride;
   if (nz == 1) {  // no z transform: the pixel's p is its plane
     for (int k = 0; k < ang.n; ++k) {
@@ -143,8 +140,7 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
       for (int sl = 0; sl < 2; ++sl) {
         if (at[sl] < 0) continue;
         C p[3];
-        p_from_tacc(acc[2 * sl].aw, acc[2 * sl].as[1], acc[2 * sl].t, ang.ce[k], ang.se[k], literal,
-                    p);
+        p_from_pten(ten[2 * sl], ang.ce[k], ang.se[k], ang.c2[k], ang.s2[k], literal, p);
         C* o = out + k * kstride + pix0 + at[sl];
         o[0] = p[0];
         o[fstride] = p[1];
@@ -159,14 +155,14 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
     const int na = ang.n - a0 < A ? ang.n - a0 : A;
     if (a0 > 0) __syncthreads();  // the previous step's reads are done
     for (int a = 0; a < na; ++a) {
-      const R ce = ang.ce[a0 + a], se = ang.se[a0 + a];
+      const R ce = ang.ce[a0 + a], se = ang.se[a0 + a], c2 = ang.c2[a0 + a], s2 = ang.s2[a0 + a];
       F* ba = buf + (size_t)a * NP * H * 3 * PX;
       if constexpr (EVEN) {
         if (at[0] < 0) continue;
         C p[4][3];
 #pragma unroll
         for (int v = 0; v < 4; ++v)
-          p_from_tacc(acc[v].aw, acc[v].as[1], acc[v].t, ce, se, literal, p[v]);
+          p_from_pten(ten[v], ce, se, c2, s2, literal, p[v]);
 #pragma unroll
         for (int f = 0; f < 3; ++f) {  // (a voxel that does not exist has p = 0)
           const C a1 = cadd(p[0][f], p[1][f]), b1 = csub(p[0][f], p[1][f]);
@@ -184,9 +180,8 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
         for (int sl = 0; sl < 2; ++sl) {
           if (at[sl] < 0) continue;
           C p[3], q[3];
-          p_from_tacc(acc[2 * sl].aw, acc[2 * sl].as[1], acc[2 * sl].t, ce, se, literal, p);
-          p_from_tacc(acc[2 * sl + 1].aw, acc[2 * sl + 1].as[1], acc[2 * sl + 1].t, ce, se, literal,
-                      q);
+          p_from_pten(ten[2 * sl], ce, se, c2, s2, literal, p);
+          p_from_pten(ten[2 * sl + 1], ce, se, c2, s2, literal, q);
 #pragma unroll
           for (int f = 0; f < 3; ++f) {
             F v;
@@ -255,7 +250,8 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
 // the kept ones are evaluated).  ~75 instructions per voxel and angle at
 // nz = 16, where the folded sums above took 160 at 64 % issue (1024 x 1024 x 16,
 // c = 3, two energies of 91 angles: the pass 19.0 ms, 13.4 so; Algorithm 2 at
-// 1024 x 1024 x 32, 37 angles: 16.5 and 13.2).
+// 1024 x 1024 x 32, 37 angles: 16.5 and 13.2; with PTen and three blocks per
+// SM 12.0 and 11.5).
 // NF = 3: the fields of p of every angle.  NF = 5: the linearity path's five
 // entries of N_t (xx, xy, yy, xz, yz, the constant left out), once.
 template <typename R, int Q> struct PlFft {
@@ -267,7 +263,7 @@ template <typename R, int Q> struct PlFft {
 };
 
 template <typename R, int SRC, int Q, int NF>
-__global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_planes_fft(
+__global__ void __launch_bounds__(kPlThreads, sizeof(R) == 8 ? 1 : Q <= 8 && NF == 3 ? 3 : 2) k_pol_planes_fft(
     const typename RT<R>::V4* __restrict__ M, const typename RT<R>::C* __restrict__ nt,
     const R* __restrict__ dir, long long npix, int kb, int ns,
     const __grid_constant__ PolParams<R> pp, const __grid_constant__ AngleBatch<R> ang,
@@ -281,28 +277,34 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
   const long long N = npix * NZ;
   const long long pix0 = (long long)blockIdx.x * PX;
   const int npx = npix - pix0 < PX ? (int)(npix - pix0) : PX;
-  TAcc<R> acc[4];
+  // NF = 5: the lab frame's terms are N_t's entries themselves
+  const bool literal = NF == 3 && pp.literal != 0;
+  PTen<R> ten[4];
   C w[4];
 #pragma unroll
   for (int n1 = 0; n1 < 4; ++n1) {
     w[n1] = twz[(n2 * (kb + n1)) % NZ];
-    TAcc<R>& a = acc[n1];
-    tacc_zero(a);
-    const size_t i = (size_t)(n2 + Q * n1) * npix + pix0 + px;
-    if (px < npx) {
-      if constexpr (SRC == 1) {
+    pten_zero(ten[n1]);
+  }
+  if (px < npx) {
+    const size_t i = (size_t)n2 * npix + pix0 + px, step = (size_t)Q * npix;
+    if constexpr (SRC == 1) {
+      const R none[2] = {R(0), R(0)};
+#pragma unroll
+      for (int n1 = 0; n1 < 4; ++n1) {
+        R tt[5][2];
 #pragma unroll
         for (int e = 0; e < 5; ++e) {
-          const C v = ld_stream(nt + (size_t)e * N + i);
-          a.t[e][0] = v.x;
-          a.t[e][1] = v.y;
+          const C v = ld_stream(nt + (size_t)e * N + i + n1 * step);
+          tt[e][0] = v.x;
+          tt[e][1] = v.y;
         }
+        pten_of(ten[n1], none, tt, literal);
       }
-    }
-  }
-  if constexpr (SRC == 0) {
-    if (px < npx) {
-      const size_t i = (size_t)n2 * npix + pix0 + px, step = (size_t)Q * npix;
+    } else {
+      TAcc<R> acc[4];
+#pragma unroll
+      for (int n1 = 0; n1 < 4; ++n1) tacc_zero(acc[n1]);
       for (int j = 0; j < pp.c; ++j) {
         const typename RT<R>::V4* Mj = M + (size_t)j * N + i;
         typename RT<R>::V4 m[4];
@@ -318,21 +320,10 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
             tacc_add(acc[n1], (R)m[n1].x, (R)m[n1].y, (R)m[n1].z, (R)m[n1].w, pp, j);
         }
       }
-      const R inv = R(1.0 / kFourPi);
 #pragma unroll
-      for (int n1 = 0; n1 < 4; ++n1) {
-        TAcc<R>& a = acc[n1];
-        a.aw = ((a.aw - R(1)) + a.as[0]) * inv;
-        a.as[1] *= inv;
-#pragma unroll
-        for (int e = 0; e < 5; ++e) {
-          a.t[e][0] *= inv;
-          a.t[e][1] *= inv;
-        }
-      }
+      for (int n1 = 0; n1 < 4; ++n1) pten_of(ten[n1], acc[n1], literal);
     }
   }
-  const bool literal = pp.literal != 0;
   const size_t fstride = (size_t)ns * npix;
   const int rot = kb & 3;  // s1 = 0 takes output kb mod 4 of the 4-point transform
   const int nang = NF == 3 ? ang.n : 1;
@@ -342,19 +333,19 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
     for (int a = 0; a < na; ++a) {
       C p[4][NF];
       if constexpr (NF == 3) {
-        const R ce = ang.ce[a0 + a], se = ang.se[a0 + a];
+        const R ce = ang.ce[a0 + a], se = ang.se[a0 + a], c2 = ang.c2[a0 + a], s2 = ang.s2[a0 + a];
 #pragma unroll
-        for (int n1 = 0; n1 < 4; ++n1)
-          p_from_tacc(acc[n1].aw, acc[n1].as[1], acc[n1].t, ce, se, literal, p[n1]);
+        for (int n1 = 0; n1 < 4; ++n1) p_from_pten(ten[n1], ce, se, c2, s2, literal, p[n1]);
       } else {
 #pragma unroll
-        for (int n1 = 0; n1 < 4; ++n1)
-#pragma unroll
-          for (int f = 0; f < NF; ++f) {
-            const bool diag = f == 0 || f == 2;
-            p[n1][f] = RT<R>::mk(acc[n1].t[f][0] + (diag ? acc[n1].aw : R(0)),
-                                 acc[n1].t[f][1] + (diag ? acc[n1].as[1] : R(0)));
-          }
+        for (int n1 = 0; n1 < 4; ++n1) {
+          const PTen<R>& q = ten[n1];
+          p[n1][0] = RT<R>::mk(q.a[0], q.a[1]);
+          p[n1][1] = RT<R>::mk(q.xy[0], q.xy[1]);
+          p[n1][2] = RT<R>::mk(q.b[0], q.b[1]);
+          p[n1][NF - 2] = RT<R>::mk(q.xz[0], q.xz[1]);
+          p[n1][NF - 1] = RT<R>::mk(q.yz[0], q.yz[1]);
+        }
       }
       C* b = buf + a * NF * 4 * KS + t;
 #pragma unroll

@@ -86,28 +86,64 @@ __device__ __forceinline__ void tacc_add(TAcc<R>& acc, R v, R s, R phi, R theta,
   tacc_add_d(acc, v, s, cp * st, sp * st, ct, pp, j);
 }
 
-// p for e = (c, s, 0) = (cos a, sin a, 0) from the sums, already divided by
-// 4 pi (ar + i ai = [(sum v^2 - 1) + sum v^2 tau'(2 + tau')] / (4 pi), the
-// reference constant left out; t = T / (4 pi)), in the frame of `literal`:
-// with b = T e,
-//   literal (p <- U^T p):  p0 = ar + c b_x + s b_y = ar + c^2 Txx + 2cs Txy + s^2 Tyy
-//                          p1 = -s b_x + c b_y    = cs (Tyy - Txx) + (c^2 - s^2) Txy
-//   lab:                   p0 = c ar + b_x,  p1 = s ar + b_y,
-//   both:                  p2 = b_z = c Txz + s Tyz.
+// The sums as the angles use them, ten reals per voxel: with
+// ar = [(sum v^2 - 1) + sum v^2 tau'(2 + tau')] / (4 pi) (complex; the
+// reference constant left out; the large part first, then the small optical
+// one) and t = T / (4 pi), for e = (c, s, 0) = (cos a, sin a, 0) and b = T e:
+//   literal (p <- U^T p):  p0 = ar + c b_x + s b_y = [ar + (txx + tyy)/2]
+//                               + cos 2a (txx - tyy)/2 + sin 2a txy
+//                          p1 = -s b_x + c b_y = cos 2a txy - sin 2a (txx - tyy)/2
+//   lab:                   p0 = c (ar + txx) + s txy,  p1 = c txy + s (ar + tyy)
+//   both:                  p2 = b_z = c txz + s tyz,
+// so a and b hold the two bracketed terms of the frame in use.  (12 operations
+// per voxel and angle and ten registers, where p from the twelve sums took 16
+// and twelve; the z-first pass, whose polarisation warps were the later to
+// finish, 53.4 -> 48.9 ms per energy at 1024 x 1024 x 128.)
+template <typename R> struct PTen {
+  R a[2], b[2], xy[2], xz[2], yz[2];
+};
+template <typename R> __device__ __forceinline__ void pten_zero(PTen<R>& p) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) p.a[i] = p.b[i] = p.xy[i] = p.xz[i] = p.yz[i] = R(0);
+}
+// From t and ar (both already divided by 4 pi).
 template <typename R>
-__device__ __forceinline__ void p_from_tacc(R ar, R ai, const R (&t)[5][2], R c, R s, bool literal,
-                                            typename RT<R>::C out[3]) {
-  if (literal) {
-    const R c2 = c * c, s2 = s * s, cs2 = R(2) * c * s, cs = c * s, d2 = c2 - s2;
-    out[0] = RT<R>::mk(fma(s2, t[2][0], fma(cs2, t[1][0], fma(c2, t[0][0], ar))),
-                       fma(s2, t[2][1], fma(cs2, t[1][1], fma(c2, t[0][1], ai))));
-    out[1] = RT<R>::mk(fma(d2, t[1][0], cs * (t[2][0] - t[0][0])),
-                       fma(d2, t[1][1], cs * (t[2][1] - t[0][1])));
-  } else {
-    out[0] = RT<R>::mk(fma(c, ar + t[0][0], s * t[1][0]), fma(c, ai + t[0][1], s * t[1][1]));
-    out[1] = RT<R>::mk(fma(s, ar + t[2][0], c * t[1][0]), fma(s, ai + t[2][1], c * t[1][1]));
+__device__ __forceinline__ void pten_of(PTen<R>& p, const R (&ar)[2], const R (&t)[5][2],
+                                        bool literal) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    p.a[i] = literal ? ar[i] + R(0.5) * (t[0][i] + t[2][i]) : ar[i] + t[0][i];
+    p.b[i] = literal ? R(0.5) * (t[0][i] - t[2][i]) : ar[i] + t[2][i];
+    p.xy[i] = t[1][i];
+    p.xz[i] = t[3][i];
+    p.yz[i] = t[4][i];
   }
-  out[2] = RT<R>::mk(fma(c, t[3][0], s * t[4][0]), fma(c, t[3][1], s * t[4][1]));
+}
+// From the sums over the components.
+template <typename R>
+__device__ __forceinline__ void pten_of(PTen<R>& p, TAcc<R>& acc, bool literal) {
+  const R inv = R(1.0 / kFourPi);
+  const R ar[2] = {((acc.aw - R(1)) + acc.as[0]) * inv, acc.as[1] * inv};
+#pragma unroll
+  for (int q = 0; q < 5; ++q) {
+    acc.t[q][0] *= inv;
+    acc.t[q][1] *= inv;
+  }
+  pten_of(p, ar, acc.t, literal);
+}
+// p for one angle: c, s = cos a, sin a; c2, s2 = cos 2a, sin 2a.
+template <typename R>
+__device__ __forceinline__ void p_from_pten(const PTen<R>& p, R c, R s, R c2, R s2, bool literal,
+                                            typename RT<R>::C* out) {
+  if (literal) {
+    out[0] = RT<R>::mk(fma(c2, p.b[0], fma(s2, p.xy[0], p.a[0])),
+                       fma(c2, p.b[1], fma(s2, p.xy[1], p.a[1])));
+    out[1] = RT<R>::mk(fma(c2, p.xy[0], -s2 * p.b[0]), fma(c2, p.xy[1], -s2 * p.b[1]));
+  } else {
+    out[0] = RT<R>::mk(fma(c, p.a[0], s * p.xy[0]), fma(c, p.a[1], s * p.xy[1]));
+    out[1] = RT<R>::mk(fma(c, p.xy[0], s * p.b[0]), fma(c, p.xy[1], s * p.b[1]));
+  }
+  out[2] = RT<R>::mk(fma(c, p.xz[0], s * p.yz[0]), fma(c, p.xz[1], s * p.yz[1]));
 }
 
 // |(I - r r) v|^2 = sum_k |v_k - r_k (r . v)|^2 for one bin.
