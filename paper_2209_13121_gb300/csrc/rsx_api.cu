@@ -481,9 +481,11 @@ cudaError_t planes_x_fft(rsx_context* c, void* data, const ZPlan& zp, long long 
                          const rsx::XMask& xm, cudaStream_t s) {
   const rsx_config& g = c->cfg;
   if (g.nx == 1) return cudaSuccess;
-  if (sizeof(R) == 4 && (g.nx == 512 || (g.nx == 1024 && c->tw4) || (g.nx == 2048 && c->tw2k)))
+  if (sizeof(R) == 4 && c->n_sm > 0 &&
+      (g.nx == 512 || (g.nx == 1024 && c->tw4) || (g.nx == 2048 && c->tw2k)))
     return rsx::launch_x_planes(data, g.nx, g.ny, zp.ns, nfields, xm,
-                                g.nx == 1024 ? c->tw4 : g.nx == 2048 ? c->tw2k : c->twx, s);
+                                g.nx == 1024 ? c->tw4 : g.nx == 2048 ? c->tw2k : c->twx, c->n_sm,
+                                s);
   const long long nrows = nfields * zp.ns * g.ny;
   if (g.nx == 1024 && c->tw4) return rsx::launch_row_fft4s<R>(data, nrows, c->tw4, s);
   return rsx::launch_row_fft<R>(data, g.nx, nrows, c->twx, s);
@@ -680,8 +682,25 @@ int x_pass(rsx_context* c, const PolParams<R>& pp, cudaStream_t s) {
   return RSX_OK;
 }
 
+bool planes_plan(const rsx_context* c, int ie, ZPlan* zp);
+// Whether one image alone is worth the planes path, whose pass over the
+// morphology is then shared by no other angle: FP64 (256 x 256 x 32, c = 3:
+// 1199 -> 917 us), lateral sizes that are not powers of two (300 x 300 x 45:
+// 598 -> 232), and from 2^21 voxels on (256 x 256 x 64: 143 -> 102; 256 x 256 x 16:
+// 45 -> 51, so not below) except for FP32 rows of 512 or 1024 points, whose
+// fused one-angle passes stay ahead (1024 x 1024 x 16: 331 against 407).
+bool single_on_planes(const rsx_config& g) {
+  if (g.precision == 64 || (g.nx & (g.nx - 1)) || (g.ny & (g.ny - 1))) return true;
+  return g.nx != 512 && g.nx != 1024 && (long long)g.nx * g.ny * g.nz >= (1 << 21);
+}
 template <typename R>
-int scatter_angle(rsx_context* c, int ie, double alpha, void* img, cudaStream_t s) {
+int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang, int rotation,
+                      const ZPlan& zp, cudaStream_t s, const double* one = nullptr,
+                      void* img = nullptr);
+
+template <typename R>
+int scatter_angle(rsx_context* c, int ie, double alpha, void* img, cudaStream_t s,
+                  bool try_planes) {
   const rsx_config& g = c->cfg;
   int rc = ensure_geo<R>(c, ie, s);
   if (rc) return rc;
@@ -693,6 +712,9 @@ int scatter_angle(rsx_context* c, int ie, double alpha, void* img, cudaStream_t 
            "Ewald kernel");
     return RSX_OK;
   }
+  ZPlan zp;
+  if (try_planes && single_on_planes(g) && planes_plan(c, ie, &zp))
+    return run_energy_planes<R>(c, ie, 0.0, 0.0, 1, 1, zp, s, &alpha, img);
   if (g.algorithm == 2 && (rc = ensure_nt<R>(c, ie, s))) return rc;
   if ((rc = x_pass<R>(c, make_params<R>(c, ie, alpha, 0), s))) return rc;
   // The constant -(c-1) e' / (4 pi) left out of p before the FFT returns at
@@ -941,7 +963,8 @@ static bool zfirst_plan(const rsx_context* c, int ie, ZPlan* zp) {
 // arithmetic is the bound).  FP32 with rows the x-first passes serve (x and
 // p fused, then y and the two bins fused: half the passes over p): while at
 // most 3/4 of the bins are kept.
-static bool planes_plan(const rsx_context* c, int ie, ZPlan* zp) {
+namespace {
+bool planes_plan(const rsx_context* c, int ie, ZPlan* zp) {
   const rsx_config& g = c->cfg;
   if (!planes_cfg(&g) || !c->imgs || ie < 0 || ie >= (int)c->energies.size()) return false;
   if (zfirst_plan(c, ie, zp)) {
@@ -971,6 +994,7 @@ static bool planes_plan(const rsx_context* c, int ie, ZPlan* zp) {
   zp->kz = kz < cap ? (int)kz : cap;
   return zp->kz >= 1;
 }
+}  // namespace
 
 size_t rsx_workspace_bytes(const rsx_config* cfg) {
   if (check_config(cfg) != RSX_OK) return 0;
@@ -1380,8 +1404,8 @@ int rsx_scatter_angle(rsx_context* c, int ie, double alpha, void* img, void* str
   RSX_DEVPTR(img, c->dev, "img_out");
   DeviceGuard dg(c->dev);
   cudaStream_t s = (cudaStream_t)stream;
-  return c->cfg.precision == 32 ? scatter_angle<float>(c, ie, alpha, img, s)
-                                : scatter_angle<double>(c, ie, alpha, img, s);
+  return c->cfg.precision == 32 ? scatter_angle<float>(c, ie, alpha, img, s, true)
+                                : scatter_angle<double>(c, ie, alpha, img, s, true);
 }
 
 namespace {
@@ -1456,10 +1480,11 @@ int run_energy_angles_batched(rsx_context* c, int ie, double start, double inc, 
 // q_z planes of every angle (angle k, field f, plane s at
 // ((k * 3 + f) * ns + s) * nx * ny of p), one launch each x- and
 // y-transforms them, then the images and the rotation into the average
-// follow, n_img angles at a time.
+// follow, n_img angles at a time.  one: a single angle (radians) instead of
+// the list, its image going to img, not rotated.
 template <typename R>
 int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang, int rotation,
-                      const ZPlan& zp, cudaStream_t s) {
+                      const ZPlan& zp, cudaStream_t s, const double* one, void* img) {
   const rsx_config& g = c->cfg;
   int rc = ensure_geo<R>(c, ie, s);
   if (rc) return rc;
@@ -1479,7 +1504,7 @@ int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang
     rsx::AngleBatch<R> ab;
     memset(&ab, 0, sizeof(ab));
     for (int k = 0; k < nk; ++k) {
-      alpha[k] = rotation ? (start + inc * (a0 + k)) * (kPi / 180.0) : 0.0;
+      alpha[k] = one ? *one : rotation ? (start + inc * (a0 + k)) * (kPi / 180.0) : 0.0;
       rsx::add_angle(ab, alpha[k], g.nx, g.ny);
     }
     {
@@ -1534,9 +1559,10 @@ int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang
         PhaseTimer pt(c, RSX_PHASE_EWALD, s);
         RSX_CK(rsx::launch_plane_images<R>((const char*)c->p + (size_t)i0 * 3 * zp.ns * c->npix * 2 * sizeof(R),
                                            g.nx, g.ny, g.nz, zp.kb, zp.ns, (const Geo<R>*)c->geo,
-                                           dc, c->imgs, s),
+                                           dc, img ? img : c->imgs, s),
                "Ewald kernel");
       }
+      if (img) continue;
       PhaseTimer pt(c, RSX_PHASE_ROTATE, s);
       RSX_CK(rsx::launch_rotate_acc_many<R>(c->imgs, c->acc, g.nx, g.ny, rb, rotation != 0, s),
              "rotation kernel");
@@ -1558,7 +1584,7 @@ int run_energy_angles(rsx_context* c, int ie, double start, double inc, int nang
   }
   for (int a = 0; a < nang; ++a) {
     const double alpha = rotation ? (start + inc * a) * (kPi / 180.0) : 0.0;
-    int rc = scatter_angle<R>(c, ie, alpha, c->img, s);
+    int rc = scatter_angle<R>(c, ie, alpha, c->img, s, false);
     if (rc) return rc;
     PhaseTimer pt(c, RSX_PHASE_ROTATE, s);
     RSX_CK(rsx::launch_rotate_acc<R>(c->img, c->acc, c->cfg.nx, c->cfg.ny, alpha, rotation != 0, s),

@@ -368,7 +368,7 @@ cudaError_t launch_y_planes(const void* tmap, void* p, int nx, int ny, int nz, i
                             const void* tw, const void* twy, int* err, int n_sm, unsigned poll,
                             cudaStream_t s);
 cudaError_t launch_x_planes(void* data, int nx, int ny, int ns, long long nfields,
-                            const XMask& mask, const void* tw, cudaStream_t s);
+                            const XMask& mask, const void* tw, int n_sm, cudaStream_t s);
 template <typename R>
 cudaError_t launch_plane_images(const void* planes, int nx, int ny, int nz, int kb, int ns,
                                 const Geo<R>* geo, const ImageDc<R>& dc, void* imgs,

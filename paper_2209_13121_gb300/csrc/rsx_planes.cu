@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
   };
   for (int i = t; nz > 1 && i < H * NSP; i += kPlThreads) {  // (nz = 1 has no shared memory)
     const int z = i / NSP, r = i - z * NSP, g = r / SBP, b = first(g) + NP * (r - g * SBP);
-    tw[i] = twz[(int)(((long long)(kb + b) * z) % nz)];
+    tw[i] = twz[(unsigned)((kb + b) * z) % (unsigned)nz];  // ((kb + b) z < 2^16)
   }
 
   // this thread's voxels: the sums of Eq. (polarization), divided by 4 pi.
@@ -701,20 +701,23 @@ __global__ void __launch_bounds__(512, 1) k_y_planes(
 // x-FFT of the planes' rows in place (FP32, nx = NX = 512, 1024 or 2048), one
 // warp per row, storing only the column groups (NX / 32 columns each) that
 // the y pass reads from the row's plane (mask.m[plane], a bit per group;
-// ~53 % of them at 1024 x 1024 x 128, 5 nm, 270 eV).  HBM-bound: the row goes to
-// shared memory by asynchronous 16-byte copies (a lane keeps all NX / 64 of
-// its copies in flight, no registers held), issued before the twiddle
-// table's loads so that the two overlap.
+// ~53 % of them at 1024 x 1024 x 128, 5 nm, 270 eV).  HBM-bound: a row comes to
+// shared memory by asynchronous 16-byte copies (no registers held), and a
+// persistent warp issues the next row's as soon as its transform has read
+// the buffer for the last time, so that they overlap the second half of the
+// transform and the stores.
 //   NX = 1024: four-step 32 x 32 in registers with one padded transpose; 512:
 //   16 x 32, the 32-point half split over lane pairs; 2048: a radix-2
 //   decimation in frequency as the row is read, then two 1024-point
 //   transforms, kept in registers (64 complex a lane) so that the even and
-//   odd outputs leave as one 16-byte store.
+//   odd outputs leave as one 16-byte store; 12 warps, one block per SM, share
+//   one twiddle table (two blocks of 4 warps, one row each: 55.7 ms per energy at
+//   2048 x 2048 x 64, 91 angles, 4.5 TB/s; 36.0 ms, 7.0 TB/s so).
 // tw_g: W512^j; W1024^(n1 k2) as [32][32]; for 2048 that, then W2048^n, n < 1024.
 template <int NX> struct XRow {
   static constexpr int FS = NX == 2048 ? 2 * 1056 : (NX / 32) * 33;
   static constexpr int NTW = NX;
-  static constexpr int W = NX == 2048 ? 4 : 8;  // warps per block, two blocks per SM
+  static constexpr int W = NX == 2048 ? 12 : 8, BPS = NX == 2048 ? 1 : 2;  // warps, blocks per SM
 };
 
 // The first half of a 1024-point transform up to and including the
@@ -731,7 +734,7 @@ __device__ __forceinline__ void fft1024_half(float2* v, float2* F, const float2*
 }
 
 template <int NX>
-__global__ void __launch_bounds__(32 * XRow<NX>::W, 2) k_x_planes(
+__global__ void __launch_bounds__(32 * XRow<NX>::W, XRow<NX>::BPS) k_x_planes(
     float2* __restrict__ data, long long nrows, int ny, int ns, const __grid_constant__ XMask mask,
     const float2* __restrict__ tw_g) {
   using C = float2;
@@ -740,66 +743,91 @@ __global__ void __launch_bounds__(32 * XRow<NX>::W, 2) k_x_planes(
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* F = tw + NTW + (threadIdx.x >> 5) * FS;
   const int lane = threadIdx.x & 31;
-  const long long row = (long long)blockIdx.x * W + (threadIdx.x >> 5);
-  const unsigned m = row < nrows ? mask.m[(int)((row / ny) % ns)] : 0u;
-  C* r = data + (size_t)row * NX;
-  if (m) {
+  const long long stride = (long long)gridDim.x * W;
+  long long row = (long long)blockIdx.x * W + (threadIdx.x >> 5);
+  // this warp's next row with columns to keep, from row on; its mask in m
+  unsigned m = 0;
+  auto seek = [&] {
+    for (; row < nrows; row += stride)
+      if ((m = mask.m[(int)((row / ny) % ns)])) return;
+    m = 0;
+  };
+  auto fetch = [&] {
+    const C* r = data + (size_t)row * NX;
 #pragma unroll
     for (int j = 0; j < NX / 64; ++j) {
       const int n = 2 * (lane + 32 * j);
       cp_async_pair(F + (NX == 2048 && n >= 1024 ? n + 32 : n), r + n);
     }
-  }
+  };
+  seek();
+  if (m) fetch();
   for (int i = threadIdx.x; i < NTW; i += 32 * W) tw[i] = tw_g[i];
   __syncthreads();
-  if (!m) return;
-  cp_async_wait_all();
-  __syncwarp();
-  C v[32];
-  if constexpr (NX == 1024) {
+  while (m) {
+    cp_async_wait_all();
+    __syncwarp();
+    const unsigned mr = m;  // this row's, and its place
+    C* const r = data + (size_t)row * NX;
+    C v[32];
+    if constexpr (NX == 1024) {
 #pragma unroll
-    for (int n2 = 0; n2 < 32; ++n2) v[n2] = F[lane + 32 * n2];
-    fft1024_half(v, F, tw, lane);
-    dft32(v);
+      for (int n2 = 0; n2 < 32; ++n2) v[n2] = F[lane + 32 * n2];
+      fft1024_half(v, F, tw, lane);
+      __syncwarp();
+      row += stride;
+      seek();
+      if (m) fetch();
+      dft32(v);
 #pragma unroll
-    for (int k1 = 0; k1 < 32; ++k1)
-      if (m >> k1 & 1u) r[lane + 32 * k1] = v[k1];
-  } else if constexpr (NX == 2048) {
-    C u[32];
+      for (int k1 = 0; k1 < 32; ++k1)
+        if (mr >> k1 & 1u) r[lane + 32 * k1] = v[k1];
+    } else if constexpr (NX == 2048) {
+      C u[32];
 #pragma unroll
-    for (int n2 = 0; n2 < 32; ++n2) {
-      const int n = lane + 32 * n2;
-      const C a = F[n], b = F[1056 + n];
-      v[n2] = cadd(a, b);
-      u[n2] = cmul(csub(a, b), tw[1024 + n]);
+      for (int n2 = 0; n2 < 32; ++n2) {
+        const int n = lane + 32 * n2;
+        const C a = F[n], b = F[1056 + n];
+        v[n2] = cadd(a, b);
+        u[n2] = cmul(csub(a, b), tw[1024 + n]);
+      }
+      fft1024_half(v, F, tw, lane);
+      fft1024_half(u, F + 1056, tw, lane);
+      __syncwarp();
+      row += stride;
+      seek();
+      if (m) fetch();
+      dft32(v);
+      dft32(u);
+#pragma unroll
+      for (int k1 = 0; k1 < 32; ++k1)
+        if (mr >> k1 & 1u)
+          reinterpret_cast<float4*>(r)[lane + 32 * k1] =
+              make_float4(v[k1].x, v[k1].y, u[k1].x, u[k1].y);
+    } else {
+#pragma unroll
+      for (int n2 = 0; n2 < 16; ++n2) v[n2] = F[lane + 32 * n2];
+      dft_reg<16>(v);
+      C u[16];
+#pragma unroll
+      for (int k2 = 0; k2 < 16; ++k2) u[k2] = cmul(v[out_pos<16>(k2)], tw[lane * k2]);
+      __syncwarp();
+#pragma unroll
+      for (int k2 = 0; k2 < 16; ++k2) F[k2 * 33 + lane] = u[k2];
+      __syncwarp();
+      const int k2 = lane & 15, h = lane >> 4;
+#pragma unroll
+      for (int n = 0; n < 16; ++n) v[n] = F[k2 * 33 + 2 * n + h];
+      __syncwarp();
+      row += stride;
+      seek();
+      if (m) fetch();
+      dft32_pair(v, u, h);
+      const unsigned mh = mr >> (16 * h);
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        if (mh >> k & 1u) r[k2 + 256 * h + 16 * k] = u[k];
     }
-    fft1024_half(v, F, tw, lane);
-    fft1024_half(u, F + 1056, tw, lane);
-    dft32(v);
-    dft32(u);
-#pragma unroll
-    for (int k1 = 0; k1 < 32; ++k1)
-      if (m >> k1 & 1u)
-        reinterpret_cast<float4*>(r)[lane + 32 * k1] = make_float4(v[k1].x, v[k1].y, u[k1].x, u[k1].y);
-  } else {
-#pragma unroll
-    for (int n2 = 0; n2 < 16; ++n2) v[n2] = F[lane + 32 * n2];
-    dft_reg<16>(v);
-    C u[16];
-#pragma unroll
-    for (int k2 = 0; k2 < 16; ++k2) u[k2] = cmul(v[out_pos<16>(k2)], tw[lane * k2]);
-    __syncwarp();
-#pragma unroll
-    for (int k2 = 0; k2 < 16; ++k2) F[k2 * 33 + lane] = u[k2];
-    __syncwarp();
-    const int k2 = lane & 15, h = lane >> 4;
-#pragma unroll
-    for (int n = 0; n < 16; ++n) v[n] = F[k2 * 33 + 2 * n + h];
-    dft32_pair(v, u, h);
-    const unsigned mh = m >> (16 * h);
-#pragma unroll
-    for (int k = 0; k < 16; ++k)
-      if (mh >> k & 1u) r[k2 + 256 * h + 16 * k] = u[k];
   }
 }
 
@@ -1049,26 +1077,28 @@ cudaError_t launch_y_planes(const void* tmap, void* p, int nx, int ny, int nz, i
 
 template <int NX>
 static cudaError_t x_planes_impl(void* data, long long nrows, int ny, int ns, const XMask& mask,
-                                 const void* tw, cudaStream_t s) {
+                                 const void* tw, int n_sm, cudaStream_t s) {
   using X = XRow<NX>;
   const size_t smem = ((size_t)X::NTW + (size_t)X::W * X::FS) * sizeof(float2);
   auto kern = k_x_planes<NX>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)((nrows + X::W - 1) / X::W), 32 * X::W, smem, s>>>(
+  const long long want = (nrows + X::W - 1) / X::W, most = (long long)n_sm * X::BPS;
+  kern<<<(unsigned)(want < most ? want : most), 32 * X::W, smem, s>>>(
       (float2*)data, nrows, ny, ns, mask, (const float2*)tw);
   return cudaGetLastError();
 }
 
 cudaError_t launch_x_planes(void* data, int nx, int ny, int ns, long long nfields,
-                            const XMask& mask, const void* tw, cudaStream_t s) {
+                            const XMask& mask, const void* tw, int n_sm, cudaStream_t s) {
   const long long nrows = nfields * ns * ny;
   if (nrows <= 0) return cudaSuccess;
   // 16-byte row copies
-  if (!tw || ((uintptr_t)data & 15) || ns < 1 || ns > kMaxPlanesNz) return cudaErrorInvalidValue;
-  if (nx == 1024) return x_planes_impl<1024>(data, nrows, ny, ns, mask, tw, s);
-  if (nx == 2048) return x_planes_impl<2048>(data, nrows, ny, ns, mask, tw, s);
-  if (nx == 512) return x_planes_impl<512>(data, nrows, ny, ns, mask, tw, s);
+  if (!tw || ((uintptr_t)data & 15) || ns < 1 || ns > kMaxPlanesNz || n_sm <= 0)
+    return cudaErrorInvalidValue;
+  if (nx == 1024) return x_planes_impl<1024>(data, nrows, ny, ns, mask, tw, n_sm, s);
+  if (nx == 2048) return x_planes_impl<2048>(data, nrows, ny, ns, mask, tw, n_sm, s);
+  if (nx == 512) return x_planes_impl<512>(data, nrows, ny, ns, mask, tw, n_sm, s);
   return cudaErrorInvalidValue;
 }
 
