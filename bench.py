@@ -351,6 +351,19 @@ def run_ours(args):
         src_bytes = c * 4 * real if args.algorithm == 1 else 5 * cplx  # M, or N_t's 5 entries
         per_voxel = {"pol_fftx": src_bytes + 3 * cplx, "ffty": y_bytes, "ewald": z_bytes,
                      "rotate": 0, "other": 0, "nt": c * 4 * real + 5 * cplx}
+    if args.algorithm != 1:
+        # Algorithms 2 and 3 keep the same planes: per launch a batch of
+        # angles shares one read of N_t (2), or the energy's one pass reads
+        # the morphology and writes the planes of N_t's five entries (3)
+        ns_kept = [rsx.zfirst_plan_for(rsx.make_config(nx, ny, nz, c, voxel_nm), E)[0]
+                   for E in mine[args.warmup:]]
+        if prec == 32 and all(ns_kept):
+            frac = sum(ns_kept) / len(ns_kept) / nz
+            if args.algorithm == 2 and phases["pol_fftx"][1]:
+                per_voxel["pol_fftx"] = (src_bytes + 3 * cplx * frac * n_ang * args.steps
+                                         / phases["pol_fftx"][1])
+            if args.algorithm == 3:
+                per_voxel["nt"] = c * 4 * real + 5 * cplx * frac
     kx = angle_batch if args.algorithm == 1 else 1
     if kx > 1:
         # the x pass reads the morphology once per batch of kx angles and
@@ -361,8 +374,10 @@ def run_ours(args):
     # the z-first path (rsx_zfirst_plan): per energy, ns q_z planes of the
     # nz slices are kept and kz angles share one read of the morphology.
     # Per launch: the polarisation + z-FFT pass reads M and writes kz x 3 x ns
-    # planes; the x-FFT reads and writes them; the y-FFT + bin selection pass
-    # reads one angle's 3 x ns planes (bins per pixel not counted)
+    # planes; the x-FFT reads them and the y-FFT + bin selection pass follows.
+    # (The x pass stores and the y pass reads only the column groups whose
+    # pixels meet a plane, about half; the figures here count whole planes,
+    # so for those two passes they are upper bounds.)
     zplans = [zplan[i] for i in range(args.warmup, n_steps)]
     zfirst = args.algorithm == 1 and all(z[0] > 0 for z in zplans)
     if zfirst:
@@ -385,8 +400,9 @@ def run_ours(args):
         n_l = args.steps
     achieved = (bytes_per_voxel * N * n_l) / (t_ms / 1e3) / 1e9 if bytes_per_voxel else None
     if args.algorithm == 3:
-        # per-energy FFT work dominates; report the x-FFT of the five N_t entries
-        top = "pol_fftx"
+        # per-energy work dominates; report the pass that forms N_t (z-first
+        # stacks: with its z-FFT), or the x-FFT of its five entries
+        top = "pol_fftx" if phases["pol_fftx"][1] else "nt"
         t_ms, n_l = phases[top]
         bytes_per_voxel = per_voxel[top]
         achieved = (bytes_per_voxel * N * n_l) / (t_ms / 1e3) / 1e9 if n_l else None

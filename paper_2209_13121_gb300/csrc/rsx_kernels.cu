@@ -1,7 +1,15 @@
 // CUDA kernels of the GB300 P-RSoXS path (sm_103a).
 //
-// Per energy and e-field angle the hot path (FP32, nx and ny 1024 or 512) runs:
-//   k_pol_fft4s_tma  Eqs. (ncorr), (nrot), (polarization) and p <- U^T p for
+// rsx_run takes the planes path (rsx_planes.cu) for Algorithms 1 and 2 up to
+// 255 slices; of this file it uses
+//   k_pol_zfft_multi       p of a batch of angles and its z transform at the kept
+//                          bins (FP32 Algorithm 1, nz = 32, 64, 128)
+//   k_pol_fft4s_tma_multi  p of a batch of angles x-transformed (films)
+//   k_row_fft*, k_col_fft*, k_fft_any   the lateral transforms of general sizes
+//   k_rotate_acc_many      detector rotation about q = 0 and accumulation (Sec. 4).
+// The x-first passes serve FP32 rows of 512, 1024 and 2048 points where most
+// bins are kept, and single images:
+//   k_pol_fft4s_tma(_multi)  Eqs. (ncorr), (nrot), (polarization) and p <- U^T p for
 //                    whole x-rows, fed by bulk copies, then the rows' x-FFT;
 //                    p is never written before its first FFT pass.
 //   k_yz_tma         the y-FFT of each z-slice (tiles by 2-D tensor copies)
@@ -9,12 +17,11 @@
 //                    pixel needs (Eq. (Ewald)), accumulated across z.
 //   k_ewald_bins     Eqs. (3Dscatter) and (Ewald) from those bins; no 3-D X
 //                    array exists.
-//   k_rotate_acc     detector rotation about q = 0 and accumulation (Sec. 4).
 // The general-size kernels (Stockham FFTs in shared memory: k_pol_fftx,
 // k_col_fft, k_ewald_pruned / k_ewald_tma), the four-step variants with
 // plain loads (FP64), Algorithm 2's N_t kernels and the linearity path's
-// kernels follow.  None of the path is a dense contraction: the x pass is
-// HBM-bound, the fused y+z pass bound by instruction issue.
+// kernels follow.  None of the path is a dense contraction: the lateral passes
+// are HBM-bound, the passes that form p bound by instruction issue.
 #include <cuda.h>  // CUtensorMap (the type only; the library does not link libcuda)
 #include <math.h>
 #include <string.h>
