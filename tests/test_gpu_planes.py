@@ -66,8 +66,9 @@ def test_edges_match_oracle_and_the_general_path(rsx, shape, c, voxel, E, prec):
             ctx.set_morphology(dev)
             ctx.set_optical_constants([E], K)
             _close(ctx.run((0.0, 40.0, 160.0)), ref, prec)
-            # one angle without rotation is the single image, which takes the
-            # passes of the general path
+            # one angle without rotation is the single image, which keeps the
+            # one-angle passes on small powers of two and FP32 rows of 512 and
+            # 1024 points, and takes the planes path elsewhere
             img = torch.empty((ny, nx), device="cuda", dtype=dev.dtype)
             ctx.scatter_angle(0, 0.0, img)
             _close(ctx.run(rotation=False)[0], img.cpu().numpy(), prec, r=1.5)
