@@ -2607,11 +2607,14 @@ __global__ void k_nt_restore(const typename RT<R>::C* __restrict__ nt, typename 
 // stays below 2^60 for n <= 4096.  The floor is a shift and the fraction a
 // mask (no FP64 arithmetic).
 constexpr int kRotTile = 16;
-// The fraction of a 48-bit fixed-point position as a weight.  FP32 takes its
-// upper 32 bits (2^-32 of a pixel, 2^-8 of an FP32 unit: a 32-bit conversion
-// instead of a 64-bit one); FP64 all 48.
+// The fraction of a 48-bit fixed-point position as a weight.  FP32: all 48
+// bits, rounded once, from two 24-bit halves (each exact as a float; two
+// 32-bit conversions and a fused multiply-add, where the 64-bit conversion
+// runs at a quarter of the rate): a weight just above a whole pixel keeps its
+// 24 significant bits.
 __device__ __forceinline__ float rot_frac(long long f, float) {
-  return (float)(unsigned)(f >> 16) * (float)(1.0 / 4294967296.0);
+  const float hi = (float)((unsigned)(f >> 24) & 0xffffffu), lo = (float)((unsigned)f & 0xffffffu);
+  return fmaf(lo, (float)(1.0 / 281474976710656.0), hi * (float)(1.0 / 16777216.0));
 }
 __device__ __forceinline__ double rot_frac(long long f, double) {
   return (double)(f & ((1LL << 48) - 1)) * (1.0 / 281474976710656.0);
