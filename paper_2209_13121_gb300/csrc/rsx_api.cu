@@ -169,6 +169,7 @@ struct rsx_context {
   // the images of a batch of n_img angles ([n_img][ny][nx]): the linearity
   // path's, or the planes path's (there in the memory of part where it exists)
   void* imgs = nullptr;
+  void* means = nullptr;  // planes path: the slices' means (launch_slice_means)
   int n_img = 0;
   bool imgs_owned = false;
   // page-locked staging of host output (grown on demand)
@@ -192,7 +193,8 @@ namespace {
 
 void free_all(rsx_context* c) {
   void* ptrs[] = {c->M_owned, c->p,    c->img, c->acc,  c->geo,  c->twx, c->twy,
-                  c->twz,     c->tw4,  c->flag, c->err, c->part, c->dir, c->tw2k, c->b0idx};
+                  c->twz,     c->tw4,  c->flag, c->err, c->part, c->dir, c->tw2k, c->b0idx,
+                  c->means};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   for (auto& r : c->recs) {
@@ -574,10 +576,17 @@ int lin_planes_bins(rsx_context* c, int ie, const ZPlan& zp, cudaStream_t s) {
   rsx::YRuns runs;
   rsx::XMask xm;
   plane_runs(g, wavenumber(c->energies[ie]), zp, &runs, &xm);
+  const PolParams<R> pp = make_params<R>(c, ie, 0.0, 0);
+  const void* nt = c->M_host ? c->nt : nullptr;
+  {
+    PhaseTimer pt(c, RSX_PHASE_OTHER, s);
+    RSX_CK(rsx::launch_slice_means<R>(c->M, nt, nullptr, c->npix, g.nz, pp, false, c->means, s),
+           "slice means kernel");
+  }
   {
     PhaseTimer pt(c, RSX_PHASE_NT, s);
-    RSX_CK(rsx::launch_lin_planes<R>(c->M, c->M_host ? c->nt : nullptr, c->npix, g.nz,
-                                     make_params<R>(c, ie, 0.0, 0), c->ft, zp.kb, zp.ns, c->twz, s),
+    RSX_CK(rsx::launch_lin_planes<R>(c->M, nt, c->npix, g.nz, pp, c->ft, zp.kb, zp.ns, c->twz,
+                                     c->means, s),
            "N_t + z-FFT kernel");
   }
   {
@@ -591,7 +600,7 @@ int lin_planes_bins(rsx_context* c, int ie, const ZPlan& zp, cudaStream_t s) {
   const double dc = -(double)(g.n_components - 1) / (4.0 * kPi) * (double)c->N;
   PhaseTimer pt(c, RSX_PHASE_EWALD, s);
   RSX_CK(rsx::launch_bins5_planes<R>(c->ft, g.nx, g.ny, g.nz, zp.kb, zp.ns, (const Geo<R>*)c->geo,
-                                     dc, c->bins5, s),
+                                     dc, c->means, nt != nullptr, c->bins5, s),
          "q_z bins kernel");
   c->bins_energy = ie;
   return RSX_OK;
@@ -906,6 +915,12 @@ static bool planes_cfg(const rsx_config* cfg) {
   return cfg->algorithm != 3 && cfg->nz <= rsx::kMaxPlanesNz;
 }
 
+// Where the z transform comes first the slices' means are taken off.
+static bool uses_means(const rsx_config* cfg) {
+  return cfg->nz > 1 && (cfg->algorithm == 3 ? rsx::lin_planes_fits(cfg->precision, cfg->nz)
+                                             : planes_cfg(cfg));
+}
+
 // Complex elements of the p workspace: one p (3 N) per angle of the batch; on
 // the planes path at least 32 angles' p or 96 MB (within the 126 MB L2, so
 // that the planes of a batch of a small grid pass from kernel to kernel
@@ -1016,6 +1031,7 @@ size_t rsx_workspace_bytes(const rsx_config* cfg) {
   if (uses_yz(cfg) || y_tuned(cfg)) b += 2 * (size_t)npix;  // lower bin of every pixel
   if (!uses_yz(cfg) || cfg->algorithm == 3)
     b += (size_t)image_batch(cfg) * npix * R;        // a batch of images
+  if (uses_means(cfg)) b += rsx::slice_means_bytes(cfg->precision, cfg->nz);
   return b;
 }
 
@@ -1118,6 +1134,13 @@ int rsx_create(const rsx_config* cfg, rsx_context** out) {
   if (cfg->precision == 64 && cfg->algorithm == 1 &&
       (e = cudaMalloc(&c->dir, 3 * (size_t)cfg->n_components * c->N * R)) != cudaSuccess) {
     rc = cuda_fail(e, "director cache");
+    free_all(c);
+    delete c;
+    return rc;
+  }
+  if (uses_means(cfg) && (e = cudaMalloc(&c->means, rsx::slice_means_bytes(
+                                                        cfg->precision, cfg->nz))) != cudaSuccess) {
+    rc = cuda_fail(e, "slice means");
     free_all(c);
     delete c;
     return rc;
@@ -1496,6 +1519,14 @@ int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang
   plane_runs(g, wavenumber(c->energies[ie]), zp, &runs, &xm);
   CUtensorMap tm_m;
   if (zp.zfft && !make_tmap_m(c, &tm_m)) return fail(RSX_ERR_CUDA, "morphology tensor map");
+  const void* nt = g.algorithm == 2 ? c->nt : nullptr;
+  const bool lit = g.frame == RSX_FRAME_LITERAL;
+  const void* means = g.nz > 1 ? c->means : nullptr;  // (one slice: no z transform)
+  if (means) {
+    PhaseTimer pt(c, RSX_PHASE_OTHER, s);
+    RSX_CK(rsx::launch_slice_means<R>(c->M, nt, c->dir, c->npix, g.nz, pp, lit, c->means, s),
+           "slice means kernel");
+  }
   // the angles spread evenly over the fewest passes of at most kz
   const int npass = (nang + zp.kz - 1) / zp.kz, per = (nang + npass - 1) / npass;
   for (int a0 = 0; a0 < nang; a0 += per) {
@@ -1522,15 +1553,15 @@ int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang
                         g.nx == 1024 ? c->tw4 : g.nx == 2048 ? c->tw2k : c->twx, c->err, c->n_sm,
                         c->wait_polls, s)
                   : rsx::launch_pol_zfft_multi(&tm_m, g.nx, g.ny, g.nz, pp, ang, c->p,
-                                               3 * fstride, fstride, zp.kb, zp.ns, c->twz, c->err,
-                                               c->n_sm, c->wait_polls, s);
+                                               3 * fstride, fstride, zp.kb, zp.ns, c->twz, means,
+                                               c->err, c->n_sm, c->wait_polls, s);
         } else {
-          e = rsx::launch_pol_planes<R>(c->M, g.algorithm == 2 ? c->nt : nullptr, c->dir, c->npix,
-                                        g.nz, pp, ab, c->p, zp.kb, zp.ns, c->twz, s);
+          e = rsx::launch_pol_planes<R>(c->M, nt, c->dir, c->npix, g.nz, pp, ab, c->p, zp.kb, zp.ns,
+                                        c->twz, means, s);
         }
       } else {
-        e = rsx::launch_pol_planes<R>(c->M, g.algorithm == 2 ? c->nt : nullptr, c->dir, c->npix,
-                                      g.nz, pp, ab, c->p, zp.kb, zp.ns, c->twz, s);
+        e = rsx::launch_pol_planes<R>(c->M, nt, c->dir, c->npix, g.nz, pp, ab, c->p, zp.kb, zp.ns,
+                                      c->twz, means, s);
       }
       RSX_CK(e, "polarisation + z-transform kernel");
     }
@@ -1550,16 +1581,20 @@ int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang
       memset(&rb, 0, sizeof(rb));
       dc.n = ni;
       for (int k = 0; k < ni; ++k) {
-        const bool lit = g.frame == RSX_FRAME_LITERAL;
         dc.x[k] = (R)(lit ? ref : ref * cos(alpha[i0 + k]));
         dc.y[k] = (R)(lit ? 0.0 : ref * sin(alpha[i0 + k]));
         rsx::add_angle(rb, alpha[i0 + k], g.nx, g.ny);
+        dc.ce[k] = rb.ce[k];
+        dc.se[k] = rb.se[k];
+        dc.c2[k] = rb.c2[k];
+        dc.s2[k] = rb.s2[k];
       }
       {
         PhaseTimer pt(c, RSX_PHASE_EWALD, s);
         RSX_CK(rsx::launch_plane_images<R>((const char*)c->p + (size_t)i0 * 3 * zp.ns * c->npix * 2 * sizeof(R),
                                            g.nx, g.ny, g.nz, zp.kb, zp.ns, (const Geo<R>*)c->geo,
-                                           dc, img ? img : c->imgs, s),
+                                           dc, means, nt != nullptr, lit, img ? img : c->imgs,
+                                           s),
                "Ewald kernel");
       }
       if (img) continue;

@@ -931,7 +931,7 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_zfft_multi(
     const __grid_constant__ CUtensorMap tmap, int nx, long long npix, long long ntiles,
     PolParams<float> pp, XAngles ang, float2* __restrict__ out, long long kstride,
     long long fstride, int kb, int ns, const float2* __restrict__ twz_g,
-    int* __restrict__ err, unsigned poll) {
+    const float* __restrict__ means, int* __restrict__ err, unsigned poll) {
   using C = float2;
   using Lay = ZfLayout<R>;
   constexpr int NZ = Lay::NZ, XW = Lay::XW, LXW = Lay::LXW, LS = Lay::LS, FS = Lay::FS;
@@ -944,7 +944,8 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_zfft_multi(
   float4* stage = reinterpret_cast<float4*>(smem_a128);  // [S][NZ][XW] voxels
   C* P = reinterpret_cast<C*>(stage + S * SV);            // [NPB][3][FS]
   C* twt = P + NPB * 3 * FS;                              // [32][R]: W_nz^(n2 (kb + s1))
-  unsigned long long* full = reinterpret_cast<unsigned long long*>(twt + 32 * R);
+  float* mean_s = reinterpret_cast<float*>(twt + 32 * R);  // [NZ][kMeanStride]
+  unsigned long long* full = reinterpret_cast<unsigned long long*>(mean_s + NZ * kMeanStride);
   unsigned long long* empty = full + S;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + S);
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
@@ -963,6 +964,7 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_zfft_multi(
   }
   for (int i = t; i < 32 * R; i += blockDim.x)
     twt[i] = twz_g[((i / R) * (kb + i % R)) & (NZ - 1)];
+  for (int i = t; i < NZ * kMeanStride; i += blockDim.x) mean_s[i] = means[i];
   __shared__ float4 ang_s[KMAX];  // cos a, sin a, cos 2a, sin 2a, indexed by a run-time angle
   if (t == 0) {
 #pragma unroll
@@ -1006,7 +1008,8 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_zfft_multi(
     for (int rr = 0; rr < (int)nmine; ++rr) {
       TAcc<float> acc[SL];
 #pragma unroll
-      for (int sl = 0; sl < SL; ++sl) tacc_zero(acc[sl]);
+      for (int sl = 0; sl < SL; ++sl)
+        tacc_start(acc[sl], mean_s + ((pt + sl * TP) >> LXW) * kMeanStride);
       for (int j = 0; j < per_row; ++j) {
         const int cs = slot, cph = ph;
         if (++slot == S) slot = 0, ph ^= 1;
@@ -2964,8 +2967,9 @@ cudaError_t launch_pol_fft4s_tma_multi(const void* M, int nx, int ny, int nz,
 template <int R>
 static cudaError_t pol_zfft_impl(const void* tmap, int nx, int ny, const PolParams<float>& pp,
                                  const XAngles& ang, void* out, long long kstride,
-                                 long long fstride, int kb, int ns, const void* twz, int* err,
-                                 int n_sm, unsigned poll, cudaStream_t s) {
+                                 long long fstride, int kb, int ns, const void* twz,
+                                 const void* means, int* err, int n_sm, unsigned poll,
+                                 cudaStream_t s) {
   // as the multi-angle x pass: 3 stages (one component of a 1024-voxel
   // tile each), 6 row buffers, 8 polarisation warps, three transform groups
   // and a producer: one 576-thread block per SM, ~200 KB of shared memory
@@ -2973,12 +2977,13 @@ static cudaError_t pol_zfft_impl(const void* tmap, int nx, int ny, const PolPara
   constexpr int S = 3, NPB = 6, PW = 8, FG = 3;
   using Lay = ZfLayout<R>;
   if (n_sm <= 0 || ang.n < 1 || ang.n > kMaxXAngles || nx % Lay::XW || ns < 1 || ns > Lay::NZ ||
-      kb < 0 || kb >= Lay::NZ)
+      kb < 0 || kb >= Lay::NZ || !means)
     return cudaErrorInvalidValue;
   const long long npix = (long long)nx * ny, ntiles = npix / Lay::XW;
   if (ntiles <= 0) return cudaSuccess;
   const size_t smem = (size_t)S * 1024 * sizeof(float4) +
-                      ((size_t)NPB * 3 * Lay::FS + 32 * R) * sizeof(float2) + 2 * S * 8 + 16;
+                      ((size_t)NPB * 3 * Lay::FS + 32 * R) * sizeof(float2) +
+                      (size_t)Lay::NZ * kMeanStride * sizeof(float) + 2 * S * 8 + 16;
   auto kern = ns > 16 * R ? k_pol_zfft_multi<R, S, NPB, PW, FG, kMaxXAngles, true>
                           : k_pol_zfft_multi<R, S, NPB, PW, FG, kMaxXAngles, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -2989,7 +2994,7 @@ static cudaError_t pol_zfft_impl(const void* tmap, int nx, int ny, const PolPara
   const long long grid = ntiles < (long long)n_sm ? ntiles : (long long)n_sm;
   kern<<<(unsigned)grid, 32 * (PW + 3 * FG + 1), smem, s>>>(
       *(const CUtensorMap*)tmap, nx, npix, ntiles, pp, ang, (float2*)out, kstride, fstride, kb, ns,
-      (const float2*)twz, err, poll);
+      (const float2*)twz, (const float*)means, err, poll);
   return cudaGetLastError();
 }
 
@@ -3001,17 +3006,17 @@ bool zfirst_fusable(int nx, int ny, int nz) {
 cudaError_t launch_pol_zfft_multi(const void* tmap, int nx, int ny, int nz,
                                   const PolParams<float>& pp, const XAngles& ang, void* out,
                                   long long kstride, long long fstride, int kb, int ns,
-                                  const void* twz, int* err, int n_sm, unsigned poll,
-                                  cudaStream_t s) {
+                                  const void* twz, const void* means, int* err, int n_sm,
+                                  unsigned poll, cudaStream_t s) {
   if (nz == 128)
-    return pol_zfft_impl<4>(tmap, nx, ny, pp, ang, out, kstride, fstride, kb, ns, twz, err, n_sm,
-                            poll, s);
+    return pol_zfft_impl<4>(tmap, nx, ny, pp, ang, out, kstride, fstride, kb, ns, twz, means, err,
+                            n_sm, poll, s);
   if (nz == 64)
-    return pol_zfft_impl<2>(tmap, nx, ny, pp, ang, out, kstride, fstride, kb, ns, twz, err, n_sm,
-                            poll, s);
+    return pol_zfft_impl<2>(tmap, nx, ny, pp, ang, out, kstride, fstride, kb, ns, twz, means, err,
+                            n_sm, poll, s);
   if (nz != 32) return cudaErrorInvalidValue;
-  return pol_zfft_impl<1>(tmap, nx, ny, pp, ang, out, kstride, fstride, kb, ns, twz, err, n_sm,
-                          poll, s);
+  return pol_zfft_impl<1>(tmap, nx, ny, pp, ang, out, kstride, fstride, kb, ns, twz, means, err,
+                          n_sm, poll, s);
 }
 
 bool yz_fusable(int nx, int ny, int nz) {

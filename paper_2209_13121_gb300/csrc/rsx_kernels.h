@@ -211,8 +211,8 @@ bool zfirst_fusable(int nx, int ny, int nz);
 cudaError_t launch_pol_zfft_multi(const void* tmap, int nx, int ny, int nz,
                                   const PolParams<float>& pp, const XAngles& ang, void* out,
                                   long long kstride, long long fstride, int kb, int ns,
-                                  const void* twz, int* err, int n_sm, unsigned poll,
-                                  cudaStream_t s);
+                                  const void* twz, const void* means, int* err, int n_sm,
+                                  unsigned poll, cudaStream_t s);
 // The same pipeline for Algorithm 2: p = N_t e from the five stored entries
 // of N_t ([5][N] complex float, 16-byte aligned; the reference constant
 // left out as k_nt_all stores it).
@@ -317,16 +317,28 @@ cudaError_t launch_rotate_acc(const void* img, void* acc, int nx, int ny, double
 // launch_plane_images: the angles' images ([n][ny][nx], fftshift order) from
 // the x- and y-transformed planes; dc: the x and y parts, per angle, of the
 // constant left out of p (returned at q = 0).
+// launch_slice_means: into means ([nz][16]) the mean of the sums behind p (or
+// of nt's entries, in the frame of literal) over a sample of each slice's
+// pixels.  means (null: none) in launch_pol_planes, launch_pol_zfft_multi and
+// launch_lin_planes: what is left out of p; in launch_plane_images and
+// launch_bins5_planes: the same rows, returned at q = 0 (from_nt: they were
+// formed from nt).
 constexpr int kMaxPlanesNz = 255;
 template <typename R> struct ImageDc {
   int n;
   R x[kMaxAngleBatch], y[kMaxAngleBatch];
+  R ce[kMaxAngleBatch], se[kMaxAngleBatch], c2[kMaxAngleBatch], s2[kMaxAngleBatch];
 };
+size_t slice_means_bytes(int precision, int nz);
+template <typename R>
+cudaError_t launch_slice_means(const void* M, const void* nt, const void* dir, long long npix,
+                               int nz, const PolParams<R>& pp, bool literal, void* means,
+                               cudaStream_t s);
 bool pol_planes_fits(int precision, int nz, int kb, int ns);
 template <typename R>
 cudaError_t launch_pol_planes(const void* M, const void* nt, const void* dir, long long npix,
                               int nz, const PolParams<R>& pp, const AngleBatch<R>& ang, void* out,
-                              int kb, int ns, const void* twz, cudaStream_t s);
+                              int kb, int ns, const void* twz, const void* means, cudaStream_t s);
 // The linearity path on the planes: N_t's five entries (from M, or nt),
 // z-transformed, the ns kept bins of entry e at out + (e * ns + s) * npix
 // (lin_planes_fits: nz = 8 .. 64 a power of two, 128 in FP32), and, from the
@@ -336,10 +348,11 @@ bool lin_planes_fits(int precision, int nz);
 template <typename R>
 cudaError_t launch_lin_planes(const void* M, const void* nt, long long npix, int nz,
                               const PolParams<R>& pp, void* out, int kb, int ns, const void* twz,
-                              cudaStream_t s);
+                              const void* means, cudaStream_t s);
 template <typename R>
 cudaError_t launch_bins5_planes(const void* planes, int nx, int ny, int nz, int kb, int ns,
-                                const Geo<R>* geo, double dc, void* bins, cudaStream_t s);
+                                const Geo<R>* geo, double dc, const void* means, bool from_nt,
+                                void* bins, cudaStream_t s);
 // The lateral transforms of the planes for tuned sizes (FP32), in place.
 // YRuns: per 16-column group cg < n the run of planes its pixels read:
 // first[cg] .. first[cg] + (start[cg + 1] - start[cg]) - 1 (start: prefix
@@ -371,8 +384,8 @@ cudaError_t launch_x_planes(void* data, int nx, int ny, int ns, long long nfield
                             const XMask& mask, const void* tw, int n_sm, cudaStream_t s);
 template <typename R>
 cudaError_t launch_plane_images(const void* planes, int nx, int ny, int nz, int kb, int ns,
-                                const Geo<R>* geo, const ImageDc<R>& dc, void* imgs,
-                                cudaStream_t s);
+                                const Geo<R>* geo, const ImageDc<R>& dc, const void* means,
+                                bool from_nt, bool literal, void* imgs, cudaStream_t s);
 template <typename R>
 cudaError_t launch_scale(const void* acc, void* out, long long n, double scale, cudaStream_t s);
 template <typename R>

@@ -20,6 +20,119 @@
 namespace rsx {
 namespace {
 
+// The mean of each slice, left out of every voxel's sums before the z
+// transform and returned at q = 0 (its transform lies there alone).  With the
+// z transform first, the mean would ride through the lateral transforms of
+// the few planes next to bin 0 and leave its rounding in every pixel of them.
+// (FP32, unrotated image away from q = 0, error against 64 bits, in units of
+// 1e-7, with the mean in and without, and transforming x and y first: six
+// materials at 300 x 180 x 45 21, 2.0 and 5.3; with a substrate below the film
+// 11, 1.3 and 1.6; one material at 45 x 512 x 16 6.4, 2.6 and 3.7.  Over 19
+// shapes and 11 morphologies, relative to x and y first: 1.24 and 0.82.)
+// Any constant near the mean serves, so it is that of 16 runs of 16 pixels
+// (FP64, whose arithmetic is slow: 8 of 8), one pixel a thread, so that its few
+// loads are all that is waited for.  Run r starts at floor((npix - len + 1)
+// frac(r / golden ratio)), which no period of a lattice resonates with.
+// means: [nz][kMeanStride] (MeanRow).
+template <typename R> constexpr int kMeanRun = sizeof(R) == 4 ? 16 : 8;
+template <typename R> constexpr int kMeanSample = kMeanRun<R> * kMeanRun<R>;
+constexpr int kMeanVals = 13;
+
+template <typename R>
+__global__ void __launch_bounds__(kMeanSample<R>) k_slice_means(
+    const typename RT<R>::V4* __restrict__ M, const typename RT<R>::C* __restrict__ nt,
+    const R* __restrict__ dir, long long npix, int nz, const __grid_constant__ PolParams<R> pp,
+    int literal, R* __restrict__ means) {
+  using C = typename RT<R>::C;
+  constexpr int LEN = kMeanRun<R>, NS = kMeanSample<R>, NW = NS / 32;
+  const int t = threadIdx.x, z = blockIdx.x;
+  const long long N = npix * nz;
+  const int S = npix < NS ? (int)npix : NS;
+  TAcc<R> a;
+  tacc_zero(a);
+  if (t < S) {
+    const unsigned long long g = (unsigned)(t / LEN) * 2654435769u;  // 2^32 frac(run / golden ratio)
+    const size_t v =
+        (size_t)z * npix +
+        (npix <= NS ? (size_t)t : (size_t)(g * (npix - LEN + 1) >> 32) + (size_t)(t % LEN));
+    if (nt) {
+#pragma unroll
+      for (int e = 0; e < 5; ++e) {
+        const C q = nt[(size_t)e * N + v];
+        a.t[e][0] = q.x;
+        a.t[e][1] = q.y;
+      }
+      PTen<R> p;
+      pten_of(p, a.as, a.t, literal != 0);  // (a.as is 0)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        a.t[0][i] = p.a[i];
+        a.t[2][i] = p.b[i];
+      }
+    } else {
+#pragma unroll 4
+      for (int j = 0; j < pp.c; ++j) {
+        const typename RT<R>::V4 m = M[(size_t)j * N + v];
+        if (dir) {
+          const R* dj = dir + (size_t)j * 3 * N + v;
+          tacc_add_d(a, (R)m.x, (R)m.y, dj[0], dj[N], dj[2 * N], pp, j);
+        } else {
+          tacc_add(a, (R)m.x, (R)m.y, (R)m.z, (R)m.w, pp, j);
+        }
+      }
+      a.aw -= R(1);
+    }
+  }
+  __shared__ R part[NW][kMeanVals];
+#pragma unroll
+  for (int q = 0; q < kMeanVals; ++q) {
+    R s = q < 10 ? a.t[q >> 1][q & 1] : q < 12 ? a.as[q & 1] : a.aw;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+    if ((t & 31) == 0) part[t >> 5][q] = s;
+  }
+  __syncthreads();
+  if (t < kMeanVals) {
+    R m = R(0);
+#pragma unroll
+    for (int k = 0; k < NW; ++k) m += part[k][t];
+    means[(size_t)z * kMeanStride + t] = m / (R)S;
+  }
+}
+
+// What leaving the means out takes from p at q = 0: PTen's ten numbers of npix
+// times their sum over z, in double.  A block of 256 threads calls
+// means_total, then those that want the result means_pten (FP64 arithmetic:
+// not more threads than need be).  from_nt: the rows are PTen's already.
+template <typename R>
+__device__ __forceinline__ void means_total(const R* __restrict__ means, int nz, long long npix,
+                                            double* total) {
+  const int t = threadIdx.x, q = t >> 4;
+  double m = 0.0;
+  if (q < kMeanVals)
+    for (int k = t & 15; k < nz; k += 16) m += (double)means[(size_t)k * kMeanStride + q];
+#pragma unroll
+  for (int d = 8; d > 0; d >>= 1) m += __shfl_xor_sync(0xffffffffu, m, d);
+  if ((t & 15) == 0 && q < kMeanVals) total[q] = m * (double)npix;
+  __syncthreads();
+}
+template <typename R>
+__device__ __forceinline__ void means_pten(const double* total, bool literal, bool from_nt,
+                                           PTen<R>& out) {
+  const double sc = from_nt ? 1.0 : 1.0 / kFourPi;
+  const bool half = literal && !from_nt;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const double* q = total + i;
+    const double ar = q[10] + (i == 0 ? total[12] : 0.0);
+    out.a[i] = (R)(sc * (half ? ar + 0.5 * (q[0] + q[4]) : ar + q[0]));
+    out.b[i] = (R)(sc * (half ? 0.5 * (q[0] - q[4]) : ar + q[4]));
+    out.xy[i] = (R)(sc * q[2]);
+    out.xz[i] = (R)(sc * q[6]);
+    out.yz[i] = (R)(sc * q[8]);
+  }
+}
+
 // A field at a fold's voxels: sum and difference.
 template <typename C> struct Folded {
   C s, d;
@@ -43,11 +156,10 @@ __device__ __forceinline__ int div_by(int it, unsigned m) { return (int)(((unsig
 // and 1 for even: ns of them, 7 at nz = 16 and 28 at nz = 45 (5 nm, 270 eV),
 // against ~10 to 25 for an FFT that would need a plan for every nz.  Before
 // the sum its z = 0 term is taken off the even bins' whole column and
-// returned to bin 0 (the other bins of a constant are 0): summed as it
-// stands, a column's mean would leave its rounding in every bin, where the
-// first stages of an FFT cancel it (one material, 45 x 40 x 40, unrotated
-// image against 64 bits away from q = 0: 3.9e-6 with it, 2.1e-6 without;
-// transforming every slice first 1.4e-6).
+// returned to bin 0 (the other bins of a constant are 0): of a column that
+// hardly changes along z (a lattice of rods, less the slices' means) the sum
+// as it stands would leave its rounding in every bin, where the first stages
+// of an FFT cancel it.
 // A thread keeps the angle-independent sums of its 4 voxels (one quad, or
 // two pairs) in registers for all angles.  Per step of A angles: every thread
 // forms p of its voxels for each angle and stores the folds (three fields) to
@@ -60,7 +172,8 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
     const typename RT<R>::V4* __restrict__ M, const typename RT<R>::C* __restrict__ nt,
     const R* __restrict__ dir, long long npix, int nz, int PX, int A, int kb, int ns,
     const __grid_constant__ PolParams<R> pp, const __grid_constant__ AngleBatch<R> ang,
-    typename RT<R>::C* __restrict__ out, const typename RT<R>::C* __restrict__ twz) {
+    typename RT<R>::C* __restrict__ out, const typename RT<R>::C* __restrict__ twz,
+    const R* __restrict__ means) {
   using C = typename RT<R>::C;
   using F = Folded<C>;
   constexpr int SBP = (SB + 1) & ~1;  // twiddles of a group, padded to pairs
@@ -116,9 +229,11 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
           tt[e][1] = v.y;
         }
         pten_of(ten[2 * sl + h], none, tt, literal);
+        if (means) pten_less(ten[2 * sl + h], means + zv * kMeanStride);
       } else {
         TAcc<R> a;
-        tacc_zero(a);
+        if (means) tacc_start(a, means + zv * kMeanStride);
+        else tacc_zero(a);
         for (int j = 0; j < pp.c; ++j) {
           const typename RT<R>::V4 m = ld_stream(M + (size_t)j * N + i);
           if (dir) {
@@ -267,13 +382,18 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 8 ? 1 : Q <= 8 && NF 
     const typename RT<R>::V4* __restrict__ M, const typename RT<R>::C* __restrict__ nt,
     const R* __restrict__ dir, long long npix, int kb, int ns,
     const __grid_constant__ PolParams<R> pp, const __grid_constant__ AngleBatch<R> ang,
-    typename RT<R>::C* __restrict__ out, const typename RT<R>::C* __restrict__ twz) {
+    typename RT<R>::C* __restrict__ out, const typename RT<R>::C* __restrict__ twz,
+    const R* __restrict__ means) {
   using C = typename RT<R>::C;
   using P = PlFft<R, Q>;
   constexpr int NZ = 4 * Q, PX = P::PX, KS = P::KS, A = NF == 3 ? P::A : 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);  // [A][NF][4][KS]
+  constexpr int NM = SRC == 1 ? NZ * kMeanStride : 0;
+  R* mean_s = reinterpret_cast<R*>(smem_raw);  // [NZ][kMeanStride] (N_t)
+  C* buf = reinterpret_cast<C*>(mean_s + NM);  // [A][NF][4][KS]
   const int t = threadIdx.x, px = t % PX, n2 = t / PX;
+  for (int i = 2 * t; i < NM; i += 2 * kPlThreads)
+    cp_async_elem(reinterpret_cast<C*>(mean_s + i), reinterpret_cast<const C*>(means + i));
   const long long N = npix * NZ;
   const long long pix0 = (long long)blockIdx.x * PX;
   const int npx = npix - pix0 < PX ? (int)(npix - pix0) : PX;
@@ -304,7 +424,7 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 8 ? 1 : Q <= 8 && NF 
     } else {
       TAcc<R> acc[4];
 #pragma unroll
-      for (int n1 = 0; n1 < 4; ++n1) tacc_zero(acc[n1]);
+      for (int n1 = 0; n1 < 4; ++n1) tacc_start(acc[n1], means + (n2 + Q * n1) * kMeanStride);
       for (int j = 0; j < pp.c; ++j) {
         const typename RT<R>::V4* Mj = M + (size_t)j * N + i;
         typename RT<R>::V4 m[4];
@@ -323,6 +443,15 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 8 ? 1 : Q <= 8 && NF 
 #pragma unroll
       for (int n1 = 0; n1 < 4; ++n1) pten_of(ten[n1], acc[n1], literal);
     }
+  }
+  if constexpr (SRC == 1) {
+    // (the means come while N_t does, and are taken off when both are here)
+    cp_async_wait_all();
+    __syncthreads();
+    if (px < npx)
+#pragma unroll
+      for (int n1 = 0; n1 < 4; ++n1)
+        pten_less(ten[n1], mean_s + (n2 + Q * n1) * kMeanStride);
   }
   const size_t fstride = (size_t)ns * npix;
   const int rot = kb & 3;  // s1 = 0 takes output kb mod 4 of the 4-point transform
@@ -395,21 +524,50 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 8 ? 1 : Q <= 8 && NF 
 }
 
 // Images of the angles of a batch from their transformed planes: per pixel
-// its two planes (b - kb mod nz) of the three fields, the constant left out
-// of p before the transform returned at q = 0 (its x and y parts per angle),
-// the projection and the interpolation; written in fftshift order.  A thread
+// its two planes (b - kb mod nz) of the three fields, what was left out of p
+// before the transform returned at q = 0 (the constant's x and y parts per
+// angle, and the slices' means, null: none), the projection and the interpolation; written in fftshift order.  A thread
 // takes AP angles of one pixel, so the 32-byte geometry is read once for
-// them; planes has kstride = 3 ns npix complex per angle.
+// them (q = 0 has a block of its own, which costs the others no registers);
+// planes has kstride = 3 ns npix complex per angle.
 template <typename R, int AP>
 __global__ void __launch_bounds__(256) k_plane_images(const typename RT<R>::C* __restrict__ planes,
                                                       int nx, int ny, int nz, int kb, int ns,
                                                       const Geo<R>* __restrict__ geo,
                                                       const __grid_constant__ ImageDc<R> dc,
-                                                      R* __restrict__ imgs) {
+                                                      const R* __restrict__ means, int literal,
+                                                      int from_nt, R* __restrict__ imgs) {
   using C = typename RT<R>::C;
   const long long npix = (long long)nx * ny;
-  const long long pix = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (pix >= npix) return;
+  const size_t fstride = (size_t)ns * npix, kstride = 3 * fstride;
+  if (blockIdx.x == 0) {  // q = 0, an angle per thread: with what was left out
+    if (blockIdx.y > 0) return;
+    __shared__ double sum[kMeanVals];
+    if (means) means_total<R>(means, nz, npix, sum);
+    const int a = threadIdx.x;
+    if (a >= dc.n) return;
+    PTen<R> total;
+    pten_zero(total);
+    if (means) means_pten(sum, literal != 0, from_nt != 0, total);
+    const Geo<R> g = geo[0];
+    const int s0 = g.b0 < kb ? g.b0 - kb + nz : g.b0 - kb, s1 = g.b1 < kb ? g.b1 - kb + nz : g.b1 - kb;
+    const C* src = planes + a * kstride;
+    C d[3], v0[3], v1[3];
+    p_from_pten(total, dc.ce[a], dc.se[a], dc.c2[a], dc.s2[a], literal != 0, d);
+    d[0].x += dc.x[a];
+    d[1].x += dc.y[a];
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      v0[f] = src[f * fstride + (size_t)s0 * npix];
+      v1[f] = src[f * fstride + (size_t)s1 * npix];
+      if (g.b0 == 0) v0[f] = cadd(v0[f], d[f]);
+      if (g.b1 == 0) v1[f] = cadd(v1[f], d[f]);
+    }
+    imgs[(size_t)a * npix + (size_t)(ny / 2) * nx + nx / 2] = ewald_value<R>(g, v0, v1);
+    return;
+  }
+  const long long pix = (long long)(blockIdx.x - 1) * blockDim.x + threadIdx.x;
+  if (pix == 0 || pix >= npix) return;
   const Geo<R> g = geo[pix];
   const int my = (int)(pix / nx), mx = (int)(pix - (long long)my * nx);
   int sy = my + ny / 2, sx = mx + nx / 2;
@@ -417,7 +575,6 @@ __global__ void __launch_bounds__(256) k_plane_images(const typename RT<R>::C* _
   if (sx >= nx) sx -= nx;
   R* dst = imgs + (size_t)sy * nx + sx;
   const int a0 = blockIdx.y * AP;
-  const size_t fstride = (size_t)ns * npix, kstride = 3 * fstride;
   int s0 = g.b0 - kb, s1 = g.b1 - kb;
   if (s0 < 0) s0 += nz;
   if (s1 < 0) s1 += nz;
@@ -433,10 +590,6 @@ __global__ void __launch_bounds__(256) k_plane_images(const typename RT<R>::C* _
       for (int f = 0; f < 3; ++f) {
         v0[f] = src[f * fstride + (size_t)s0 * npix];
         v1[f] = src[f * fstride + (size_t)s1 * npix];
-      }
-      if (pix == 0) {
-        if (g.b0 == 0) v0[0].x += dc.x[a], v0[1].x += dc.y[a];
-        if (g.b1 == 0) v1[0].x += dc.x[a], v1[1].x += dc.y[a];
       }
       val = ewald_value<R>(g, v0, v1);
     }
@@ -852,7 +1005,7 @@ PlShape pl_shape(int nz, int kb, int ns) {
 template <typename R, int SRC, int SB, bool EVEN>
 cudaError_t pol_planes_sb(const void* M, const void* nt, const void* dir, long long npix, int nz,
                           const PolParams<R>& pp, const AngleBatch<R>& ang, void* out, int kb,
-                          int ns, const void* twz, cudaStream_t s) {
+                          int ns, const void* twz, const void* means, cudaStream_t s) {
   using C = typename RT<R>::C;
   using F = Folded<C>;
   const PlShape sh = pl_shape(nz, kb, ns);
@@ -879,20 +1032,39 @@ cudaError_t pol_planes_sb(const void* M, const void* nt, const void* dir, long l
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)((npix + PX - 1) / PX), kPlThreads, smem, s>>>(
       (const typename RT<R>::V4*)M, (const C*)nt, (const R*)dir, npix, nz, PX, A, kb, ns, pp, ang,
-      (C*)out, (const C*)twz);
+      (C*)out, (const C*)twz, (const R*)means);
   return cudaGetLastError();
 }
 
 // The linearity path's bins ([5][2][npix]) from the transformed planes of
-// N_t's entries: per pixel its two planes of each, the constant returned to
-// xx and yy at q = 0.
+// N_t's entries: per pixel its two planes of each; returned at q = 0 (by block
+// 0): the constant to xx and yy, and the slices' means (a, xy, b, xz, yz of the
+// lab frame's PTen are xx, xy, yy, xz, yz).
 template <typename R>
 __global__ void __launch_bounds__(256) k_bins5_planes(const typename RT<R>::C* __restrict__ planes,
                                                       long long npix, int nz, int kb, int ns,
                                                       const Geo<R>* __restrict__ geo, R dc,
+                                                      const R* __restrict__ means, int from_nt,
                                                       typename RT<R>::C* __restrict__ bins) {
-  const long long pix = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (pix >= npix) return;
+  using C = typename RT<R>::C;
+  const long long pix =
+      blockIdx.x == 0 ? 0 : (long long)(blockIdx.x - 1) * blockDim.x + threadIdx.x;
+  if (pix >= npix || (blockIdx.x > 0 && pix == 0)) return;
+  C d[5];
+#pragma unroll
+  for (int q = 0; q < 5; ++q) d[q] = RT<R>::mk(R(0), R(0));
+  if (blockIdx.x == 0) {
+    __shared__ double sum[kMeanVals];
+    means_total<R>(means, nz, npix, sum);
+    if (threadIdx.x > 0) return;
+    PTen<R> m;
+    means_pten(sum, false, from_nt != 0, m);
+    d[0] = RT<R>::mk(m.a[0] + dc, m.a[1]);
+    d[1] = RT<R>::mk(m.xy[0], m.xy[1]);
+    d[2] = RT<R>::mk(m.b[0] + dc, m.b[1]);
+    d[3] = RT<R>::mk(m.xz[0], m.xz[1]);
+    d[4] = RT<R>::mk(m.yz[0], m.yz[1]);
+  }
   const Geo<R> g = geo[pix];
   if (g.b0 < 0) return;  // off the sphere: the bins are not read
 #pragma unroll
@@ -901,9 +1073,8 @@ __global__ void __launch_bounds__(256) k_bins5_planes(const typename RT<R>::C* _
     const int s = bin < kb ? bin - kb + nz : bin - kb;
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-      typename RT<R>::C v = planes[((size_t)q * ns + s) * npix + pix];
-      if (pix == 0 && bin == 0 && (q == 0 || q == 2)) v.x += dc;
-      bins[(size_t)(2 * q + b) * npix + pix] = v;
+      const C v = planes[((size_t)q * ns + s) * npix + pix];
+      bins[(size_t)(2 * q + b) * npix + pix] = bin == 0 ? cadd(v, d[q]) : v;
     }
   }
 }
@@ -911,39 +1082,41 @@ __global__ void __launch_bounds__(256) k_bins5_planes(const typename RT<R>::C* _
 template <typename R, int SRC, int Q, int NF = 3>
 cudaError_t pol_planes_fft(const void* M, const void* nt, const void* dir, long long npix,
                            const PolParams<R>& pp, const AngleBatch<R>& ang, void* out, int kb,
-                           int ns, const void* twz, cudaStream_t s) {
+                           int ns, const void* twz, const void* means, cudaStream_t s) {
   using C = typename RT<R>::C;
   using P = PlFft<R, Q>;
-  const size_t smem = (size_t)(NF == 3 ? P::A : 1) * 4 * NF * P::KS * sizeof(C);
+  const size_t smem = (SRC == 1 ? (size_t)4 * Q * kMeanStride * sizeof(R) : 0) +
+                      (size_t)(NF == 3 ? P::A : 1) * 4 * NF * P::KS * sizeof(C);
   auto kern = k_pol_planes_fft<R, SRC, Q, NF>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)((npix + P::PX - 1) / P::PX), kPlThreads, smem, s>>>(
       (const typename RT<R>::V4*)M, (const C*)nt, (const R*)dir, npix, kb, ns, pp, ang, (C*)out,
-      (const C*)twz);
+      (const C*)twz, (const R*)means);
   return cudaGetLastError();
 }
 
 template <typename R, int SRC, bool EVEN>
 cudaError_t pol_planes_src(const void* M, const void* nt, const void* dir, long long npix, int nz,
                            const PolParams<R>& pp, const AngleBatch<R>& ang, void* out, int kb,
-                           int ns, const void* twz, cudaStream_t s) {
+                           int ns, const void* twz, const void* means, cudaStream_t s) {
+  if (nz > 1 && !means) return cudaErrorInvalidValue;
   if constexpr (EVEN) {
     // FP64 at nz = 128 would not fit its registers (64 of data, 96 of sums)
     switch (nz) {
-      case 8: return pol_planes_fft<R, SRC, 2>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, s);
-      case 16: return pol_planes_fft<R, SRC, 4>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, s);
-      case 32: return pol_planes_fft<R, SRC, 8>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, s);
-      case 64: return pol_planes_fft<R, SRC, 16>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, s);
+      case 8: return pol_planes_fft<R, SRC, 2>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, means, s);
+      case 16: return pol_planes_fft<R, SRC, 4>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, means, s);
+      case 32: return pol_planes_fft<R, SRC, 8>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, means, s);
+      case 64: return pol_planes_fft<R, SRC, 16>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, means, s);
       case 128:
         if constexpr (sizeof(R) == 4)
-          return pol_planes_fft<R, SRC, 32>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, s);
+          return pol_planes_fft<R, SRC, 32>(M, nt, dir, npix, pp, ang, out, kb, ns, twz, means, s);
         break;
       default: break;
     }
   }
 #define RSX_PL(B) \
-  case B: return pol_planes_sb<R, SRC, B, EVEN>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, s);
+  case B: return pol_planes_sb<R, SRC, B, EVEN>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, means, s);
   switch (pl_shape(nz, kb, ns).SB) {
     RSX_PL(2) RSX_PL(3) RSX_PL(4) RSX_PL(5) RSX_PL(6) RSX_PL(7) RSX_PL(8)
     default: return cudaErrorInvalidValue;
@@ -959,14 +1132,14 @@ bool lin_planes_fits(int precision, int nz) {
 template <typename R>
 cudaError_t launch_lin_planes(const void* M, const void* nt, long long npix, int nz,
                               const PolParams<R>& pp, void* out, int kb, int ns, const void* twz,
-                              cudaStream_t s) {
-  if (!lin_planes_fits(8 * (int)sizeof(R), nz) || ns < 1 || ns > nz || kb < 0 || kb >= nz)
+                              const void* means, cudaStream_t s) {
+  if (!means || !lin_planes_fits(8 * (int)sizeof(R), nz) || ns < 1 || ns > nz || kb < 0 || kb >= nz)
     return cudaErrorInvalidValue;
   AngleBatch<R> none;
   memset(&none, 0, sizeof(none));
 #define RSX_LIN(Q)                                                                                \
-  return nt ? pol_planes_fft<R, 1, Q, 5>(M, nt, nullptr, npix, pp, none, out, kb, ns, twz, s)     \
-            : pol_planes_fft<R, 0, Q, 5>(M, nt, nullptr, npix, pp, none, out, kb, ns, twz, s);
+  return nt ? pol_planes_fft<R, 1, Q, 5>(M, nt, nullptr, npix, pp, none, out, kb, ns, twz, means, s) \
+            : pol_planes_fft<R, 0, Q, 5>(M, nt, nullptr, npix, pp, none, out, kb, ns, twz, means, s);
   switch (nz) {
     case 8: RSX_LIN(2)
     case 16: RSX_LIN(4)
@@ -981,11 +1154,13 @@ cudaError_t launch_lin_planes(const void* M, const void* nt, long long npix, int
 
 template <typename R>
 cudaError_t launch_bins5_planes(const void* planes, int nx, int ny, int nz, int kb, int ns,
-                                const Geo<R>* geo, double dc, void* bins, cudaStream_t s) {
+                                const Geo<R>* geo, double dc, const void* means, bool from_nt,
+                                void* bins, cudaStream_t s) {
   using C = typename RT<R>::C;
   const long long npix = (long long)nx * ny;
-  k_bins5_planes<R><<<(unsigned)((npix + 255) / 256), 256, 0, s>>>((const C*)planes, npix, nz, kb, ns,
-                                                                   geo, (R)dc, (C*)bins);
+  if (!means) return cudaErrorInvalidValue;
+  k_bins5_planes<R><<<(unsigned)((npix + 255) / 256) + 1, 256, 0, s>>>(
+      (const C*)planes, npix, nz, kb, ns, geo, (R)dc, (const R*)means, from_nt ? 1 : 0, (C*)bins);
   return cudaGetLastError();
 }
 
@@ -999,31 +1174,45 @@ bool pol_planes_fits(int precision, int nz, int kb, int ns) {
 template <typename R>
 cudaError_t launch_pol_planes(const void* M, const void* nt, const void* dir, long long npix,
                               int nz, const PolParams<R>& pp, const AngleBatch<R>& ang, void* out,
-                              int kb, int ns, const void* twz, cudaStream_t s) {
+                              int kb, int ns, const void* twz, const void* means, cudaStream_t s) {
   if (nz < 1 || nz > kMaxPlanesNz || ns < 1 || ns > nz || kb < 0 || kb >= nz || ang.n < 1 ||
       ang.n > kMaxAngleBatch)
     return cudaErrorInvalidValue;
   if (nz % 2)
-    return nt ? pol_planes_src<R, 1, false>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, s)
-              : pol_planes_src<R, 0, false>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, s);
-  return nt ? pol_planes_src<R, 1, true>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, s)
-            : pol_planes_src<R, 0, true>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, s);
+    return nt ? pol_planes_src<R, 1, false>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, means, s)
+              : pol_planes_src<R, 0, false>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, means, s);
+  return nt ? pol_planes_src<R, 1, true>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, means, s)
+            : pol_planes_src<R, 0, true>(M, nt, dir, npix, nz, pp, ang, out, kb, ns, twz, means, s);
 }
 
 template <typename R>
 cudaError_t launch_plane_images(const void* planes, int nx, int ny, int nz, int kb, int ns,
-                                const Geo<R>* geo, const ImageDc<R>& dc, void* imgs,
-                                cudaStream_t s) {
+                                const Geo<R>* geo, const ImageDc<R>& dc, const void* means,
+                                bool from_nt, bool literal, void* imgs, cudaStream_t s) {
   using C = typename RT<R>::C;
   const long long npix = (long long)nx * ny;
-  const unsigned gx = (unsigned)((npix + 255) / 256);
+  const unsigned gx = (unsigned)((npix + 255) / 256) + 1;  // block 0: q = 0
   // four angles per thread once one angle's pixels fill the chip
-  if (npix >= (1 << 18))
-    k_plane_images<R, 4><<<dim3(gx, (dc.n + 3) / 4), 256, 0, s>>>((const C*)planes, nx, ny, nz, kb,
-                                                                  ns, geo, dc, (R*)imgs);
-  else
-    k_plane_images<R, 1><<<dim3(gx, dc.n), 256, 0, s>>>((const C*)planes, nx, ny, nz, kb, ns, geo,
-                                                        dc, (R*)imgs);
+  const bool big = npix >= (1 << 18);
+  auto kern = big ? k_plane_images<R, 4> : k_plane_images<R, 1>;
+  kern<<<dim3(gx, big ? (dc.n + 3) / 4 : dc.n), 256, 0, s>>>(
+      (const C*)planes, nx, ny, nz, kb, ns, geo, dc, (const R*)means, literal ? 1 : 0,
+      from_nt ? 1 : 0, (R*)imgs);
+  return cudaGetLastError();
+}
+
+size_t slice_means_bytes(int precision, int nz) {
+  return (size_t)nz * kMeanStride * (precision / 8);
+}
+
+template <typename R>
+cudaError_t launch_slice_means(const void* M, const void* nt, const void* dir, long long npix,
+                               int nz, const PolParams<R>& pp, bool literal, void* means,
+                               cudaStream_t s) {
+  if (!means || nz < 1 || npix < 1) return cudaErrorInvalidValue;
+  k_slice_means<R><<<nz, kMeanSample<R>, 0, s>>>((const typename RT<R>::V4*)M,
+                                                 (const typename RT<R>::C*)nt, (const R*)dir, npix,
+                                                 nz, pp, literal ? 1 : 0, (R*)means);
   return cudaGetLastError();
 }
 
@@ -1105,15 +1294,18 @@ cudaError_t launch_x_planes(void* data, int nx, int ny, int ns, long long nfield
 #define RSX_INST(R)                                                                               \
   template cudaError_t launch_pol_planes<R>(const void*, const void*, const void*, long long, int, \
                                             const PolParams<R>&, const AngleBatch<R>&, void*, int, \
-                                            int, const void*, cudaStream_t);                      \
+                                            int, const void*, const void*, cudaStream_t);         \
   template cudaError_t launch_lin_planes<R>(const void*, const void*, long long, int,             \
                                             const PolParams<R>&, void*, int, int, const void*,    \
-                                            cudaStream_t);                                        \
+                                            const void*, cudaStream_t);                           \
   template cudaError_t launch_bins5_planes<R>(const void*, int, int, int, int, int,               \
-                                              const Geo<R>*, double, void*, cudaStream_t);        \
+                                              const Geo<R>*, double, const void*, bool, void*,    \
+                                              cudaStream_t);                                      \
   template cudaError_t launch_plane_images<R>(const void*, int, int, int, int, int,               \
-                                              const Geo<R>*, const ImageDc<R>&, void*,            \
-                                              cudaStream_t);
+                                              const Geo<R>*, const ImageDc<R>&, const void*, bool, \
+                                              bool, void*, cudaStream_t);                               \
+  template cudaError_t launch_slice_means<R>(const void*, const void*, const void*, long long,    \
+                                             int, const PolParams<R>&, bool, void*, cudaStream_t);
 RSX_INST(float)
 RSX_INST(double)
 #undef RSX_INST

@@ -59,6 +59,37 @@ template <typename R> __device__ __forceinline__ void tacc_zero(TAcc<R>& a) {
   for (int q = 0; q < 5; ++q) a.t[q][0] = a.t[q][1] = R(0);
 }
 
+// A row of k_slice_means: the sums' mean over a slice in the order t, as, aw - 1
+// (from N_t: PTen's, see pten_less).  Starting the sums at minus the mean takes it off without an operation (aw -
+// 1 is formed after the sum, so aw starts at minus the mean of aw - 1).
+constexpr int kMeanStride = 16;
+template <typename R> struct MeanRow {
+  R t[5][2], as[2], aw1;
+};
+__device__ __forceinline__ void mean_load(const float* m, MeanRow<float>& v) {
+  const float4* q = reinterpret_cast<const float4*>(m);
+  const float4 a = q[0], b = q[1], c = q[2];
+  v.t[0][0] = a.x, v.t[0][1] = a.y, v.t[1][0] = a.z, v.t[1][1] = a.w;
+  v.t[2][0] = b.x, v.t[2][1] = b.y, v.t[3][0] = b.z, v.t[3][1] = b.w;
+  v.t[4][0] = c.x, v.t[4][1] = c.y, v.as[0] = c.z, v.as[1] = c.w;
+  v.aw1 = m[12];
+}
+__device__ __forceinline__ void mean_load(const double* m, MeanRow<double>& v) {
+  const double2* q = reinterpret_cast<const double2*>(m);
+#pragma unroll
+  for (int e = 0; e < 5; ++e) v.t[e][0] = q[e].x, v.t[e][1] = q[e].y;
+  v.as[0] = q[5].x, v.as[1] = q[5].y, v.aw1 = m[12];
+}
+template <typename R> __device__ __forceinline__ void tacc_start(TAcc<R>& a, const R* mean) {
+  MeanRow<R> v;
+  mean_load(mean, v);
+  a.aw = -v.aw1;
+  a.as[0] = -v.as[0];
+  a.as[1] = -v.as[1];
+#pragma unroll
+  for (int q = 0; q < 5; ++q) a.t[q][0] = -v.t[q][0], a.t[q][1] = -v.t[q][1];
+}
+
 // Adds component j with the director (dx, dy, dz).
 template <typename R>
 __device__ __forceinline__ void tacc_add_d(TAcc<R>& acc, R v, R s, R dx, R dy, R dz,
@@ -130,6 +161,19 @@ __device__ __forceinline__ void pten_of(PTen<R>& p, TAcc<R>& acc, bool literal) 
     acc.t[q][1] *= inv;
   }
   pten_of(p, ar, acc.t, literal);
+}
+// Less a slice's mean of PTen (k_slice_means from N_t; t holds a, xy, b, xz, yz).
+template <typename R> __device__ __forceinline__ void pten_less(PTen<R>& p, const R* mean) {
+  MeanRow<R> m;
+  mean_load(mean, m);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    p.a[i] -= m.t[0][i];
+    p.xy[i] -= m.t[1][i];
+    p.b[i] -= m.t[2][i];
+    p.xz[i] -= m.t[3][i];
+    p.yz[i] -= m.t[4][i];
+  }
 }
 // p for one angle: c, s = cos a, sin a; c2, s2 = cos 2a, sin 2a.
 template <typename R>

@@ -44,3 +44,39 @@ def test_rotation_weights_keep_all_fraction_bits(rsx, bits, prec):
     inside = (dy < -1) & (dy > -n // 2)
     tol = 5 * 2.0 ** -24 if prec == 32 else 5 * 2.0 ** -53 + 2.0 ** (bits - 49)
     assert np.all(np.abs(got - want)[inside] <= tol * want[inside]), (got, want)
+
+
+# (nz, ny, nx): register-FFT stacks, folded ones (even, odd), the pass of 1024-voxel tiles
+FAINT = [(16, 24, 20), (45, 20, 24), (62, 20, 18), (64, 20, 24), (128, 12, 20), (32, 101, 96),
+         (64, 75, 80)]
+
+
+# Algorithm 3 transforms z first for the register-FFT stacks alone
+@pytest.mark.parametrize("shape,alg", [(sh, a) for sh in FAINT for a in (1, 2, 3)
+                                       if a < 3 or sh[0] & (sh[0] - 1) == 0],
+                         ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else f"alg{v}")
+def test_a_uniform_background_leaves_no_rounding_in_faint_images(rsx, shape, alg):
+    """One unaligned material with v = 0.5 + 0.01 x, x uniform and white: the
+    contrast v^2 - 1 has a mean near -0.75 and a standard deviation s of about
+    0.003 per voxel.  Forming it and dividing it by 4 pi rounds twice at that
+    size (at most 2^-25 each, root mean square 2^-25 sqrt(2/3) together), and
+    a white error below a white signal is the image's relative L2 error away
+    from q = 0; the transforms of a field without its mean add far less.  A
+    mean that is still there when z is transformed adds nz roundings of its
+    size to bin 0 and grows the error as sqrt(nz).  Bound: 2 2^-25 / s."""
+    from oracle import cyrsoxs_oracle as O
+    from paper_2209_13121_gb300 import synth
+    nz, ny, nx = shape
+    M = np.zeros((1, nz, ny, nx, 4), dtype=np.float32)
+    M[..., 0] = 0.5 + 0.01 * np.random.default_rng(5).random((nz, ny, nx))
+    K = synth.optical_constants([285.0], 1, seed=6)
+    s = float(np.std(M[..., 0].astype(np.float64) ** 2))
+    ref = O.scatter_one_angle(M.astype(np.float64), K[0], 285.0, 5.0, 0.0)
+    iy, ix = np.meshgrid(np.arange(ny) - ny // 2, np.arange(nx) - nx // 2, indexing="ij")
+    far = np.hypot(ix, iy) > 0.5
+    with rsx.Context(nx, ny, nz, 1, 5.0, algorithm=alg) as ctx:
+        ctx.set_morphology(torch.from_numpy(M).cuda())
+        ctx.set_optical_constants([285.0], K)
+        got = ctx.run(rotation=False)[0].astype(np.float64)
+    err = np.linalg.norm((got - ref)[far]) / np.linalg.norm(ref[far])
+    assert err <= 2 * 2.0 ** -25 / s, (err, 2.0 ** -25 / s)
