@@ -691,17 +691,7 @@ int x_pass(rsx_context* c, const PolParams<R>& pp, cudaStream_t s) {
   return RSX_OK;
 }
 
-bool planes_plan(const rsx_context* c, int ie, ZPlan* zp);
-// Whether one image alone is worth the planes path, whose pass over the
-// morphology is then shared by no other angle: FP64 (256 x 256 x 32, c = 3:
-// 1199 -> 917 us), lateral sizes that are not powers of two (300 x 300 x 45:
-// 598 -> 232), and from 2^21 voxels on (256 x 256 x 64: 143 -> 102; 256 x 256 x 16:
-// 45 -> 51, so not below) except for FP32 rows of 512 or 1024 points, whose
-// fused one-angle passes stay ahead (1024 x 1024 x 16: 331 against 407).
-bool single_on_planes(const rsx_config& g) {
-  if (g.precision == 64 || (g.nx & (g.nx - 1)) || (g.ny & (g.ny - 1))) return true;
-  return g.nx != 512 && g.nx != 1024 && (long long)g.nx * g.ny * g.nz >= (1 << 21);
-}
+bool planes_plan(const rsx_context* c, int ie, int nang, bool single, ZPlan* zp);
 template <typename R>
 int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang, int rotation,
                       const ZPlan& zp, cudaStream_t s, const double* one = nullptr,
@@ -722,7 +712,7 @@ int scatter_angle(rsx_context* c, int ie, double alpha, void* img, cudaStream_t 
     return RSX_OK;
   }
   ZPlan zp;
-  if (try_planes && single_on_planes(g) && planes_plan(c, ie, &zp))
+  if (try_planes && planes_plan(c, ie, 1, true, &zp))
     return run_energy_planes<R>(c, ie, 0.0, 0.0, 1, 1, zp, s, &alpha, img);
   if (g.algorithm == 2 && (rc = ensure_nt<R>(c, ie, s))) return rc;
   if ((rc = x_pass<R>(c, make_params<R>(c, ie, alpha, 0), s))) return rc;
@@ -967,38 +957,107 @@ static bool zfirst_plan(const rsx_context* c, int ie, ZPlan* zp) {
   return zfirst_plan_of(g, c->kx, wavenumber(c->energies[ie]), zp);
 }
 
-// The planes path's plan: the z-first path's where that serves the energy
-// (its p and z-FFT pass also takes other lateral sizes, FP32 Algorithm 1);
-// else the run of bins the pixels read (all of them where the run would wrap
-// onto itself) and the angles whose planes fit in p.
-// FP64: the general pass evaluates the kept bins one by one, 6 ns fused
-// multiply-adds per voxel and angle, and the lateral transforms of the kept
-// planes take ~230 ns / nz; it pays while that is below what transforming
-// every slice and evaluating the morphology per angle takes (~330; FP64
-// arithmetic is the bound).  FP32 with rows the x-first passes serve (x and
-// p fused, then y and the two bins fused: half the passes over p): while at
-// most 3/4 of the bins are kept.
+// Whether nang angles of one energy (single: one image, not rotated) are
+// better served by the planes path (plan zp) or by the x-first passes: both
+// sides' times in us, fitted to 9538 measurements of both (GB300; 1 to 255
+// slices, rows of 24 to 4096 points, 1 to 8 materials, 1 to 24 angles, voxels of
+// 1 to 10 nm, both precisions, Algorithms 1 and 2; nine in ten within 20 to 25 %).
+// The planes path shares a read of the morphology and its sums among a batch
+// and transforms only the kept planes laterally, but where nz has no register
+// FFT it spends up to 2 ns multiply-adds per voxel, field and angle on their z
+// transform, and with a batch of one angle (one image, or a grid whose
+// workspace holds no more) it shares nothing.  What the choice is worth,
+// x-first against planes: 128 x 128 x 16, 24 angles 1.0 and 0.12 ms; 256 x 256 x
+// 64, one angle 145 and 112 us; but 256 x 256 x 255 at 2 nm (120 bins), 24 angles
+// 11.9 and 44.3 ms, one angle 0.51 and 2.6; 256 x 2048 x 9 (a batch holds one
+// angle), 24 angles 3.8 and 5.7 ms.  Taking the planes path is then slower by
+// more than 10 % than the other in 0.7 % of the measured calls (1.4 times at
+// most), not taking it in 1.5 %.
 namespace {
-bool planes_plan(const rsx_context* c, int ie, ZPlan* zp) {
+// the largest prime factor of n, if the transforms sum over it (above 13)
+int long_prime(int n) {
+  int p = 1;
+  for (int f = 2; f * f <= n; ++f)
+    while (n % f == 0) n /= f, p = f;
+  if (n > p) p = n;
+  return p > 13 ? p : 0;
+}
+
+bool planes_pay(const rsx_config& g, const ZPlan& zp, int nang, bool single) {
+  const bool f32 = g.precision == 32;
+  auto rank = [](int n) {  // 0: 512, 1024, 2048; 1: other powers of two; 2: the rest
+    return n & (n - 1) ? 2 : n == 512 || n == 1024 || n == 2048 ? 0 : 1;
+  };
+  const int rx = rank(g.nx), ry = rank(g.ny);
+  // one FP32 image of a small power-of-two grid: three launches against six
+  if (f32 && single && rx < 2 && ry < 2 && (long long)g.nx * g.ny * g.nz < (1 << 21) && !zp.film)
+    return false;
+  // million pixels, voxels, kept plane elements; angles and batches; components
+  // whose morphology is read per batch
+  const double npix = 1e-6 * g.nx * g.ny, M = npix * g.nz, P = npix * zp.ns;
+  const double n = nang, b = (nang + zp.kz - 1) / zp.kz;
+  const bool a1 = g.algorithm == 1;
+  const double c = a1 ? g.n_components : 0, prime = long_prime(g.nx) + long_prime(g.ny);
+  const rsx::PlanesWork w =
+      rsx::pol_planes_work(g.precision, g.nz, zp.kb, zp.ns, nang < zp.kz ? nang : zp.kz);
+  double planes, rows;
+  if (f32) {
+    static const double lateral[3][3] = {{15, 17, 26}, {17, 24, 37}, {26, 37, 45}};
+    const double lat = n * (lateral[rx][ry] + 2.2 * prime) * P;
+    planes = lat + (w.fft ? 13 * !single + b * (24 + (4.9 * c + (a1 ? 3.8 : 7.6)) * M) +
+                                n * (6.9 * npix + 2.6 * M)
+                          : 11 * !single + b * (29 + (8.5 * c + (a1 ? 4.5 : 12) + 62.0 / w.px) * M) +
+                                n * (28 * npix +
+                                     (w.slots * (w.lone ? 45.4 : 1.35) + 0.137 * w.sums) * M));
+    // rows with passes of their own, p overlapping the transform: 512 and 1024
+    // points (one image: a pass for one angle), 2048 in Algorithm 1's runs
+    const bool tuned = g.nx == 512 || g.nx == 1024 || (g.nx == 2048 && a1 && !single);
+    const bool yz = rsx::yz_fusable(g.nx, g.ny, g.nz);
+    const double voxel = tuned            ? (single && a1 ? (yz ? 14 : ry == 2 ? 19 : 17)
+                                                          : (yz ? 18 : ry == 2 ? 28 : 22))
+                         : rx == 2        ? (ry == 2 ? 47 : 44)
+                         : g.nx >= 2048   ? (ry == 2 ? 55 : g.nx == 2048 ? 41 : 45)
+                         : ry == 2        ? 33
+                                          : 22.4;
+    const int kx = tuned && a1 && !single ? angle_batch_of(&g) : 1;
+    rows = 10 * !single + n * (20 + 0.35 * g.nz + 20 * npix + (voxel + 2.3 * prime) * M) +
+           (double)((nang + kx - 1) / kx) * 1.8 * c * M;
+  } else {
+    const int cls = rx == 2 || ry == 2 ? 2 : g.nx >= 1024 || g.ny >= 1024 ? 1 : 0;
+    static const double lateral[2][3] = {{305, 370, 462}, {230, 320, 412}};
+    static const double voxel[3] = {317, 450, 488};
+    const double lat = n * (lateral[w.fft][cls] + (w.fft ? 41 : 37) * prime) * P;
+    planes = lat + (w.fft ? 19 * !single + b * (64 + (64 * c + (a1 ? 47 : 29)) * M) +
+                                n * (39 * npix + 116 * M)
+                          : 22 * !single + b * (72 + (66 * c + (a1 ? 54 : 25) + 84.0 / w.px) * M) +
+                                n * (72 * w.slots + 3.4 * w.sums) * M);
+    rows = 10 * !single +
+           n * (66 + 4.4 * g.nz + 137 * npix + (voxel[cls] + 52 * c + 37 * prime) * M);
+  }
+  return planes * (w.fft ? 1.0 : 1.02) < rows;
+}
+
+// The planes path's plan for nang angles (single: one image, not rotated): the
+// z-first path's where that serves a run of the energy (its p and z-FFT pass
+// also takes other lateral sizes, FP32 Algorithm 1); else the run of bins the
+// pixels read (all of them where the run would wrap onto itself) and the
+// angles whose planes fit in p.  False where the x-first passes serve better.
+bool planes_plan(const rsx_context* c, int ie, int nang, bool single, ZPlan* zp) {
   const rsx_config& g = c->cfg;
   if (!planes_cfg(&g) || !c->imgs || ie < 0 || ie >= (int)c->energies.size()) return false;
   if (zfirst_plan(c, ie, zp)) {
     zp->zfft = true;
-    return true;
+    return !single || planes_pay(g, *zp, 1, true);
   }
   const int blo = lowest_bin(g, wavenumber(c->energies[ie]));
   zp->ns = 2 - blo < g.nz ? 2 - blo : g.nz;
   zp->kb = zp->ns == g.nz ? 0 : ((blo % g.nz) + g.nz) % g.nz;
-  const bool x_first =
-      x_multi_cap(&g) || (g.precision == 32 && g.algorithm == 2 && (g.nx == 512 || g.nx == 1024));
   // a film needs no z transform: the multi-angle x pass forms p x-transformed
   if (g.nz == 1 && x_multi_cap(&g) && y_tuned(&g) && c->n_sm > 0 && ((uintptr_t)c->M & 15) == 0) {
     zp->film = true;
     zp->kz = c->kx < x_multi_cap(&g) ? c->kx : x_multi_cap(&g);
-    return true;
+    return planes_pay(g, *zp, nang, single);
   }
-  if (x_first && 4 * zp->ns > 3 * g.nz) return false;
-  if (g.precision == 64 && 6.0 * zp->ns + 230.0 * zp->ns / g.nz > 330.0) return false;
   // the z-first pass's tiles of 1024 / nz pixels of a row, at least two per SM
   zp->zfft = g.precision == 32 && g.algorithm == 1 && (g.nz == 32 || g.nz == 64 || g.nz == 128) &&
              g.nx % (1024 / g.nz) == 0 && c->n_sm > 0 && ((uintptr_t)c->M & 15) == 0 &&
@@ -1007,7 +1066,7 @@ bool planes_plan(const rsx_context* c, int ie, ZPlan* zp) {
   const long long kz = c->p_cap / (3LL * zp->ns * c->npix);
   const int cap = zp->zfft ? rsx::kMaxXAngles : rsx::kMaxAngleBatch;
   zp->kz = kz < cap ? (int)kz : cap;
-  return zp->kz >= 1;
+  return zp->kz >= 1 && planes_pay(g, *zp, nang, single);
 }
 }  // namespace
 
@@ -1610,7 +1669,7 @@ template <typename R>
 int run_energy_angles(rsx_context* c, int ie, double start, double inc, int nang, int rotation,
                       cudaStream_t s) {
   ZPlan zp;
-  if (planes_plan(c, ie, &zp))
+  if (planes_plan(c, ie, nang, false, &zp))
     return run_energy_planes<R>(c, ie, start, inc, nang, rotation, zp, s);
   if constexpr (sizeof(R) == 4) {
     if ((c->kx > 1 || c->cfg.nx == 2048) && x_multi_cap(&c->cfg) && c->n_sm > 0 &&

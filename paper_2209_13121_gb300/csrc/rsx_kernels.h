@@ -335,6 +335,15 @@ cudaError_t launch_slice_means(const void* M, const void* nt, const void* dir, l
                                int nz, const PolParams<R>& pp, bool literal, void* means,
                                cudaStream_t s);
 bool pol_planes_fits(int precision, int nz, int kb, int ns);
+// What the pass does for a stack: its z transform by a register FFT (fft), or
+// else, per voxel and angle, thread slots for p and multiply-adds of the
+// folded sums, whether an SM holds one block alone (lone), pixels of a block.
+struct PlanesWork {
+  bool fft, lone;
+  double slots, sums;
+  int px;
+};
+PlanesWork pol_planes_work(int precision, int nz, int kb, int ns, int nang);
 template <typename R>
 cudaError_t launch_pol_planes(const void* M, const void* nt, const void* dir, long long npix,
                               int nz, const PolParams<R>& pp, const AngleBatch<R>& ang, void* out,

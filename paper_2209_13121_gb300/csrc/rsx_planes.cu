@@ -1002,37 +1002,49 @@ PlShape pl_shape(int nz, int kb, int ns) {
   return p;
 }
 
+// Its launch for nang angles: pixels of a block (its threads' folds in use,
+// whole 32-byte sectors per plane row), angles per step (up to 4 within ~100
+// KB, two FP32 blocks per SM, with the fewest idle threads in the last round
+// of the items), rounds of the items, shared memory.
+struct PlLaunch {
+  int PX, A, rounds;
+  size_t smem;
+};
+PlLaunch pl_launch(const PlShape& sh, bool even, size_t cs, int nang) {
+  PlLaunch l;
+  const int unit = 32 / (int)cs;
+  l.PX = (even ? kPlThreads : 2 * kPlThreads) / sh.H / unit * unit;
+  const size_t per = (size_t)sh.np * sh.H * 3 * l.PX * 2 * cs,
+               twb = (size_t)sh.H * sh.G * ((sh.SB + 1) & ~1) * cs;
+  l.A = 1;
+  double best = 0.0;
+  for (int a = 1; a <= 4 && a <= nang; ++a) {
+    const int items = a * 3 * sh.G * l.PX, rounds = (items + kPlThreads - 1) / kPlThreads;
+    if (a > 1 && (a * per + twb > 104 * 1024 || items >= 2048)) break;
+    const double eff = (double)items / (rounds * kPlThreads) + 0.02 * a;
+    if (eff > best) best = eff, l.A = a;
+  }
+  l.rounds = (l.A * 3 * sh.G * l.PX + kPlThreads - 1) / kPlThreads;
+  l.smem = l.A * per + twb;
+  return l;
+}
+
 template <typename R, int SRC, int SB, bool EVEN>
 cudaError_t pol_planes_sb(const void* M, const void* nt, const void* dir, long long npix, int nz,
                           const PolParams<R>& pp, const AngleBatch<R>& ang, void* out, int kb,
                           int ns, const void* twz, const void* means, cudaStream_t s) {
   using C = typename RT<R>::C;
-  using F = Folded<C>;
   const PlShape sh = pl_shape(nz, kb, ns);
-  // pixels of a block: its threads' folds in use, whole 32-byte sectors per plane row
-  constexpr int unit = 32 / (int)sizeof(C);
-  const int PX = (EVEN ? kPlThreads : 2 * kPlThreads) / sh.H / unit * unit;
-  if (PX < unit) return cudaErrorInvalidValue;
-  // angles per step: up to 4 within ~100 KB (two FP32 blocks per SM), the
-  // fewest idle threads in the last round of the items
-  const size_t per = (size_t)sh.np * sh.H * 3 * PX * sizeof(F),
-               twb = (size_t)sh.H * sh.G * ((SB + 1) & ~1) * sizeof(C);
-  int A = 1;
-  double best = 0.0;
-  for (int a = 1; a <= 4 && a <= ang.n; ++a) {
-    const int items = a * 3 * sh.G * PX, rounds = (items + kPlThreads - 1) / kPlThreads;
-    if (a > 1 && (a * per + twb > 104 * 1024 || items >= 2048)) break;
-    const double eff = (double)items / (rounds * kPlThreads) + 0.02 * a;
-    if (eff > best) best = eff, A = a;
-  }
-  if (3 * sh.G * PX >= 2048 || A * 3 * sh.G >= 2048) return cudaErrorInvalidValue;  // div_by's range
-  const size_t smem = nz == 1 ? 0 : A * per + twb;
+  const PlLaunch l = pl_launch(sh, EVEN, sizeof(C), ang.n);
+  if (l.PX < 1 || 3 * sh.G * l.PX >= 2048 || l.A * 3 * sh.G >= 2048)
+    return cudaErrorInvalidValue;  // (div_by's range)
+  const size_t smem = nz == 1 ? 0 : l.smem;
   auto kern = k_pol_planes<R, SRC, SB, EVEN>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)((npix + PX - 1) / PX), kPlThreads, smem, s>>>(
-      (const typename RT<R>::V4*)M, (const C*)nt, (const R*)dir, npix, nz, PX, A, kb, ns, pp, ang,
-      (C*)out, (const C*)twz, (const R*)means);
+  kern<<<(unsigned)((npix + l.PX - 1) / l.PX), kPlThreads, smem, s>>>(
+      (const typename RT<R>::V4*)M, (const C*)nt, (const R*)dir, npix, nz, l.PX, l.A, kb, ns, pp,
+      ang, (C*)out, (const C*)twz, (const R*)means);
   return cudaGetLastError();
 }
 
@@ -1162,6 +1174,23 @@ cudaError_t launch_bins5_planes(const void* planes, int nx, int ny, int nz, int 
   k_bins5_planes<R><<<(unsigned)((npix + 255) / 256) + 1, 256, 0, s>>>(
       (const C*)planes, npix, nz, kb, ns, geo, (R)dc, (const R*)means, from_nt ? 1 : 0, (C*)bins);
   return cudaGetLastError();
+}
+
+PlanesWork pol_planes_work(int precision, int nz, int kb, int ns, int nang) {
+  PlanesWork w;
+  memset(&w, 0, sizeof(w));
+  w.fft = nz == 1 || lin_planes_fits(precision, nz);
+  if (w.fft) return w;
+  const PlShape sh = pl_shape(nz, kb, ns);
+  const PlLaunch l =
+      pl_launch(sh, nz % 2 == 0, precision == 32 ? sizeof(float2) : sizeof(double2), nang);
+  if (l.PX < 1) return w;
+  const double vox = (double)l.PX * nz;
+  w.slots = kPlThreads * kPlVoxels / vox;
+  w.sums = (double)l.rounds * kPlThreads * sh.H * sh.SB / (l.A * vox);
+  w.lone = l.smem > 112 * 1024;
+  w.px = l.PX;
+  return w;
 }
 
 bool pol_planes_fits(int precision, int nz, int kb, int ns) {
