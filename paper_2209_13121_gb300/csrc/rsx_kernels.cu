@@ -2623,14 +2623,32 @@ __device__ __forceinline__ double rot_frac(long long f, double) {
   return (double)(f & ((1LL << 48) - 1)) * (1.0 / 281474976710656.0);
 }
 // Bilinear sample of img (fftshift order) at the source position (fx, fy),
-// 2^-48 fixed point; corners outside the grid count as zero.  No branches:
-// the corners' addresses are clamped and the value of an outside one dropped,
-// so that the samples of several angles or pixels can be in flight together.
+// 2^-48 fixed point; corners outside the grid count as zero.  FP32 has no
+// branches: the corners' addresses are clamped and the value of an outside one
+// dropped, so that the samples of several angles or pixels can be in flight
+// together.  FP64, whose arithmetic is the bound, skips what lies outside
+// (1024 x 1024, 91 angles: 2.64 ms, without branches 3.25).
 template <typename R>
 __device__ __forceinline__ R rotated_sample(const R* __restrict__ img, int nx, int ny, long long fx,
                                             long long fy) {
   const int x0 = (int)(fx >> 48), y0 = (int)(fy >> 48);
   const R tx = rot_frac(fx, R(0)), ty = rot_frac(fy, R(0));
+  if constexpr (sizeof(R) == 8) {
+    R val = R(0);
+#pragma unroll
+    for (int dy = 0; dy < 2; ++dy) {
+      const int yy = y0 + dy;
+      if (yy < 0 || yy >= ny) continue;
+      const R wy = dy ? ty : R(1) - ty;
+#pragma unroll
+      for (int dx = 0; dx < 2; ++dx) {
+        const int xx = x0 + dx;
+        if (xx < 0 || xx >= nx) continue;
+        val += wy * (dx ? tx : R(1) - tx) * __ldg(img + (size_t)yy * nx + xx);
+      }
+    }
+    return val;
+  }
   const int xa = min(max(x0, 0), nx - 1), xb = min(max(x0 + 1, 0), nx - 1);
   const R* ra = img + (size_t)min(max(y0, 0), ny - 1) * nx;
   const R* rb = img + (size_t)min(max(y0 + 1, 0), ny - 1) * nx;
@@ -2668,10 +2686,11 @@ __global__ void __launch_bounds__(kRotTile * kRotTile) k_rotate_acc(const R* __r
 // thread takes PY pixels of a column, kRotTile rows apart: the 64-bit
 // products of the source position are formed once for them (the others are
 // sums away), and 4 PY corner loads are in flight; with PY = 1 (images that
-// would not fill the chip otherwise) the angles go UA at a time instead.
-// What bounds it is the L1 lines a rotated row of pixels touches.  (Per angle
-// at 2048 x 2048: 21.1 -> 18.8 us; 182 angles at 128 x 128: 0.158 -> 0.124 ms;
-// four pixels per thread at 1024 x 1024 were slower, 0.82 -> 0.97 ms per 182.)
+// would not fill the chip otherwise) the angles go UA at a time instead (FP32;
+// FP64 takes one of each).  What bounds it in FP32 is the L1 lines a rotated
+// row of pixels touches.  (Per angle at 2048 x 2048: 21.1 -> 19.2 us; 182 angles
+// at 128 x 128: 0.158 -> 0.127 ms; four pixels per thread at 1024 x 1024 were
+// slower, 0.82 -> 0.97 ms per 182.)
 template <typename R, int PY, int UA>
 __global__ void __launch_bounds__(kRotTile * kRotTile) k_rotate_acc_many(
     const R* __restrict__ imgs, R* __restrict__ acc, int nx, int ny,
@@ -3453,9 +3472,13 @@ cudaError_t launch_ewald_linear_many(const void* bins, int nx, int ny, const Geo
   if (ab.n > kMaxAngleBatch) return cudaErrorInvalidValue;
   const long long npix = (long long)nx * ny;
   // 16 angles per thread once one angle's pixels fill the chip
-  const bool big = npix >= (1 << 17);
+  // (FP64 is bound by its arithmetic, not by the bins: 1024 x 1024, 91 angles
+  // 13.85 ms, 13.96 with 16 a thread)
+  const bool big = sizeof(R) == 4 && npix >= (1 << 17);
   const dim3 grid(grid1(npix, 256), big ? (ab.n + 15) / 16 : ab.n);
-  auto kern = big ? k_ewald_linear_many<R, 16> : k_ewald_linear_many<R, 1>;
+  auto kern = k_ewald_linear_many<R, 1>;
+  if constexpr (sizeof(R) == 4)
+    if (big) kern = k_ewald_linear_many<R, 16>;
   kern<<<grid, 256, 0, s>>>((const typename RT<R>::C*)bins, nx, ny, geo, ab, literal ? 1 : 0,
                             (R*)imgs);
   return cudaGetLastError();
@@ -3468,11 +3491,15 @@ cudaError_t launch_rotate_acc_many(const void* imgs, void* acc, int nx, int ny,
   if (ab.n > kMaxAngleBatch) return cudaErrorInvalidValue;
   const dim3 block(kRotTile, kRotTile);
   const long long npix = (long long)nx * ny;
-  const int py = kRotTile * (npix >= (1 << 21) ? 4 : 1);
+  // FP64: one angle of one pixel at a time (no sample computed for nothing)
+  const bool f32 = sizeof(R) == 4;
+  const int py = kRotTile * (f32 && npix >= (1 << 21) ? 4 : 1);
   const dim3 grid((nx + kRotTile - 1) / kRotTile, (ny + py - 1) / py);
-  auto kern = npix >= (1 << 21)   ? k_rotate_acc_many<R, 4, 1>
-              : npix >= (1 << 18) ? k_rotate_acc_many<R, 1, 1>
-                                  : k_rotate_acc_many<R, 1, 4>;
+  auto kern = k_rotate_acc_many<R, 1, 1>;
+  if constexpr (sizeof(R) == 4) {
+    if (npix >= (1 << 21)) kern = k_rotate_acc_many<R, 4, 1>;
+    else if (npix < (1 << 18)) kern = k_rotate_acc_many<R, 1, 4>;
+  }
   kern<<<grid, block, 0, s>>>((const R*)imgs, (R*)acc, nx, ny, ab, rotate ? 1 : 0);
   return cudaGetLastError();
 }
