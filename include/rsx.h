@@ -29,9 +29,9 @@
  *    the voxel edge in nm and integer division.
  *  - Supported sizes: nx and ny in [1, 4096], nz in [1, 65535],
  *    1 <= n_components <= RSX_MAX_COMPONENTS.  Any nx and ny are
- *    transformed exactly (mixed-radix passes; a prime factor p above 7 costs
+ *    transformed exactly (mixed-radix passes; a prime factor p above 13 costs
  *    an O(p) pass per element); the fastest kernels serve FP32 grids with nx
- *    and ny 512 or 1024.
+ *    and ny 512, 1024 or 2048.
  */
 #ifndef RSX_H
 #define RSX_H
@@ -85,7 +85,12 @@ typedef struct rsx_config {
                       /* or 1024 (up to 8) and nx = 2048 (up to 3; larger    */
                       /* values are lowered to that); elsewhere 1.  Each     */
                       /* angle's arithmetic is unchanged (Algorithm 1's      */
-                      /* angle loop, the morphology sums shared).            */
+                      /* angle loop, the morphology sums shared).  Where the */
+                      /* q_z planes alone are kept (rsx_create) the same     */
+                      /* buffers serve more angles per read, and a given     */
+                      /* value bounds the rest of that workspace, on any     */
+                      /* shape, in either precision and in Algorithm 2: 1    */
+                      /* holds one p and one image, the least memory.        */
 } rsx_config;
 
 #define RSX_MAX_ANGLE_BATCH 8
@@ -102,8 +107,10 @@ typedef struct rsx_context rsx_context;
  * pixel of the fused y-FFT + z pass (up to 4 partial slots of 3 x 2 x 16
  * bytes per pixel; 5 x 2 x 16 for Algorithm 3).  For Algorithms 1 and 2 with
  * nz <= 255 the p workspace is at least the lesser of 32 angles' p and 96 MB
- * (FP64: 1 GB),
- * and a batch of images (at most 64, 64 MB or one) is held.  *out
+ * (FP64: 1 GB), and a batch of images (at most 64, or 64 MB, unless the bins
+ * have room for them) is held; a given angle_batch k makes that at most k
+ * angles' p and as many images, and where the device has no room for the rest the context is
+ * created with one angle's p and one image.  *out
  * receives the handle.  Errors: RSX_ERR_INVALID (sizes, precision,
  * algorithm), RSX_ERR_OOM. */
 int rsx_create(const rsx_config* cfg, rsx_context** out);
@@ -117,12 +124,14 @@ int rsx_destroy(rsx_context* ctx);
 const char* rsx_last_error(void);
 
 /* Device bytes rsx_create would allocate for cfg, morphology copy included
- * (Tables 1 and 2, plus the buffers listed under rsx_create).  Returns 0 for
- * an invalid cfg. */
+ * (Tables 1 and 2, plus the buffers listed under rsx_create; less where it has
+ * to make do).  Returns 0 for an invalid cfg. */
 size_t rsx_workspace_bytes(const rsx_config* cfg);
 
-/* The angle batch in effect for ctx (rsx_config.angle_batch after the
- * default and the shape rules above), or -1 for a NULL context. */
+/* The angle batch in effect for ctx, in p buffers of 3 N complex
+ * (rsx_config.angle_batch after the default and the shape rules above; where
+ * planes are kept more angles share a read, see rsx_create), or -1 for a NULL
+ * context. */
 int rsx_angle_batch(const rsx_context* ctx);
 
 /* The z-first path of Algorithm 1 (FP32, nz = 32, 64 or 128, nx and ny =

@@ -912,26 +912,39 @@ static bool uses_means(const rsx_config* cfg) {
 }
 
 // Complex elements of the p workspace: one p (3 N) per angle of the batch; on
-// the planes path at least 32 angles' p or 96 MB (within the 126 MB L2, so
-// that the planes of a batch of a small grid pass from kernel to kernel
-// there), whichever is less.
-static long long p_elems(const rsx_config* cfg) {
+// the planes path at least 32 angles' p (the caller's angle_batch where given)
+// or 96 MB (FP32: within the 126 MB L2, so that the planes of a batch of a small
+// grid pass from kernel to kernel there; FP64, whose sums over the morphology
+// are the dear part: 1 GB), whichever is less.  least: what a context cannot do
+// without.
+static long long p_elems(const rsx_config* cfg, bool least = false) {
   const long long one = 3LL * cfg->nx * cfg->ny * cfg->nz, base = one * angle_batch_of(cfg);
-  if (!planes_cfg(cfg)) return base;
+  if (!planes_cfg(cfg) || least) return base;
   const long long pool = ((cfg->precision == 32 ? 96LL : 1024LL) << 20) /
                          (long long)complex_size(cfg->precision);
-  const long long want = 32 * one < pool ? 32 * one : pool;
+  const long long most = (cfg->angle_batch > 0 ? cfg->angle_batch : 32) * one;
+  const long long want = most < pool ? most : pool;
   return want > base ? want : base;
 }
 
 // Images held at once: a launch's worth for the linearity path; on the
-// planes path as many as the fused y+z pass's bins have room for, or 64 MB.
-static int image_batch(const rsx_config* cfg) {
+// planes path as many as the fused y+z pass's bins have room for, or 64 MB,
+// but with the caller's angle_batch no more than there are p's.  (One is held
+// anyway.)
+static int image_batch(const rsx_config* cfg, bool least = false) {
   if (cfg->algorithm == 3) return rsx::kMaxAngleBatch;
   if (!planes_cfg(cfg)) return 0;
   const long long img = (long long)cfg->nx * cfg->ny * (long long)real_size(cfg->precision);
-  const long long n = uses_yz(cfg) ? (long long)part_bytes(cfg) / img : (64LL << 20) / img;
-  return n < 1 ? 1 : n > rsx::kMaxAngleBatch ? rsx::kMaxAngleBatch : (int)n;
+  long long n = rsx::kMaxAngleBatch;
+  if (uses_yz(cfg)) {
+    if ((long long)part_bytes(cfg) / img < n) n = (long long)part_bytes(cfg) / img;
+  } else {
+    if ((64LL << 20) / img < n) n = (64LL << 20) / img;
+    const long long ps = p_elems(cfg) / (3LL * cfg->nx * cfg->ny * cfg->nz);
+    if (cfg->angle_batch > 0 && ps < n) n = ps;
+    if (least) n = 1;
+  }
+  return n < 1 ? 1 : (int)n;
 }
 
 namespace {
@@ -1088,7 +1101,7 @@ size_t rsx_workspace_bytes(const rsx_config* cfg) {
   b += (size_t)(cfg->nx + cfg->ny + cfg->nz) * Cs + sizeof(int);
   if (uses_yz(cfg)) b += part_bytes(cfg);            // fused y + z pass: bins
   if (uses_yz(cfg) || y_tuned(cfg)) b += 2 * (size_t)npix;  // lower bin of every pixel
-  if (!uses_yz(cfg) || cfg->algorithm == 3)
+  if ((!uses_yz(cfg) && image_batch(cfg) > 1) || cfg->algorithm == 3)
     b += (size_t)image_batch(cfg) * npix * R;        // a batch of images
   if (uses_means(cfg)) b += rsx::slice_means_bytes(cfg->precision, cfg->nz);
   return b;
@@ -1133,11 +1146,9 @@ int rsx_angle_count(double start, double inc, double end, int rotation) {
   return (int)n;
 }
 
-int rsx_create(const rsx_config* cfg, rsx_context** out) {
-  if (!out) return fail(RSX_ERR_INVALID, "out is NULL");
-  *out = nullptr;
-  int rc = check_config(cfg);
-  if (rc) return rc;
+// least: with the smallest p workspace and one image.
+static int create_context(const rsx_config* cfg, bool least, rsx_context** out) {
+  int rc;
   rsx_context* c = new (std::nothrow) rsx_context();
   if (!c) return fail(RSX_ERR_OOM, "no host memory for the context");
   c->cfg = *cfg;
@@ -1150,13 +1161,13 @@ int rsx_create(const rsx_config* cfg, rsx_context** out) {
     return cuda_fail(e, "cudaGetDevice");
   }
   const size_t R = real_size(cfg->precision), Cs = complex_size(cfg->precision);
-  c->p_cap = p_elems(cfg);
+  c->p_cap = p_elems(cfg, least);
   struct {
     void** dst;
     size_t bytes;
     const char* what;
   } allocs[] = {
-      {&c->p, (size_t)p_elems(cfg) * Cs, "p workspace"},
+      {&c->p, (size_t)c->p_cap * Cs, "p workspace"},
       {&c->img, (size_t)c->npix * R, "Ewald image"},
       {&c->acc, (size_t)c->npix * R, "Ewald average"},
       {&c->geo, (size_t)c->npix * geo_size(cfg->precision), "Ewald geometry"},
@@ -1255,9 +1266,11 @@ int rsx_create(const rsx_config* cfg, rsx_context** out) {
     delete c;
     return rc;
   }
-  c->n_img = image_batch(cfg);
+  c->n_img = image_batch(cfg, least);
   if (c->n_img > 0 && cfg->algorithm != 3 && c->part) {
     c->imgs = c->part;  // the planes path does not use the bins
+  } else if (c->n_img == 1) {
+    c->imgs = c->img;
   } else if (c->n_img > 0) {
     if ((e = cudaMalloc(&c->imgs, (size_t)c->n_img * c->npix * R)) != cudaSuccess) {
       c->imgs = nullptr;
@@ -1276,6 +1289,21 @@ int rsx_create(const rsx_config* cfg, rsx_context** out) {
   }
   *out = c;
   return RSX_OK;
+}
+
+int rsx_create(const rsx_config* cfg, rsx_context** out) {
+  if (!out) return fail(RSX_ERR_INVALID, "out is NULL");
+  *out = nullptr;
+  int rc = check_config(cfg);
+  if (rc) return rc;
+  rc = create_context(cfg, false, out);
+  if (rc == RSX_ERR_OOM && (p_elems(cfg) > p_elems(cfg, true) ||
+                            image_batch(cfg) > image_batch(cfg, true))) {
+    cudaGetLastError();  // the failed allocation
+    rc = create_context(cfg, true, out);
+    if (rc == RSX_OK) g_err.clear();
+  }
+  return rc;
 }
 
 int rsx_destroy(rsx_context* c) {
