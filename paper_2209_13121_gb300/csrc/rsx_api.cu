@@ -324,7 +324,7 @@ bool make_tmap(rsx_context* c, void* base, long long nslices, CUtensorMap* m, un
 }
 
 // The z-first pass's tensor map over the FP32 morphology, viewed as
-// [c nz][ny][4 nx] floats: boxes of 128 / nz adjacent voxels (4 floats each)
+// [c nz][ny][4 nx] floats: boxes of 1024 / nz adjacent voxels (4 floats each)
 // of one row y by the nz slices of one component (16 KB).
 bool make_tmap_m(rsx_context* c, CUtensorMap* m) {
   const PFN_cuTensorMapEncodeTiled_v12000 encode = tmap_encoder();
@@ -493,11 +493,10 @@ cudaError_t planes_x_fft(rsx_context* c, void* data, const ZPlan& zp, long long 
   return rsx::launch_row_fft<R>(data, g.nx, nrows, c->twx, s);
 }
 
-// (A film's whole plane is stored: 2048 rows then go 4 columns, 32 bytes, at a
-// time, 15.4 ms per two energies of 91 angles at 2048 x 2048; the 8-column
-// kernel 12.0.)
 // y-FFT of nfields x ns contiguous [ny][nx] planes at data, in place; on the
-// tuned sizes only what the image reads is transformed and stored.
+// tuned sizes only what the image reads is transformed and stored.  (Of a film
+// that is everything: 2048 rows would go 4 columns, 32 bytes, at a time, 15.4 ms
+// per two energies of 91 angles at 2048 x 2048; the 8-column kernel 12.0.)
 template <typename R>
 cudaError_t planes_y_fft(rsx_context* c, void* data, const ZPlan& zp, long long nfields,
                          const rsx::YRuns& runs, cudaStream_t s) {
@@ -565,9 +564,10 @@ void plane_runs(const rsx_config& g, double k, const ZPlan& zp, rsx::YRuns* runs
   }
 }
 
-// The same for stacks the z-first form serves: N_t's entries z-transformed
-// as they are formed (from the device morphology; from N_t where that was
-// streamed from the host) and only the kept planes transformed laterally.
+// The linearity path's bins (see ensure_bins) for stacks the z-first form
+// serves: N_t's entries, less their slices' means, z-transformed as they are
+// formed (from the device morphology; from N_t where that was streamed from
+// the host) and only the kept planes transformed laterally.
 template <typename R>
 int lin_planes_bins(rsx_context* c, int ie, const ZPlan& zp, cudaStream_t s) {
   const rsx_config& g = c->cfg;
@@ -805,12 +805,12 @@ const char* rsx_last_error(void) { return g_err.c_str(); }
 static bool uses_yz(const rsx_config* cfg) {
   return cfg->precision == 32 && rsx::yz_fusable(cfg->nx, cfg->ny, cfg->nz);
 }
-// kYzSlots slots of (3 fields of p, or the linearity path's 5 N_t entries) x 2 bins
 // The planes path's tuned y pass (FP32).
 static bool y_tuned(const rsx_config* cfg) {
   return cfg->precision == 32 && cfg->algorithm != 3 && cfg->nz <= rsx::kMaxPlanesNz &&
          rsx::y_planes_ok(cfg->nx, cfg->ny);
 }
+// kYzSlots slots of (3 fields of p, or the linearity path's 5 N_t entries) x 2 bins
 static size_t part_bytes(const rsx_config* cfg) {
   return rsx::kYzSlots * (size_t)(cfg->algorithm == 3 ? 5 : 3) * cfg->nx * cfg->ny * 16;
 }
@@ -962,7 +962,7 @@ bool lin_plan(const rsx_context* c, int ie, ZPlan* zp) {
 
 static bool zfirst_plan(const rsx_context* c, int ie, ZPlan* zp) {
   const rsx_config& g = c->cfg;
-  if (!zfirst_ok(&g) || c->n_sm <= 0 || !c->part || !c->b0idx || ie < 0 ||
+  if (!zfirst_ok(&g) || c->n_sm <= 0 || !c->b0idx || ie < 0 ||
       ie >= (int)c->energies.size() || (c->M && ((uintptr_t)c->M & 15)))
     return false;
   if ((g.nx == 1024 && !c->tw4) || (g.nx == 2048 && !c->tw2k) || (g.ny == 2048 && !c->twy))
@@ -1519,8 +1519,6 @@ int rsx_scatter_angle(rsx_context* c, int ie, double alpha, void* img, void* str
 }
 
 namespace {
-// All angles of one energy, one after the other: the image of each angle
-// (scatter_angle), rotated into the average.
 // Algorithm 1 with the morphology read once per batch of kx angles: the
 // multi-angle x pass writes each angle's x-transformed p to its own buffer,
 // then every angle of the batch goes through the fused y+z pass, the Ewald
@@ -1668,8 +1666,8 @@ int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang
       memset(&rb, 0, sizeof(rb));
       dc.n = ni;
       for (int k = 0; k < ni; ++k) {
-        dc.x[k] = (R)(lit ? ref : ref * cos(alpha[i0 + k]));
-        dc.y[k] = (R)(lit ? 0.0 : ref * sin(alpha[i0 + k]));
+        dc.x[k] = lit ? ref : ref * cos(alpha[i0 + k]);
+        dc.y[k] = lit ? 0.0 : ref * sin(alpha[i0 + k]);
         rsx::add_angle(rb, alpha[i0 + k], g.nx, g.ny);
         dc.ce[k] = rb.ce[k];
         dc.se[k] = rb.se[k];
@@ -1693,6 +1691,9 @@ int run_energy_planes(rsx_context* c, int ie, double start, double inc, int nang
   return RSX_OK;
 }
 
+// All angles of one energy: on the planes path, in batches through the
+// multi-angle x pass, or one after the other (scatter_angle, then the rotation
+// into the average).
 template <typename R>
 int run_energy_angles(rsx_context* c, int ie, double start, double inc, int nang, int rotation,
                       cudaStream_t s) {

@@ -890,7 +890,9 @@ __global__ void __launch_bounds__(32 * (PW + 3 * FG + 1), 1) k_pol_fft4s_tma_mul
 //            shared memory and copied out bin by bin: 59.8 ms per energy
 //            at 1024 x 1024 x 128, 91 angles, 53.4 so; 2048 x 2048 x 64
 //            121.7 and 109.0; with the ten-real form of the sums, PTen,
-//            48.9 and 99.0.)
+//            48.9 and 99.0, and with the slices' means left out 49.6 and
+//            100.8.)  The sums start at minus their slice's mean, which
+//            costs loads and no operation.
 // zf_pos(a, b) = 32 a + b, for R = 4 with b xor a (the low bits swizzled by
 // a); with LS = 130 (R = 4) or nz + 1 that keeps the polarisation stores and
 // stage 2's loads free of shared-memory bank conflicts (checked per
@@ -903,15 +905,13 @@ template <int R> __device__ __forceinline__ int zf_pos(int a, int b) {
   return 32 * a + (R == 4 ? (b ^ a) : b);
 }
 
-// Roles of the 18 warps of the z-first pass for nz = 128.  The split was
-// set when a transform warp also ran the z transform's first radix stage
-// (~1.2x the per-tile work of a polarisation warp): over the four
-// schedulers (warp index mod 4) Prod T T T P | P P P P P | T T T P
-// | T T T P kept every scheduler within ~7 % of the mean, and each
-// transform group (three consecutive indices) spans three schedulers: warps
-// 0, 2, 3, 4, 6, 7, 8, 10, 11 transform (0..8), 16 produces, 1, 5, 9, 13,
-// 17, 12, 14, 15 polarise (0..7).  (P1: x pass 72.8 -> 72.2 ms per energy;
-// nz = 64 measured 3 % slower with it and keeps multi_role.)
+// Roles of the 18 warps of the z-first pass for nz = 128: over the four
+// schedulers (warp index mod 4) Prod T T T P | P P P P P | T T T P | T T T P,
+// each transform group (three consecutive indices) over three schedulers:
+// warps 0, 2, 3, 4, 6, 7, 8, 10, 11 transform (0..8), 16 produces, 1, 5, 9, 13,
+// 17, 12, 14, 15 polarise (0..7).  The balance is close: 1024 x 1024 x 128, 91
+// angles 49.6 ms so and 49.8 with multi_role; nz = 64 takes multi_role (2048 x
+// 2048 x 64, 91 angles: 99.5 ms, 102.5 with this table).
 __device__ __forceinline__ void zf_role(int w, int& kind, int& idx) {
   const int q = w & 3;
   if (w == 16) {

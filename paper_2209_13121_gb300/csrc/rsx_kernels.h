@@ -202,8 +202,8 @@ cudaError_t launch_pol_fft4s_tma_multi(const void* M, int nx, int ny, int nz,
 // kb .. kb + ns - 1 (mod nz) kept: angle k's plane s of field f goes to
 // out + k * kstride + f * fstride + s * nx * ny as an [ny][nx] complex plane
 // (not yet x- or y-transformed).  tmap: a CUtensorMap over the morphology
-// viewed as [c nz][ny][4 nx] floats with (128 / nz) x 1 x nz boxes (see
-// make_tmap_m); twz: exp(-2 pi i j / nz), j < nz.  nz = 32, 64 or 128, nx a
+// viewed as [c nz][ny][4 nx] floats with 4 (1024 / nz) x 1 x nz boxes (see
+// make_tmap_m); twz: exp(-2 pi i j / nz), j < nz; means: launch_slice_means.  nz = 32, 64 or 128, nx a
 // multiple of 1024 / nz.  zfirst_fusable: the shapes whose lateral passes
 // are tuned too (nx and ny = 512, 1024 or 2048).  One persistent CTA per SM
 // (n_sm).
@@ -326,7 +326,7 @@ cudaError_t launch_rotate_acc(const void* img, void* acc, int nx, int ny, double
 constexpr int kMaxPlanesNz = 255;
 template <typename R> struct ImageDc {
   int n;
-  R x[kMaxAngleBatch], y[kMaxAngleBatch];
+  double x[kMaxAngleBatch], y[kMaxAngleBatch];
   R ce[kMaxAngleBatch], se[kMaxAngleBatch], c2[kMaxAngleBatch], s2[kMaxAngleBatch];
 };
 size_t slice_means_bytes(int precision, int nz);

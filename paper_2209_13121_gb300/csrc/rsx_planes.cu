@@ -1,13 +1,17 @@
-// The general planes path: Algorithm 1 or 2 for any grid with nz <= 254 in
-// either precision, a batch of e-field angles at a time.
+// The general planes path: Algorithm 1 or 2 for any grid with nz <= 255 in
+// either precision, a batch of e-field angles at a time, and (z transform
+// first too) the linearity path's five entries of N_t.
 //
-//   k_pol_planes    per pixel column: the angle-independent sums of Eq.
-//                   (polarization) once, then for each angle p, its z
-//                   transform, and only the ns q_z planes the detector reads
+//   k_slice_means   a constant near each slice's mean, left out of p.
+//   k_pol_planes, k_pol_planes_fft   per pixel column: the angle-independent
+//                   sums of Eq. (polarization) once, then for each angle p, its
+//                   z transform, and only the ns q_z planes the detector reads
 //                   (the run kb .. kb + ns - 1 mod nz; see rsx_zfirst_plan).
-//   (x-FFT, y-FFT)  the lateral transforms of those planes, in place.
+//   k_x_planes, k_y_planes   the lateral transforms of those planes, in place,
+//                   for tuned sizes (others: the general row and column FFTs).
 //   k_plane_images  Eqs. (3Dscatter) and (Ewald): each pixel's two planes to
 //                   the detector image, for every angle of the batch.
+//   k_bins5_planes  the same for the linearity path's bins.
 // The rotation and average follow as on the other paths.  The 3-D DFT is
 // separable, so the values are the full transform's up to rounding order.
 #include <cuda.h>  // CUtensorMap (the type only)
@@ -103,7 +107,9 @@ __global__ void __launch_bounds__(kMeanSample<R>) k_slice_means(
 // What leaving the means out takes from p at q = 0: PTen's ten numbers of npix
 // times their sum over z, in double.  A block of 256 threads calls
 // means_total, then those that want the result means_pten (FP64 arithmetic:
-// not more threads than need be).  from_nt: the rows are PTen's already.
+// not more threads than need be).  from_nt: the rows are PTen's already.  The
+// value at q = 0 is rounded once, when what was left out has been added: it
+// outweighs the rest of the image.
 template <typename R>
 __device__ __forceinline__ void means_total(const R* __restrict__ means, int nz, long long npix,
                                             double* total) {
@@ -116,20 +122,19 @@ __device__ __forceinline__ void means_total(const R* __restrict__ means, int nz,
   if ((t & 15) == 0 && q < kMeanVals) total[q] = m * (double)npix;
   __syncthreads();
 }
-template <typename R>
 __device__ __forceinline__ void means_pten(const double* total, bool literal, bool from_nt,
-                                           PTen<R>& out) {
+                                           PTen<double>& out) {
   const double sc = from_nt ? 1.0 : 1.0 / kFourPi;
   const bool half = literal && !from_nt;
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     const double* q = total + i;
     const double ar = q[10] + (i == 0 ? total[12] : 0.0);
-    out.a[i] = (R)(sc * (half ? ar + 0.5 * (q[0] + q[4]) : ar + q[0]));
-    out.b[i] = (R)(sc * (half ? 0.5 * (q[0] - q[4]) : ar + q[4]));
-    out.xy[i] = (R)(sc * q[2]);
-    out.xz[i] = (R)(sc * q[6]);
-    out.yz[i] = (R)(sc * q[8]);
+    out.a[i] = sc * (half ? ar + 0.5 * (q[0] + q[4]) : ar + q[0]);
+    out.b[i] = sc * (half ? 0.5 * (q[0] - q[4]) : ar + q[4]);
+    out.xy[i] = sc * q[2];
+    out.xz[i] = sc * q[6];
+    out.yz[i] = sc * q[8];
   }
 }
 
@@ -362,11 +367,11 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 4 ? 2 : 1) k_pol_plan
 // three fields to shared memory (thread order: contiguous); then the threads
 // take (angle, field, s1, pixel) items: a Q-point transform over n2 in
 // registers, whose first outputs s2 go straight to their planes (Q = 32: only
-// the kept ones are evaluated).  ~75 instructions per voxel and angle at
-// nz = 16, where the folded sums above took 160 at 64 % issue (1024 x 1024 x 16,
-// c = 3, two energies of 91 angles: the pass 19.0 ms, 13.4 so; Algorithm 2 at
-// 1024 x 1024 x 32, 37 angles: 16.5 and 13.2; with PTen and three blocks per
-// SM 12.0 and 11.5).
+// the kept ones are evaluated).  119 instructions per voxel and angle at
+// nz = 16 and 74 % issue (1024 x 1024 x 16, c = 3, 18 angles: 1.22 ms), where the
+// folded sums above took 160 at 64 % (1.88 ms).  Two energies of 91 angles there:
+// the pass 19.0 ms, 12.2 so; Algorithm 2 at 1024 x 1024 x 32, 37 angles: 16.5 and
+// 12.3 (FP32, nz <= 32: three blocks per SM).
 // NF = 3: the fields of p of every angle.  NF = 5: the linearity path's five
 // entries of N_t (xx, xy, yy, xz, yz, the constant left out), once.
 template <typename R, int Q> struct PlFft {
@@ -528,10 +533,12 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 8 ? 1 : Q <= 8 && NF 
 // before the transform returned at q = 0 (the constant's x and y parts per
 // angle, and the slices' means, null: none), the projection and the interpolation; written in fftshift order.  A thread
 // takes AP angles of one pixel, so the 32-byte geometry is read once for
-// them (q = 0 has a block of its own, which costs the others no registers);
+// them; q = 0 has a block of its own, and with AP = 4 the registers are held to
+// what the other blocks need (2048 x 2048 film, 182 angles: 5.05 ms; 5.37 with
+// q = 0's 40 registers, 6.4 with its code behind the loop).
 // planes has kstride = 3 ns npix complex per angle.
 template <typename R, int AP>
-__global__ void __launch_bounds__(256) k_plane_images(const typename RT<R>::C* __restrict__ planes,
+__global__ void __launch_bounds__(256, sizeof(R) == 8 ? 4 : AP == 4 ? 8 : 5) k_plane_images(const typename RT<R>::C* __restrict__ planes,
                                                       int nx, int ny, int nz, int kb, int ns,
                                                       const Geo<R>* __restrict__ geo,
                                                       const __grid_constant__ ImageDc<R> dc,
@@ -546,22 +553,24 @@ __global__ void __launch_bounds__(256) k_plane_images(const typename RT<R>::C* _
     if (means) means_total<R>(means, nz, npix, sum);
     const int a = threadIdx.x;
     if (a >= dc.n) return;
-    PTen<R> total;
+    PTen<double> total;
     pten_zero(total);
     if (means) means_pten(sum, literal != 0, from_nt != 0, total);
     const Geo<R> g = geo[0];
     const int s0 = g.b0 < kb ? g.b0 - kb + nz : g.b0 - kb, s1 = g.b1 < kb ? g.b1 - kb + nz : g.b1 - kb;
     const C* src = planes + a * kstride;
-    C d[3], v0[3], v1[3];
-    p_from_pten(total, dc.ce[a], dc.se[a], dc.c2[a], dc.s2[a], literal != 0, d);
+    double2 d[3];
+    C v0[3], v1[3];
+    p_from_pten<double>(total, dc.ce[a], dc.se[a], dc.c2[a], dc.s2[a], literal != 0, d);
     d[0].x += dc.x[a];
     d[1].x += dc.y[a];
+    auto plus = [](C v, double2 w) { return RT<R>::mk((R)(v.x + w.x), (R)(v.y + w.y)); };
 #pragma unroll
     for (int f = 0; f < 3; ++f) {
       v0[f] = src[f * fstride + (size_t)s0 * npix];
       v1[f] = src[f * fstride + (size_t)s1 * npix];
-      if (g.b0 == 0) v0[f] = cadd(v0[f], d[f]);
-      if (g.b1 == 0) v1[f] = cadd(v1[f], d[f]);
+      if (g.b0 == 0) v0[f] = plus(v0[f], d[f]);
+      if (g.b1 == 0) v1[f] = plus(v1[f], d[f]);
     }
     imgs[(size_t)a * npix + (size_t)(ny / 2) * nx + nx / 2] = ewald_value<R>(g, v0, v1);
     return;
@@ -1055,39 +1064,41 @@ cudaError_t pol_planes_sb(const void* M, const void* nt, const void* dir, long l
 template <typename R>
 __global__ void __launch_bounds__(256) k_bins5_planes(const typename RT<R>::C* __restrict__ planes,
                                                       long long npix, int nz, int kb, int ns,
-                                                      const Geo<R>* __restrict__ geo, R dc,
+                                                      const Geo<R>* __restrict__ geo, double dc,
                                                       const R* __restrict__ means, int from_nt,
                                                       typename RT<R>::C* __restrict__ bins) {
   using C = typename RT<R>::C;
   const long long pix =
       blockIdx.x == 0 ? 0 : (long long)(blockIdx.x - 1) * blockDim.x + threadIdx.x;
   if (pix >= npix || (blockIdx.x > 0 && pix == 0)) return;
-  C d[5];
-#pragma unroll
-  for (int q = 0; q < 5; ++q) d[q] = RT<R>::mk(R(0), R(0));
+  const Geo<R> g = geo[pix];
   if (blockIdx.x == 0) {
     __shared__ double sum[kMeanVals];
     means_total<R>(means, nz, npix, sum);
     if (threadIdx.x > 0) return;
-    PTen<R> m;
+    PTen<double> m;
     means_pten(sum, false, from_nt != 0, m);
-    d[0] = RT<R>::mk(m.a[0] + dc, m.a[1]);
-    d[1] = RT<R>::mk(m.xy[0], m.xy[1]);
-    d[2] = RT<R>::mk(m.b[0] + dc, m.b[1]);
-    d[3] = RT<R>::mk(m.xz[0], m.xz[1]);
-    d[4] = RT<R>::mk(m.yz[0], m.yz[1]);
+    const double2 d[5] = {{m.a[0] + dc, m.a[1]}, {m.xy[0], m.xy[1]}, {m.b[0] + dc, m.b[1]},
+                          {m.xz[0], m.xz[1]}, {m.yz[0], m.yz[1]}};
+    for (int b = 0; b < 2; ++b) {
+      const int bin = b ? g.b1 : g.b0, s = bin < kb ? bin - kb + nz : bin - kb;
+#pragma unroll
+      for (int q = 0; q < 5; ++q) {
+        C v = planes[((size_t)q * ns + s) * npix];
+        if (bin == 0) v = RT<R>::mk((R)(v.x + d[q].x), (R)(v.y + d[q].y));
+        bins[(size_t)(2 * q + b) * npix] = v;
+      }
+    }
+    return;
   }
-  const Geo<R> g = geo[pix];
   if (g.b0 < 0) return;  // off the sphere: the bins are not read
 #pragma unroll
   for (int b = 0; b < 2; ++b) {
     const int bin = b ? g.b1 : g.b0;
     const int s = bin < kb ? bin - kb + nz : bin - kb;
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      const C v = planes[((size_t)q * ns + s) * npix + pix];
-      bins[(size_t)(2 * q + b) * npix + pix] = bin == 0 ? cadd(v, d[q]) : v;
-    }
+    for (int q = 0; q < 5; ++q)
+      bins[(size_t)(2 * q + b) * npix + pix] = planes[((size_t)q * ns + s) * npix + pix];
   }
 }
 
@@ -1172,7 +1183,7 @@ cudaError_t launch_bins5_planes(const void* planes, int nx, int ny, int nz, int 
   const long long npix = (long long)nx * ny;
   if (!means) return cudaErrorInvalidValue;
   k_bins5_planes<R><<<(unsigned)((npix + 255) / 256) + 1, 256, 0, s>>>(
-      (const C*)planes, npix, nz, kb, ns, geo, (R)dc, (const R*)means, from_nt ? 1 : 0, (C*)bins);
+      (const C*)planes, npix, nz, kb, ns, geo, dc, (const R*)means, from_nt ? 1 : 0, (C*)bins);
   return cudaGetLastError();
 }
 
