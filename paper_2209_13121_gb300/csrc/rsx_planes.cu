@@ -393,12 +393,23 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 8 ? 1 : Q <= 8 && NF 
   using P = PlFft<R, Q>;
   constexpr int NZ = 4 * Q, PX = P::PX, KS = P::KS, A = NF == 3 ? P::A : 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int NM = SRC == 1 ? NZ * kMeanStride : 0;
-  R* mean_s = reinterpret_cast<R*>(smem_raw);  // [NZ][kMeanStride] (N_t)
-  C* buf = reinterpret_cast<C*>(mean_s + NM);  // [A][NF][4][KS]
+  // N_t: the rows of the slices' means a warp needs (4 n1, NR n2), fetched by
+  // the warp itself, so that no warp waits for another's loads
+  constexpr int NR = PX >= 32 ? 1 : 32 / PX, kRow = kMeanStride * (int)sizeof(R);
+  constexpr int NM = SRC == 1 ? kPlThreads / 32 * 4 * NR * kRow : 0;
+  unsigned char* const mean_s = smem_raw + (threadIdx.x >> 5) * 4 * NR * kRow;
+  C* buf = reinterpret_cast<C*>(smem_raw + NM);  // [A][NF][4][KS]
   const int t = threadIdx.x, px = t % PX, n2 = t / PX;
-  for (int i = 2 * t; i < NM; i += 2 * kPlThreads)
-    cp_async_elem(reinterpret_cast<C*>(mean_s + i), reinterpret_cast<const C*>(means + i));
+  if constexpr (SRC == 1) {
+    constexpr int CH = 10 * (int)sizeof(R) / 16 + (sizeof(R) == 4);  // 16-byte pieces in use
+    const int first = (t & ~31) / PX;                                // the warp's lowest n2
+    for (int i = t & 31; i < 4 * NR * CH; i += 32) {
+      const int r = i / CH, c = i % CH, z = first + r % NR + Q * (r / NR);
+      cp_async_pair(reinterpret_cast<float2*>(mean_s + r * kRow + c * 16),
+                    reinterpret_cast<const float2*>(
+                        reinterpret_cast<const unsigned char*>(means) + z * kRow + c * 16));
+    }
+  }
   const long long N = npix * NZ;
   const long long pix0 = (long long)blockIdx.x * PX;
   const int npx = npix - pix0 < PX ? (int)(npix - pix0) : PX;
@@ -452,11 +463,13 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 8 ? 1 : Q <= 8 && NF 
   if constexpr (SRC == 1) {
     // (the means come while N_t does, and are taken off when both are here)
     cp_async_wait_all();
-    __syncthreads();
-    if (px < npx)
+    __syncwarp();
+    if (px < npx) {
+      const int j = n2 - (t & ~31) / PX;
 #pragma unroll
       for (int n1 = 0; n1 < 4; ++n1)
-        pten_less(ten[n1], mean_s + (n2 + Q * n1) * kMeanStride);
+        pten_less(ten[n1], reinterpret_cast<const R*>(mean_s + (n1 * NR + j) * kRow));
+    }
   }
   const size_t fstride = (size_t)ns * npix;
   const int rot = kb & 3;  // s1 = 0 takes output kb mod 4 of the 4-point transform
@@ -531,9 +544,9 @@ __global__ void __launch_bounds__(kPlThreads, sizeof(R) == 8 ? 1 : Q <= 8 && NF 
 // Images of the angles of a batch from their transformed planes: per pixel
 // its two planes (b - kb mod nz) of the three fields, what was left out of p
 // before the transform returned at q = 0 (the constant's x and y parts per
-// angle, and the slices' means, null: none), the projection and the interpolation; written in fftshift order.  A thread
-// takes AP angles of one pixel, so the 32-byte geometry is read once for
-// them; q = 0 has a block of its own, and with AP = 4 the registers are held to
+// angle, and the slices' means, null: none), the projection and the
+// interpolation; written in fftshift order.  A thread takes AP angles of one
+// pixel, so the 32-byte geometry is read once for them; q = 0 has a block of its own, and with AP = 4 the registers are held to
 // what the other blocks need (2048 x 2048 film, 182 angles: 5.05 ms; 5.37 with
 // q = 0's 40 registers, 6.4 with its code behind the loop).
 // planes has kstride = 3 ns npix complex per angle.
@@ -1108,7 +1121,8 @@ cudaError_t pol_planes_fft(const void* M, const void* nt, const void* dir, long 
                            int ns, const void* twz, const void* means, cudaStream_t s) {
   using C = typename RT<R>::C;
   using P = PlFft<R, Q>;
-  const size_t smem = (SRC == 1 ? (size_t)4 * Q * kMeanStride * sizeof(R) : 0) +
+  constexpr int NR = P::PX >= 32 ? 1 : 32 / P::PX;  // (as in the kernel)
+  const size_t smem = (SRC == 1 ? (size_t)kPlThreads / 32 * 4 * NR * kMeanStride * sizeof(R) : 0) +
                       (size_t)(NF == 3 ? P::A : 1) * 4 * NF * P::KS * sizeof(C);
   auto kern = k_pol_planes_fft<R, SRC, Q, NF>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -63,7 +63,9 @@ def test_a_uniform_background_leaves_no_rounding_in_faint_images(rsx, shape, alg
     a white error below a white signal is the image's relative L2 error away
     from q = 0; the transforms of a field without its mean add far less.  A
     mean that is still there when z is transformed adds nz roundings of its
-    size to bin 0 and grows the error as sqrt(nz).  Bound: 2 2^-25 / s."""
+    size to bin 0 and grows the error as sqrt(nz).  Bound: 2 2^-25 / s.  Eight
+    angles of 0 and 180 degrees, whose rotations are exact, so that the planes
+    path is taken."""
     from oracle import cyrsoxs_oracle as O
     from paper_2209_13121_gb300 import synth
     nz, ny, nx = shape
@@ -71,12 +73,15 @@ def test_a_uniform_background_leaves_no_rounding_in_faint_images(rsx, shape, alg
     M[..., 0] = 0.5 + 0.01 * np.random.default_rng(5).random((nz, ny, nx))
     K = synth.optical_constants([285.0], 1, seed=6)
     s = float(np.std(M[..., 0].astype(np.float64) ** 2))
-    ref = O.scatter_one_angle(M.astype(np.float64), K[0], 285.0, 5.0, 0.0)
+    angles = (0.0, 180.0, 1260.0)
+    ref = O.run_alg1(M.astype(np.float64), K, [285.0], 5.0, angles_deg=angles)[0]
     iy, ix = np.meshgrid(np.arange(ny) - ny // 2, np.arange(nx) - nx // 2, indexing="ij")
     far = np.hypot(ix, iy) > 0.5
     with rsx.Context(nx, ny, nz, 1, 5.0, algorithm=alg) as ctx:
         ctx.set_morphology(torch.from_numpy(M).cuda())
         ctx.set_optical_constants([285.0], K)
-        got = ctx.run(rotation=False)[0].astype(np.float64)
+        ctx.set_timing(True)
+        got = ctx.run(angles)[0].astype(np.float64)
+        assert ctx.phase_times()["fftx"][1] > 0  # the planes path
     err = np.linalg.norm((got - ref)[far]) / np.linalg.norm(ref[far])
     assert err <= 2 * 2.0 ** -25 / s, (err, 2.0 ** -25 / s)
