@@ -562,26 +562,32 @@ __global__ void __launch_bounds__(256, sizeof(R) == 8 ? 4 : AP == 4 ? 8 : 5) k_p
   const size_t fstride = (size_t)ns * npix, kstride = 3 * fstride;
   if (blockIdx.x == 0) {  // q = 0, an angle per thread: with what was left out
     if (blockIdx.y > 0) return;
+    const int a = threadIdx.x;
+    // (the loads first: they and the means' arrive together)
+    const Geo<R> g = geo[0];
+    const int s0 = g.b0 < kb ? g.b0 - kb + nz : g.b0 - kb, s1 = g.b1 < kb ? g.b1 - kb + nz : g.b1 - kb;
+    C v0[3], v1[3];
+    if (a < dc.n) {
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        const C* src = planes + a * kstride + f * fstride;
+        v0[f] = src[(size_t)s0 * npix];
+        v1[f] = src[(size_t)s1 * npix];
+      }
+    }
     __shared__ double sum[kMeanVals];
     if (means) means_total<R>(means, nz, npix, sum);
-    const int a = threadIdx.x;
     if (a >= dc.n) return;
     PTen<double> total;
     pten_zero(total);
     if (means) means_pten(sum, literal != 0, from_nt != 0, total);
-    const Geo<R> g = geo[0];
-    const int s0 = g.b0 < kb ? g.b0 - kb + nz : g.b0 - kb, s1 = g.b1 < kb ? g.b1 - kb + nz : g.b1 - kb;
-    const C* src = planes + a * kstride;
     double2 d[3];
-    C v0[3], v1[3];
     p_from_pten<double>(total, dc.ce[a], dc.se[a], dc.c2[a], dc.s2[a], literal != 0, d);
     d[0].x += dc.x[a];
     d[1].x += dc.y[a];
     auto plus = [](C v, double2 w) { return RT<R>::mk((R)(v.x + w.x), (R)(v.y + w.y)); };
 #pragma unroll
     for (int f = 0; f < 3; ++f) {
-      v0[f] = src[f * fstride + (size_t)s0 * npix];
-      v1[f] = src[f * fstride + (size_t)s1 * npix];
       if (g.b0 == 0) v0[f] = plus(v0[f], d[f]);
       if (g.b1 == 0) v1[f] = plus(v1[f], d[f]);
     }
